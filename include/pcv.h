@@ -206,10 +206,14 @@ int64_t pcv_distribution_tc_workspace(int m, int n);
 int64_t pcv_distribution_workspace(int m, int n);
 int64_t pcv_distribution_workspace_min(int m, int n);
 
-/* The algorithm pcv_distribution (PCV_ALGO_AUTO) runs for m modes, n photons
+/* The path pcv_distribution (PCV_ALGO_AUTO) takes for m modes, n photons
  * and a workspace of workspace_bytes: PCV_ALGO_FACTOR_TC when 2 <= n <= 10,
  * m >= 2 and workspace_bytes >= pcv_distribution_tc_workspace(m, n), else
- * PCV_ALGO_FACTOR.  Both give the same amplitudes to double precision.  Returns
+ * PCV_ALGO_FACTOR, which here names the FP64 path: by state expansion (the
+ * computation of PCV_ALGO_SLOS) when the workspace also holds its level
+ * buffers (pcv_distribution_slos_workspace(1, m, n) + 256 bytes), else the
+ * factorised sum with FP64 products, in as many passes as the workspace
+ * asks for.  All give the same amplitudes to double precision.  Returns
  * the algorithm code, or PCV_EINVAL for sizes out of range.  No counterpart in
  * the paper. */
 int pcv_distribution_auto_algo(int m, int n, int64_t workspace_bytes);
@@ -224,8 +228,8 @@ int pcv_distribution_auto_algo(int m, int n, int64_t workspace_bytes);
  * the product splits into the modes below and above m/2, so each output costs
  * one complex multiply-add per sign vector.  Those products run on the tensor
  * cores in exact integer arithmetic (PCV_ALGO_FACTOR_TC below) when the input
- * has 2..10 photons and the workspace holds that plan, else as FP64 multiply-
- * adds (PCV_ALGO_FACTOR); pcv_distribution_auto_algo tells which. */
+ * has 2..10 photons and the workspace holds that plan, else the call takes the
+ * FP64 path; pcv_distribution_auto_algo tells which. */
 int pcv_distribution(const pcv_c64* U, int m, const uint8_t* input_occ,
                      double* prob, pcv_c64* amp,
                      void* workspace, int64_t workspace_bytes, void* stream);
@@ -279,8 +283,9 @@ int pcv_distribution_range_plan(int m, int n, int64_t begin, int64_t end, int64_
 int pcv_distribution_tc_blocks(int m, int n, int64_t begin, int64_t end, int64_t* out, int64_t out_len,
                                int64_t* needed);
 
-/* Full distributions of B unitaries with the same input state (the
- * factorised algorithm of pcv_distribution, all B in the same launches).
+/* Full distributions of B unitaries with the same input state (the FP64
+ * path of pcv_distribution, all B in the same launches: the state expansion
+ * with the workspace named here, the factorised sum with a smaller one).
  *   U     device, B*m*m pcv_c64 (entry b at U + b*m*m)
  *   B     1..65535
  *   prob  device, B*C(m+n-1,n) doubles or NULL; amp likewise pcv_c64 or NULL

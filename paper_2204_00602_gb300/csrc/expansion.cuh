@@ -1,0 +1,70 @@
+// Photon-by-photon state expansion: index arithmetic and launch interface
+// shared by the full distribution (slos.cu), its adjoint (expansion_grad.cu),
+// the source model (distinguish.cu) and the split amplitudes (split.cu).
+//
+// Ranks.  With MC(w, j) = C(w + j - 1, j), the multisets of size j over w
+// modes, and t(l, j) = MC(m - l - 1, j), those over the modes above l, the
+// canonical index of a sorted mode list l_0 <= ... <= l_{L-1} of S_{m,L} is
+//     rank = |S_{m,L}| - 1 - sum_q t(l_q, L - q):
+// the q-th sum of the lists before it, MC(m - l_{q-1}, L - q) - MC(m - l_q,
+// L - q), telescopes through MC(w, j) = MC(w - 1, j) + MC(w, j - 1).  So each
+// position contributes one entry of the table of counts, and taking a photon
+// out, or putting one in, moves the later positions' entries by one column.
+#pragma once
+
+#include "pcv_common.cuh"
+
+namespace pcv {
+
+// Where a batch entry of a level launch takes its photon and its parent from.
+enum ExpandSource {
+    kExpandBatch = 0,    // entry b: unitary b, the same photon (column col[0]) for all
+    kExpandSides = 1,    // entry b: column col[b] of one unitary
+    kExpandSubsets = 2,  // entry b: the b-th k-subset of the photons (colex order); its
+                         // largest photon is added to the entry of the other k - 1
+};
+
+struct ExpandArgs {
+    int source;
+    const double2* U;          // [B][m][m] (kExpandBatch) or [m][m]
+    int m, k;                  // modes, level built (k >= 1)
+    int col[PCV_MAX_PHOTONS];  // columns (kExpandSubsets: of every photon)
+    const int64_t* mc;         // multiset counts MC[a][j], row length kmax + 1
+    int kmax;
+    int B;                     // batch entries
+    int64_t count;             // states of level k
+    int64_t prev_count;        // states of level k - 1
+    int64_t lo, hi;            // states written (the whole level unless it is the last one)
+    const double2* prev;       // [entries of level k-1][prev_stride]; not read at k = 1
+    int64_t prev_stride;
+    double2* cur;              // [B][cur_stride] (or null: the last level)
+    int64_t cur_stride;
+    double2* amp;              // last level: at [b][i - lo], stride out_stride, scaled
+    double* prob;
+    int64_t out_stride;
+    double norm_t;             // 1 / sqrt(prod t!)
+    double* weighted;          // kExpandSubsets: weight * |a|^2 at [b][i], stride count, or null
+    double weight;
+    double sqrtfact[PCV_MAX_PHOTONS + 1];   // sqrt(j!)
+};
+
+// Fills the fields that depend on no particular level (sqrtfact included).
+void expand_defaults(ExpandArgs* a);
+cudaError_t launch_expand(const ExpandArgs& a, cudaStream_t s);
+
+#ifdef __CUDACC__
+// Sorted mode list of index i of S_{m,k}, from the shared or global table t
+// (row length w1): t[a * w1 + j] = MC(a, j).
+template <typename I>
+__device__ __forceinline__ int next_mode(const I* t, int w1, int m, int v, int rest, I& idx)
+{
+    for (;;) {
+        const I c = t[(m - v) * w1 + rest];
+        if (idx < c) return v;
+        idx -= c;
+        ++v;
+    }
+}
+#endif
+
+}  // namespace pcv

@@ -146,6 +146,15 @@ struct MultQueue {
 cudaError_t launch_glynn_mult(const pcv_batch_desc& d, int parts, int side, double2* partial, cudaStream_t s);
 cudaError_t launch_glynn_mult_persistent(const pcv_batch_desc* descs, const MultQueue& q, int sms, cudaStream_t s);
 
+// Explicit outputs from two half expansions (split.cu): FP64 instructions
+// (-1: does not apply), workspace, and the many-unitaries form, which needs
+// none.
+double split_cost(int m, int n, int64_t n_out);
+int64_t split_workspace(int m, int n);
+cudaError_t launch_split(const Plan& p, const pcv_batch_desc& d, void* ws, cudaStream_t s);
+bool split_multi_applies(int m, int n, int64_t n_out);
+cudaError_t launch_split_multi(const Plan& p, const pcv_batch_desc& d, int B, cudaStream_t s);
+
 // Adjoint (adjoint.cu): the plan of one call (B batch entries, `count`
 // outputs each) in a workspace of ws_bytes (< 0: the default budget): Gray
 // sequence split in `parts` of part_steps, lanes per row q and columns per
@@ -190,9 +199,37 @@ cudaError_t launch_class_conv(const int64_t* mc, const int64_t* cum, int m, int 
 cudaError_t launch_scale_add(double* acc, const double* x, double w, int64_t count, cudaStream_t s);
 cudaError_t launch_set_one(double* p, cudaStream_t s);
 
+// The source model over all pure sets at once (distinguish.cu); total -1
+// where it does not apply.  N[k] = |S_{m,k}|.
+struct SourcePlan {
+    int64_t N[18];
+    size_t table, amp, st[2];
+    int64_t total;
+};
+SourcePlan source_plan(int m, int n, const int64_t* N);
+cudaError_t launch_source(const SourcePlan& p, int m, int n, const int* modes, const double2* U, double alpha,
+                          double beta, double gamma, double* prob, void* ws, cudaStream_t s);
+
 // Photon-by-photon state expansion (slos.cu)
+// outputs [lo, hi) of every batch entry, at [b][o - lo]
 int64_t slos_workspace(int B, int m, int n);
-cudaError_t launch_slos(const Plan& p, int B, const double2* U, double* prob, double2* amp, void* ws, cudaStream_t s);
+cudaError_t launch_slos(const Plan& p, int B, const double2* U, int64_t lo, int64_t hi, double* prob, double2* amp,
+                        void* ws, cudaStream_t s);
+
+// Adjoint of the full distribution by the state expansion
+// (expansion_grad.cu).  The plan's total is -1 where it does not apply (n = 0,
+// or a level beyond 32-bit indices).
+struct ExpandGradPlan {
+    int64_t cnt[PCV_MAX_PHOTONS + 1];    // states of level L
+    int64_t off[PCV_MAX_PHOTONS + 1];    // states of the levels below L
+    int64_t tiles[PCV_MAX_PHOTONS], base[PCV_MAX_PHOTONS];   // blocks and partial sums of level L
+    int64_t parts;
+    size_t table, succ, levels, d0, d1, part;
+    int64_t total;
+};
+ExpandGradPlan expand_grad_plan(int m, int n, int B);
+cudaError_t launch_expand_grad(const Plan& p, const double2* U, int B, const double2* gbar, double2* gradU, void* ws,
+                               const ExpandGradPlan& gp, cudaStream_t s);
 
 // Factorised full distribution (glynn_dist.cu)
 struct DistPlan {
