@@ -439,9 +439,13 @@ int pcv_amplitudes_backward_multi(const pcv_c64* U, int B, int m, const uint8_t*
                                   pcv_c64* grad_U, void* workspace, int64_t workspace_bytes, void* stream);
 
 /* The same for every output of the distributions of B unitaries (grad_amp
- * [B][C(m+n-1,n)] in canonical order, grad_U [B][m][m]); the workspace
- * (default plan: pcv_distribution_backward_workspace(B, m, n)) also holds the
- * multiset-count table used to unrank outputs. */
+ * [B][C(m+n-1,n)] in canonical order, grad_U [B][m][m]), by the state
+ * expansion run in reverse: D_n(S) = grad_amp(S) sqrt(prod S!) / sqrt(prod t!),
+ * D_{k-1}(s) = sum_r conj(U[r][c_k]) D_k(s + e_r), grad_U[r][c_k] += sum_s
+ * D_k(s + e_r) conj(C_{k-1}(s)), every sum in one fixed order.  A workspace
+ * smaller than pcv_distribution_backward_workspace(B, m, n) takes the minors
+ * as Glynn sums instead, in chunks (its minimum as above, with the multiset
+ * table). */
 int64_t pcv_distribution_backward_workspace(int B, int m, int n);
 int pcv_distribution_backward(const pcv_c64* U, int B, int m, const uint8_t* input_occ,
                               const pcv_c64* grad_amp, pcv_c64* grad_U,

@@ -892,12 +892,18 @@ int pcv_amplitudes_backward_multi(const pcv_c64* U, int B, int m, const uint8_t*
     return e == cudaSuccess ? PCV_OK : cuda_fail(e, "adjoint");
 }
 
+// The reverse state expansion is planned for by default up to this many
+// bytes; a smaller workspace takes the minors as Glynn sums.
+constexpr int64_t kGradBudget = 16ll << 30;
+
 int64_t pcv_distribution_backward_workspace(int B, int m, int n)
 {
     if (B < 1 || m < 1 || m > PCV_MAX_MODES || n < 0 || n > PCV_MAX_PHOTONS) return fail(PCV_EINVAL, "bad sizes");
     const int64_t N = msets(m, n);
     if (N < 0) return fail(PCV_ERANGE, "output space too large");
-    return (int64_t)pcv::adjoint_plan(m, n, B, N, -1).total;
+    const int64_t r = (int64_t)pcv::adjoint_plan(m, n, B, N, -1).total;
+    const int64_t x = pcv::expand_grad_plan(m, n, B).total;
+    return x <= kGradBudget ? std::max(r, x) : r;
 }
 
 int pcv_distribution_backward(const pcv_c64* U, int B, int m, const uint8_t* input_occ,
@@ -913,6 +919,12 @@ int pcv_distribution_backward(const pcv_c64* U, int B, int m, const uint8_t* inp
     pcv::AdjPlan ap;
     int rc = backward_common(U, B, m, input_occ, N, grad_amp, grad_U, workspace, workspace_bytes, &p, &ap);
     if (rc) return rc;
+    const pcv::ExpandGradPlan gp = pcv::expand_grad_plan(m, p.n, B);
+    if (gp.total >= 0 && workspace && workspace_bytes >= gp.total) {
+        cudaError_t e = pcv::launch_expand_grad(p, (const double2*)U, B, (const double2*)grad_amp, (double2*)grad_U,
+                                                workspace, gp, (cudaStream_t)stream);
+        return e == cudaSuccess ? PCV_OK : cuda_fail(e, "distribution adjoint");
+    }
     cudaError_t e = pcv::launch_adjoint(p, (const double2*)U, B, nullptr, N, (const double2*)grad_amp,
                                         (double2*)grad_U, workspace, ap, (cudaStream_t)stream);
     return e == cudaSuccess ? PCV_OK : cuda_fail(e, "distribution adjoint");
