@@ -398,7 +398,10 @@ int64_t pcv_distribution_source_workspace(int m, const uint8_t* input_occ);
  * splitter show HOM visibility = indistinguishability. Pure photons form one
  * class, each noisy photon a class of its own; the result is the mixture
  * over all 2^n choices of the pure set, each folded with the other photons'
- * (absent or noisy) one-photon terms.
+ * (absent or noisy) one-photon terms.  With the workspace of
+ * pcv_distribution_source_workspace all sets of one size run in one launch;
+ * a smaller one (the tables, two photon-number-resolved vectors and one
+ * distribution's workspace) takes the sets one after the other.
  *   prob  device, pcv_distribution_source_size(m, n) doubles (written): the
  *         blocks S_{m,0}, S_{m,1}, ..., S_{m,n} concatenated, each in
  *         canonical order; they sum to 1 together.

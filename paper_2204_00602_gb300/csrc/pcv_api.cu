@@ -1194,6 +1194,19 @@ int64_t source_ws(int m, int n)
     return tables_bytes(m, n) + 2 * (int64_t)align256((size_t)T * 8) + dws;
 }
 
+// The plan over all pure sets at once, up to this many bytes; a smaller
+// workspace (or a larger problem) takes one pure set at a time.
+constexpr int64_t kSourceBudget = 8ll << 30;
+
+pcv::SourcePlan make_source_plan(int m, int n)
+{
+    int64_t N[18];
+    for (int k = 0; k <= n; ++k) N[k] = msets(m, k);
+    pcv::SourcePlan p = pcv::source_plan(m, n, N);
+    if (p.total > kSourceBudget) p.total = -1;
+    return p;
+}
+
 int check_source_input(int m, const uint8_t* input_occ, int* n)
 {
     if (m < 1 || m > PCV_MAX_MODES) return fail(PCV_EINVAL, "m=%d outside [1, %d]", m, PCV_MAX_MODES);
@@ -1219,7 +1232,8 @@ int64_t pcv_distribution_source_workspace(int m, const uint8_t* input_occ)
     int n = 0;
     const int rc = check_source_input(m, input_occ, &n);
     if (rc) return rc;
-    return source_ws(m, n);
+    const int64_t one = source_ws(m, n);
+    return one < 0 ? one : std::max(one, make_source_plan(m, n).total);
 }
 
 int pcv_distribution_source(const pcv_c64* U, int m, const uint8_t* input_occ, double transmittance,
@@ -1240,6 +1254,18 @@ int pcv_distribution_source(const pcv_c64* U, int m, const uint8_t* input_occ, d
         return fail(PCV_ENOMEM, "workspace of %lld bytes needed, %lld given", (long long)need, (long long)workspace_bytes);
     if (!aligned(workspace, 256)) return fail(PCV_EINVAL, "workspace is not 256-byte aligned");
     cudaStream_t s = (cudaStream_t)stream;
+    // photon j enters mode modes[j]; a photon is absent (1 - eta), pure
+    // (eta q) or noisy (eta (1 - q)), q = sqrt(indistinguishability)
+    int modes[PCV_MAX_PHOTONS];
+    for (int j = 0, c = 0; j < m; ++j)
+        for (int r = 0; r < input_occ[j]; ++r) modes[c++] = j;
+    const double eta = transmittance, q = std::sqrt(indistinguishability);
+    const double alpha = 1.0 - eta, beta = eta * (1.0 - q), gamma = eta * q;
+    const pcv::SourcePlan sp = make_source_plan(m, n);
+    if (sp.total >= 0 && workspace_bytes >= sp.total) {
+        cudaError_t e = pcv::launch_source(sp, m, n, modes, (const double2*)U, alpha, beta, gamma, prob, workspace, s);
+        return e == cudaSuccess ? PCV_OK : cuda_fail(e, "source model");
+    }
     const int64_t T = graded_size(m, n);
     int64_t off[PCV_MAX_PHOTONS + 2];
     off[0] = 0;
@@ -1255,13 +1281,6 @@ int pcv_distribution_source(const pcv_c64* U, int m, const uint8_t* input_occ, d
     if (e != cudaSuccess) return cuda_fail(e, "clear output");
     if ((e = pcv::build_multiset_table(mc, m, n, s)) != cudaSuccess) return cuda_fail(e, "multiset table");
     if ((e = pcv::build_cum_table(mc, m, n, cum, s)) != cudaSuccess) return cuda_fail(e, "rank table");
-    // photon j enters mode modes[j]; a photon is absent (1 - eta), pure
-    // (eta q) or noisy (eta (1 - q)), q = sqrt(indistinguishability)
-    int modes[PCV_MAX_PHOTONS];
-    for (int j = 0, c = 0; j < m; ++j)
-        for (int r = 0; r < input_occ[j]; ++r) modes[c++] = j;
-    const double eta = transmittance, q = std::sqrt(indistinguishability);
-    const double alpha = 1.0 - eta, beta = eta * (1.0 - q), gamma = eta * q;
     std::vector<uint8_t> tP(m);
     for (uint32_t P = 0; P < (1u << n); ++P) {
         const int kP = __builtin_popcount(P);
