@@ -97,7 +97,9 @@ enum {
     PCV_ALGO_FACTOR_TC = 7, /* factorised Glynn sum, products on the tensor cores (exact digits) */
 };
 
-/* Workspace bytes pcv_amplitudes needs for these sizes (0 if none). */
+/* Workspace bytes pcv_amplitudes wants for these sizes (0 if none).  Where
+ * PCV_ALGO_AUTO would use two half expansions, less is accepted too, down to
+ * the Glynn kernel's own need. */
 int64_t pcv_amplitudes_workspace(int m, int n, int64_t n_out);
 
 /* Amplitudes a(S) of explicit outputs (Eq. eqperm; the Naive back-end's
@@ -113,8 +115,12 @@ int64_t pcv_amplitudes_workspace(int m, int n, int64_t n_out);
  * vectors d with d_1 = +1 of (prod_k d_k) prod_i sum_j d_j a_ij, with the
  * sign vectors visited in reflected Gray-code order so each step updates the
  * row sums by one column (Sec. 3.2.3 names Glynn's algorithm).  The kernel
- * is chosen from m, n and n_out: with m <= 128 and enough outputs to fill
- * the GPU, the shared-row-sum tile kernel (n <= 12), or for n >= 13 a
+ * is chosen from m, n and n_out: where the whole product polynomial splits
+ * cheaply (n <= 16, m moderate, enough outputs), a(S) is summed over the
+ * ways to give the first half of the photons a part of S, from the state
+ * expansions of the two halves (at most C(n, n/2) terms per output; needs the
+ * workspace pcv_amplitudes_workspace names, a smaller one takes the Glynn
+ * kernels); else, with m <= 128 and enough outputs to fill the GPU, the shared-row-sum tile kernel (n <= 12), or for n >= 13 a
  * per-output choice between the tile kernel and Glynn's sum with
  * multiplicities (PCV_ALGO_MULT below), whichever issues fewer FP64
  * instructions for that output; otherwise the plain Glynn kernels. */
@@ -334,7 +340,8 @@ int pcv_distribution_ex(const pcv_c64* U, int m, const uint8_t* input_occ,
                         double* prob, pcv_c64* amp, int algo, int param,
                         void* workspace, int64_t workspace_bytes, void* stream);
 
-/* The same explicit outputs for B unitaries with one input state (the tile
+/* The same explicit outputs for B unitaries with one input state (two half
+ * expansions held in shared memory where they fit, n <= 10, else the tile
  * kernel of PCV_ALGO_TILE with a batch dimension; m <= 128, n >= 1).
  *   U       device, B*m*m pcv_c64;  output_occ device, n_out*m uint8
  *   amp     device, B*n_out pcv_c64 or NULL;  prob device, B*n_out doubles or NULL */

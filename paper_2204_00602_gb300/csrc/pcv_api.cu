@@ -99,6 +99,23 @@ int auto_splits(int n, int64_t n_out)
 
 struct AmpChoice { int algo, param; };
 
+// PCV_ALGO_AUTO takes the two half expansions (split.cu) when they need
+// clearly fewer FP64 instructions than the Glynn kernel it would choose
+// otherwise: their k1 + 2 launches cost about as much as kSplitOverhead
+// instructions, and from kRouteMinPhotons on bunched outputs can cost the
+// routed kernels a small part of 2^{n-1} (4n - 2), so an eighth of it is
+// compared.  Measured at m=20 n=10, 4096 outputs: 307 us by the group kernel.
+constexpr double kSplitOverhead = 8e6;
+constexpr int64_t kSplitBudget = 1ll << 30;
+
+bool split_pays(int m, int n, int64_t n_out)
+{
+    const double c = pcv::split_cost(m, n, n_out);
+    if (c < 0.0 || pcv::split_workspace(m, n) > kSplitBudget || n_out * 32 > INT32_MAX) return false;
+    const double plain = std::ldexp(4.0 * n - 2.0, n - 1) * (double)n_out;
+    return c + kSplitOverhead < (n >= kRouteMinPhotons ? plain / 8 : plain);
+}
+
 AmpChoice choose_amp(int m, int n, int64_t n_out, int algo, int param)
 {
     if (algo == PCV_ALGO_AUTO) {
@@ -155,6 +172,29 @@ int64_t amp_workspace(const AmpChoice& c, int64_t n_out)
     if ((c.algo == PCV_ALGO_BLOCK || c.algo == PCV_ALGO_MULT) && c.param > 1)
         return (int64_t)align256((size_t)n_out * c.param * sizeof(double2));
     return 0;
+}
+
+// Workspace of PCV_ALGO_AUTO: what lets it take its first choice.  A smaller
+// one, down to the Glynn kernel's own need (often none), is accepted.
+int64_t auto_amp_workspace(int m, int n, int64_t n_out)
+{
+    const int64_t w = amp_workspace(choose_amp(m, n, n_out, PCV_ALGO_AUTO, 0), n_out);
+    return split_pays(m, n, n_out) ? std::max(w, pcv::split_workspace(m, n)) : w;
+}
+
+pcv_batch_desc make_desc(const pcv::Plan& p, const pcv_c64* U, const uint8_t* outputs, int64_t n_out, pcv_c64* amp,
+                         double* prob)
+{
+    pcv_batch_desc d;
+    d.U = U;
+    d.outputs = outputs;
+    d.amp = amp;
+    d.prob = prob;
+    d.n_out = n_out;
+    d.m = p.m;
+    d.n = p.n;
+    for (int j = 0; j < PCV_MAX_PHOTONS; ++j) d.cols[j] = p.cols[j];
+    return d;
 }
 
 // ------------------------------------------------------ stage timing
@@ -324,7 +364,7 @@ int64_t pcv_rank(int m, const uint8_t* occ)
 int64_t pcv_amplitudes_workspace(int m, int n, int64_t n_out)
 {
     if (m < 1 || m > PCV_MAX_MODES || n < 0 || n > PCV_MAX_PHOTONS || n_out < 0) return fail(PCV_EINVAL, "bad sizes");
-    return amp_workspace(choose_amp(m, n, n_out, PCV_ALGO_AUTO, 0), n_out);
+    return auto_amp_workspace(m, n, n_out);
 }
 
 int64_t pcv_amplitudes_ex_workspace(int m, int n, int64_t n_out, int algo, int param)
@@ -334,7 +374,7 @@ int64_t pcv_amplitudes_ex_workspace(int m, int n, int64_t n_out, int algo, int p
     const AmpChoice c = choose_amp(m, n, n_out, algo, param);
     const int rc = check_choice(c, n);
     if (rc) return rc;
-    return amp_workspace(c, n_out);
+    return algo == PCV_ALGO_AUTO ? auto_amp_workspace(m, n, n_out) : amp_workspace(c, n_out);
 }
 
 int pcv_amplitudes_ex(const pcv_c64* U, int m, const uint8_t* input_occ,
@@ -357,6 +397,13 @@ int pcv_amplitudes_ex(const pcv_c64* U, int m, const uint8_t* input_occ,
                                                 (double2*)amp, prob, 1, s);
         return e == cudaSuccess ? PCV_OK : cuda_fail(e, "n0 kernel");
     }
+    if (algo == PCV_ALGO_AUTO && split_pays(m, p.n, n_out) && workspace && aligned(workspace, 256) &&
+        workspace_bytes >= pcv::split_workspace(m, p.n)) {
+        pcv::stage_begin(pcv::kStagePlain, s);
+        cudaError_t e = pcv::launch_split(p, make_desc(p, U, output_occ, n_out, amp, prob), workspace, s);
+        pcv::stage_end(pcv::kStagePlain, s);
+        return e == cudaSuccess ? PCV_OK : cuda_fail(e, "split launch");
+    }
     AmpChoice c = choose_amp(m, p.n, n_out, algo, param);
     if ((rc = check_choice(c, p.n))) return rc;
     const int64_t need = amp_workspace(c, n_out);
@@ -366,15 +413,7 @@ int pcv_amplitudes_ex(const pcv_c64* U, int m, const uint8_t* input_occ,
     if ((int64_t)n_out * ((c.algo == PCV_ALGO_BLOCK || c.algo == PCV_ALGO_MULT) ? c.param : 1) > INT32_MAX)
         return fail(PCV_ERANGE, "too many permanents for one launch");
     if (c.algo == kAlgoRouted) {
-        pcv_batch_desc d;
-        d.U = U;
-        d.outputs = output_occ;
-        d.amp = amp;
-        d.prob = prob;
-        d.n_out = n_out;
-        d.m = m;
-        d.n = p.n;
-        for (int j = 0; j < PCV_MAX_PHOTONS; ++j) d.cols[j] = p.cols[j];
+        const pcv_batch_desc d = make_desc(p, U, output_occ, n_out, amp, prob);
         int dev = 0, sms = 0;
         cudaError_t e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -388,15 +427,7 @@ int pcv_amplitudes_ex(const pcv_c64* U, int m, const uint8_t* input_occ,
         return e == cudaSuccess ? PCV_OK : cuda_fail(e, "routed launch");
     }
     if (c.algo == PCV_ALGO_MULT) {
-        pcv_batch_desc d;
-        d.U = U;
-        d.outputs = output_occ;
-        d.amp = amp;
-        d.prob = prob;
-        d.n_out = n_out;
-        d.m = m;
-        d.n = p.n;
-        for (int j = 0; j < PCV_MAX_PHOTONS; ++j) d.cols[j] = p.cols[j];
+        const pcv_batch_desc d = make_desc(p, U, output_occ, n_out, amp, prob);
         pcv::stage_begin(pcv::kStagePlain, s);
         cudaError_t e = pcv::launch_glynn_mult(d, c.param, 0, (double2*)workspace, s);
         pcv::stage_end(pcv::kStagePlain, s);
@@ -404,15 +435,7 @@ int pcv_amplitudes_ex(const pcv_c64* U, int m, const uint8_t* input_occ,
     }
     if (c.algo == PCV_ALGO_TILE) {
         if (m > pcv::tile_max_modes()) return fail(PCV_EINVAL, "tile kernel supports m <= %d (m=%d)", pcv::tile_max_modes(), m);
-        pcv_batch_desc d;
-        d.U = U;
-        d.outputs = output_occ;
-        d.amp = amp;
-        d.prob = prob;
-        d.n_out = n_out;
-        d.m = m;
-        d.n = p.n;
-        for (int j = 0; j < PCV_MAX_PHOTONS; ++j) d.cols[j] = p.cols[j];
+        const pcv_batch_desc d = make_desc(p, U, output_occ, n_out, amp, prob);
         pcv::stage_begin(pcv::kStagePlain, s);
         cudaError_t e = pcv::launch_glynn_tile(d, s);
         pcv::stage_end(pcv::kStagePlain, s);
@@ -451,20 +474,13 @@ int pcv_amplitudes_multi(const pcv_c64* U, int B, int m, const uint8_t* input_oc
     if (n_out == 0) return PCV_OK;
     if (!output_occ || (!amp && !prob)) return fail(PCV_EINVAL, "bad output pointers");
     if (amp && !aligned(amp, 16)) return fail(PCV_EINVAL, "amp is not 16-byte aligned");
-    pcv_batch_desc d;
-    d.U = U;
-    d.outputs = output_occ;
-    d.amp = amp;
-    d.prob = prob;
-    d.n_out = n_out;
-    d.m = m;
-    d.n = p.n;
-    for (int j = 0; j < PCV_MAX_PHOTONS; ++j) d.cols[j] = p.cols[j];
+    const pcv_batch_desc d = make_desc(p, U, output_occ, n_out, amp, prob);
     cudaStream_t s = (cudaStream_t)stream;
+    const bool split = pcv::split_multi_applies(m, p.n, n_out);
     pcv::stage_begin(pcv::kStagePlain, s);
-    cudaError_t e = pcv::launch_glynn_tile_multi(d, B, s);
+    cudaError_t e = split ? pcv::launch_split_multi(p, d, B, s) : pcv::launch_glynn_tile_multi(d, B, s);
     pcv::stage_end(pcv::kStagePlain, s);
-    return e == cudaSuccess ? PCV_OK : cuda_fail(e, "tile multi launch");
+    return e == cudaSuccess ? PCV_OK : cuda_fail(e, split ? "split multi launch" : "tile multi launch");
 }
 
 int64_t pcv_amplitudes_batched_workspace(int n_circ, int64_t total_outputs)
