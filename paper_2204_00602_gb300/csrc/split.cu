@@ -27,7 +27,11 @@
 //                       both tables of its unitaries in shared memory and a
 //                       thread takes an output.  The ranks do not depend on
 //                       the unitary, so a thread forms them once for the
-//                       block's kMulti unitaries.
+//                       block's kMulti unitaries.  Its callers take logarithms
+//                       of probabilities that can be zero but for rounding; an
+//                       amplitude below 2^-30 of the product of its rows'
+//                       norms, where rounding decides, is formed by Glynn's
+//                       sum in the tile kernel's FP64 order (glynn_row_sums).
 
 #include <algorithm>
 #include <cmath>
@@ -240,6 +244,31 @@ struct SplitMultiArgs {
     int n1, n2, ns;                      // |S_{m,k1}|, |S_{m,k2}|, |S_{m,k1-1}| (scratch)
 };
 
+// Glynn's sum of one output in Gray order, rows ascending, FP64 throughout.
+template <int NMAX>
+__device__ __noinline__ double2 glynn_row_sums(const double2* U, const SplitMultiArgs& a, const int* row)
+{
+    const int m = a.o.m, n = a.o.n, w1 = a.o.k1 + 1;
+    double2 y[NMAX];
+    for (int i = 0; i < n; ++i) {
+        const double2* Ur = U + (size_t)(m - 1 - row[i] / w1) * m;
+        y[i] = Ur[a.cols[0]];
+        for (int j = 1; j < n; ++j) caxpy(y[i], 1.0, Ur[a.cols[j]]);
+    }
+    double2 acc = make_double2(0.0, 0.0);
+    const uint32_t steps = 1u << (n - 1);
+    for (uint32_t k = 0; k < steps; ++k) {
+        double2 p = y[0];
+        for (int i = 1; i < n; ++i) p = cmul(p, y[i]);
+        caxpy(acc, (k & 1) ? -1.0 : 1.0, p);
+        if (k + 1 == steps) break;
+        const int b = __ffs(k + 1) - 1;
+        const double sd = (((k + 1) >> (b + 1)) & 1) ? 2.0 : -2.0;
+        for (int i = 0; i < n; ++i) caxpy(y[i], sd, U[(size_t)(m - 1 - row[i] / w1) * m + a.cols[b + 1]]);
+    }
+    return acc;
+}
+
 template <int NMAX>
 __global__ void __launch_bounds__(kThreads) split_multi_kernel(const __grid_constant__ SplitMultiArgs a)
 {
@@ -248,8 +277,18 @@ __global__ void __launch_bounds__(kThreads) split_multi_kernel(const __grid_cons
     double2* s_scratch = s_tab + kMulti * (a.n1 + a.n2);
     double2* s_u = s_scratch + a.ns;
     uint32_t* s_t = (uint32_t*)(s_u + m);
+    int* s_e = (int*)(s_t + (m + 1) * w1);   // per unitary and mode: exponent of the row's squared norm
     const int b0 = blockIdx.y * kMulti;
     count_table(s_t, m, k1);
+    for (int q = threadIdx.x; q < kMulti * m; q += kThreads) {
+        const double2* Ur = a.U + ((size_t)min(b0 + q / m, a.B - 1) * m + q % m) * m;
+        double f = 0.0;
+        for (int j = 0; j < n; ++j) {
+            const double2 u = Ur[a.cols[j]];
+            f = fma(u.x, u.x, fma(u.y, u.y, f));
+        }
+        s_e[q] = f > 0.0 && isfinite(f) ? ilogb(f) : 0;
+    }
     // both tables of each unitary, level by level; the last level lands in
     // place, the one before in the scratch, and so on back
     for (int j = 0; j < kMulti; ++j) {
@@ -335,7 +374,21 @@ __global__ void __launch_bounds__(kThreads) split_multi_kernel(const __grid_cons
 #pragma unroll
         for (int j = 0; j < kMulti; ++j) {
             if (b0 + j >= a.B) break;
-            const double2 v = ok ? make_double2(acc[j].x * sc, acc[j].y * sc) : make_double2(0.0, 0.0);
+            double2 v = make_double2(0.0, 0.0);
+            if (ok) {
+                const double w = fma(acc[j].x, acc[j].x, acc[j].y * acc[j].y) * f;      // |Perm|^2 / prod S!
+                int e = -60;
+#pragma unroll
+                for (int p = 0; p < NMAX; ++p)
+                    if (p < n) e += s_e[j * m + m - 1 - row[p] / w1];
+                if (w < scalbn(1.0, e)) {
+                    const double gs = ldexp(1.0 / sqrt(f) * a.o.norm_t, -(n - 1));
+                    const double2 g = glynn_row_sums<NMAX>(a.U + (size_t)(b0 + j) * m * m, a, row);
+                    v = make_double2(g.x * gs, g.y * gs);
+                } else {
+                    v = make_double2(acc[j].x * sc, acc[j].y * sc);
+                }
+            }
             const int64_t at = (int64_t)(b0 + j) * a.o.n_out + o;
             if (a.o.amp) a.o.amp[at] = v;
             if (a.o.prob) a.o.prob[at] = fma(v.x, v.x, v.y * v.y);
@@ -373,7 +426,8 @@ size_t multi_smem(int m, int n)
     const int k1 = (n + 1) / 2;
     const int64_t n1 = mset_h(m, k1), n2 = mset_h(m, n - k1), ns = mset_h(m, k1 - 1);
     if (n1 < 0 || n1 > (1 << 20)) return SIZE_MAX;
-    return (size_t)(kMulti * (n1 + n2) + ns + m) * sizeof(double2) + (size_t)(m + 1) * (k1 + 1) * sizeof(uint32_t);
+    return (size_t)(kMulti * (n1 + n2) + ns + m) * sizeof(double2) + (size_t)(m + 1) * (k1 + 1) * sizeof(uint32_t) +
+           (size_t)kMulti * m * sizeof(int);
 }
 
 SplitOut split_out(const pcv_batch_desc& d, double norm_t)
