@@ -10,10 +10,27 @@
 // The k leave-one-column-out permanents come from one Glynn sum over the
 // k-1 rows: with x_j(d) = sum_i d_i M[i][j] and leave-one-out products,
 //     Perm(M_{-l}) = 2^{-(k-2)} sum_{d, d_1=+1} (prod d) prod_{j != l} x_j(d).
-// One warp per sample: lanes split the Gray-code sequence of sign vectors
-// (shuffle reduction), then the m weights, then an inverse-CDF draw with a
-// warp prefix sum.  The random numbers (column permutation, one uniform per
-// photon) are inputs, so a sample is a deterministic function of them.
+// The random numbers (column permutation, one uniform per photon) are inputs,
+// so a sample is a deterministic function of them.
+//
+// Two forms of the sub-permanents:
+//   subset_sampler_kernel  n <= 15: f_k(S) = Perm(A[r_1..r_k; S]) for every
+//                          k-subset S of the n columns, level by level,
+//                              f_k(S) = sum_{l in S} A[r_k][l] f_{k-1}(S \ l),
+//                          so f_{k-1}({0..k-1} \ l) are the k sub-permanents
+//                          of step k: n 2^{n-1} complex multiply-adds for the
+//                          whole sample, 4 FP64 instructions each, where the
+//                          Glynn sums of the steps take about 14 n 2^{n-1}
+//                          (n = 14: 0.46 M against 1.6 M), and no sign
+//                          cancellation.  Two neighbouring levels live in
+//                          shared memory (n = 14: 103 KB, two samples per SM;
+//                          n = 15: 206 KB), which ends the form at n = 15;
+//   sampler_kernel         n = 16: one Glynn sum per step (below), one warp
+//                          per sample, lanes splitting the Gray-code sequence.
+// Either way the m weights follow, then an inverse-CDF draw with a warp
+// prefix sum.
+
+#include <algorithm>
 
 #include "pcv_common.cuh"
 
@@ -31,6 +48,169 @@ struct SampArgs {
     int64_t count;
     uint8_t* out;             // [count][m] occupations
 };
+
+// Inverse-CDF draw by one warp from the weights of its lanes (wloc[c]: mode
+// lane + 32 c; the cumulative order runs lane by lane), u in [0, 1).
+__device__ int draw_mode(const double* wloc, int m, double u)
+{
+    const int lane = threadIdx.x & 31;
+    double part = 0.0;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) part += wloc[c];
+    // total and lane prefix of the per-lane sums
+    double incl = part;
+    for (int off = 1; off < 32; off <<= 1) {
+        const double v = __shfl_up_sync(0xffffffffu, incl, off);
+        if (lane >= off) incl += v;
+    }
+    const double total = __shfl_sync(0xffffffffu, incl, 31);
+    const double target = u * total;
+    // the lane whose cumulative range holds the target picks within its modes
+    const double before = incl - part;
+    int pick = -1;
+    if (target >= before && target < incl) {
+        double acc = before;
+        int lastpos = -1;
+        for (int c = 0; c < 4; ++c) {
+            const int i = lane + 32 * c;
+            if (i >= m) break;
+            if (wloc[c] > 0.0) lastpos = i;
+            acc += wloc[c];
+            if (target < acc) { pick = i; break; }
+        }
+        if (pick < 0) pick = lastpos;          // rounding: this lane's last mode with weight
+    }
+    const unsigned ball = __ballot_sync(0xffffffffu, pick >= 0);
+    if (ball) return __shfl_sync(0xffffffffu, pick, __ffs(ball) - 1);
+    int last = -1;                             // rounding at the top end: last mode with weight
+    for (int c = 3; c >= 0 && last < 0; --c) {
+        const int i = lane + 32 * c;
+        if (i < m && wloc[c] > 0.0) last = i;
+    }
+    for (int off = 16; off > 0; off >>= 1) last = max(last, __shfl_xor_sync(0xffffffffu, last, off));
+    return last < 0 ? 0 : last;
+}
+
+// Entries of the even and odd levels 1 .. n-1 (C(n, k) at most).
+__host__ __device__ inline int subset_level(int n, int odd)
+{
+    int c = 1, best = 1;
+    for (int k = 1; k < n; ++k) {
+        c = c * (n + 1 - k) / k;
+        if ((k & 1) == odd && c > best) best = c;
+    }
+    return best;
+}
+
+// Shared memory of one sample: two levels, the drawn row, the weights, the
+// sample's columns and rows.
+__host__ __device__ inline size_t subset_bytes(int m, int n)
+{
+    return (size_t)(subset_level(n, 0) + subset_level(n, 1) + n) * sizeof(double2) +
+           (size_t)(m + (m & 1)) * sizeof(double) + 2 * 16 * sizeof(int);      // a multiple of 16
+}
+
+constexpr int kBinom = 17;
+
+// Position of the lowest bit (15 for none: a valid row of the tables).
+__device__ __forceinline__ int low_bit(uint32_t x) { return (__ffs((int)x) - 1) & 15; }
+
+// A group of T threads per sample (T = 32: several samples per block).
+template <int T>
+__global__ void subset_sampler_kernel(const __grid_constant__ SampArgs a)
+{
+    extern __shared__ double2 s_mem[];
+    __shared__ int s_c[kBinom][kBinom];        // C(t, j)
+    for (int q = threadIdx.x; q < kBinom * kBinom; q += blockDim.x) {
+        const int t = q / kBinom, j = q % kBinom;
+        int c = j <= t ? 1 : 0;
+        for (int i = 1; i <= j && j <= t; ++i) c = c * (t + 1 - i) / i;
+        s_c[t][j] = c;
+    }
+    __syncthreads();
+    const int m = a.m, n = a.n;
+    const int grp = threadIdx.x / T, tid = threadIdx.x % T;
+    const int64_t smp = (int64_t)blockIdx.x * (blockDim.x / T) + grp;
+    if (smp >= a.count) return;                // whole groups
+    auto sync = [] {
+        if (T == 32) __syncwarp();
+        else __syncthreads();
+    };
+    const int n_even = subset_level(n, 0), n_odd = subset_level(n, 1);
+    double2* base = (double2*)((char*)s_mem + (size_t)grp * subset_bytes(m, n));
+    double2* s_a = base + n_even + n_odd;      // A[r_k][.], the drawn row
+    double* s_w = (double*)(s_a + n);
+    int* s_pc = (int*)(s_w + m + (m & 1));               // input mode of each permuted photon
+    int* s_rows = s_pc + 16;
+    if (tid < n) s_pc[tid] = a.cols[min((int)a.perm[smp * n + tid], n - 1)];   // clamp keeps reads in bounds
+    sync();
+    for (int k = 1; k <= n; ++k) {
+        // weights: sub-permanent of {0..k-1} \ l is entry k-1-l of level k-1
+        const double2* f = base + ((k - 1) & 1 ? n_even : 0);      // level k - 1: even levels first, then odd
+        for (int i = tid; i < m; i += T) {
+            const double2* Ui = a.U + (size_t)i * m;
+            double2 s = make_double2(0.0, 0.0);
+            if (k == 1) s = __ldg(Ui + s_pc[0]);
+            else
+                for (int l = 0; l < k; ++l) cmac(s, __ldg(Ui + s_pc[l]), f[k - 1 - l]);
+            s_w[i] = fma(s.x, s.x, s.y * s.y);
+        }
+        sync();
+        if (tid < 32) {
+            double wloc[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) wloc[c] = tid + 32 * c < m ? s_w[tid + 32 * c] : 0.0;
+            const int r = draw_mode(wloc, m, a.uni[smp * n + k - 1]);
+            if (tid == 0) s_rows[k - 1] = r;
+            if (tid < n) s_a[tid] = __ldg(a.U + (size_t)r * m + s_pc[tid]);
+        }
+        sync();
+        if (k == n) break;
+        // level k: contiguous runs of subsets (increasing masks) per thread.
+        // The rank of S is sum_i C(s_i, i + 1) over its elements in order;
+        // without s_j the elements after it move down one place.
+        double2* cur = base + (k & 1 ? n_even : 0);
+        const int cnt = s_c[n][k];
+        const int below = s_c[n][k - 1];       // entries of level k - 1
+        const int per = (cnt + T - 1) / T;
+        const int q0 = tid * per;
+        uint32_t mask = 0;
+        for (int b = min(q0, cnt - 1), j = k, t = n - 1; j >= 1; --j) {
+            while (t > 0 && s_c[t][j] > b) --t;
+            mask |= 1u << t;
+            b -= s_c[t][j];
+        }
+        __syncwarp();                          // the search leaves the lanes apart
+        for (int q = q0; q < q0 + per; ++q) {
+            // every lane runs the same k steps (those past the level redo its
+            // last subset and store nothing), so a warp stays together
+            int suf = 0;                       // sum over the elements not yet passed, one place down
+            uint32_t x = mask;
+            for (int i = 0; i < k; ++i, x &= x - 1) suf += s_c[low_bit(x)][i];
+            double2 acc = make_double2(0.0, 0.0);
+            int pre = 0;
+            x = mask;
+            for (int i = 0; i < k; ++i, x &= x - 1) {
+                const int l = low_bit(x);
+                suf -= s_c[l][i];
+                if (k == 1) acc = s_a[l];
+                else cmac(acc, s_a[l], f[min((uint32_t)(pre + suf), (uint32_t)(below - 1))]);
+                pre += s_c[l][i + 1];
+            }
+            if (q < cnt) cur[q] = acc;
+            if (q + 1 < cnt) {
+                const uint32_t c = mask & (0u - mask), r = mask + c;
+                mask = r | (((mask ^ r) >> 2) >> (__ffs(mask) - 1));
+            }
+        }
+        sync();
+    }
+    for (int i = tid; i < m; i += T) {
+        int c = 0;
+        for (int p = 0; p < n; ++p) c += s_rows[p] == i;
+        a.out[smp * m + i] = (uint8_t)c;
+    }
+}
 
 template <int NMAX>
 __global__ void __launch_bounds__(32 * kSampWarps) sampler_kernel(const SampArgs a)
@@ -122,7 +302,6 @@ __global__ void __launch_bounds__(32 * kSampWarps) sampler_kernel(const SampArgs
         }
         // ---- weights of the m candidate positions, inverse-CDF draw
         double wloc[4];
-        double part = 0.0;
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
             const int i = lane + 32 * c;
@@ -135,47 +314,8 @@ __global__ void __launch_bounds__(32 * kSampWarps) sampler_kernel(const SampArgs
                 w = fma(s.x, s.x, s.y * s.y);
             }
             wloc[c] = w;
-            part += w;
         }
-        // total and lane prefix of the per-lane sums (modes lane, lane+32, ... belong to lane)
-        double incl = part;
-        for (int off = 1; off < 32; off <<= 1) {
-            const double v = __shfl_up_sync(0xffffffffu, incl, off);
-            if (lane >= off) incl += v;
-        }
-        const double total = __shfl_sync(0xffffffffu, incl, 31);
-        const double target = uni[k - 1] * total;
-        // the lane whose cumulative range holds the target picks within its modes
-        const double before = incl - part;
-        int pick = -1;
-        if (target >= before && target < incl) {
-            double acc = before;
-            int lastpos = -1;
-            for (int c = 0; c < 4; ++c) {
-                const int i = lane + 32 * c;
-                if (i >= m) break;
-                if (wloc[c] > 0.0) lastpos = i;
-                acc += wloc[c];
-                if (target < acc) { pick = i; break; }
-            }
-            if (pick < 0) pick = lastpos;          // rounding: this lane's last mode with weight
-        }
-        const unsigned ball = __ballot_sync(0xffffffffu, pick >= 0);
-        int chosen;
-        if (ball) {
-            const int src = __ffs(ball) - 1;
-            chosen = __shfl_sync(0xffffffffu, pick, src);
-        } else {                                        // rounding at the top end: last mode with weight
-            int last = -1;
-            for (int c = 3; c >= 0 && last < 0; --c) {
-                const int i = lane + 32 * c;
-                if (i < m && wloc[c] > 0.0) last = i;
-            }
-            int best = last;
-            for (int off = 16; off > 0; off >>= 1) best = max(best, __shfl_xor_sync(0xffffffffu, best, off));
-            chosen = best < 0 ? 0 : best;
-        }
-        rows[k - 1] = chosen;
+        rows[k - 1] = draw_mode(wloc, m, uni[k - 1]);
     }
     for (int i = lane; i < m; i += 32) {
         int c = 0;
@@ -198,20 +338,39 @@ cudaError_t launch_sampler(const Plan& p, const double2* U, const uint8_t* perm,
     a.uni = uni;
     a.count = count;
     a.out = out;
+    cudaError_t e;
+    if (p.n <= 15) {
+        // threads per sample: enough for the largest level of a sample, as many
+        // samples per SM as shared memory holds
+        auto go = [&](auto kernel, int threads, int samples) {
+            const size_t smem = (size_t)samples * subset_bytes(p.m, p.n);
+            cudaError_t r = cudaSuccess;
+            if (smem > 48 * 1024)
+                r = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (r != cudaSuccess) return r;
+            for (int64_t c0 = 0; c0 < count && r == cudaSuccess; c0 += 1 << 30) {      // grid limit
+                SampArgs p1 = a;
+                p1.count = std::min<int64_t>(count - c0, 1 << 30);
+                p1.perm = perm + c0 * p.n;
+                p1.uni = uni + c0 * p.n;
+                p1.out = out + c0 * p.m;
+                kernel<<<(unsigned)((p1.count + samples - 1) / samples), threads, smem, s>>>(p1);
+                note_launches(1);
+                r = cudaGetLastError();
+            }
+            return r;
+        };
+        if (p.n <= 8) return go(subset_sampler_kernel<32>, 256, 8);
+        if (p.n <= 11) return go(subset_sampler_kernel<32>, 64, 2);
+        if (p.n <= 14) return go(subset_sampler_kernel<128>, 128, 1);
+        return go(subset_sampler_kernel<256>, 256, 1);
+    }
     const size_t smem = (size_t)p.m * p.n * sizeof(double2);
     const unsigned blocks = (unsigned)((count + kSampWarps - 1) / kSampWarps);
-    cudaError_t e;
-    if (p.n <= 8) {
-        if (smem > 48 * 1024 &&
-            (e = cudaFuncSetAttribute(sampler_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-            return e;
-        sampler_kernel<8><<<blocks, 32 * kSampWarps, smem, s>>>(a);
-    } else {
-        if (smem > 48 * 1024 &&
-            (e = cudaFuncSetAttribute(sampler_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-            return e;
-        sampler_kernel<16><<<blocks, 32 * kSampWarps, smem, s>>>(a);
-    }
+    if (smem > 48 * 1024 &&
+        (e = cudaFuncSetAttribute(sampler_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+        return e;
+    sampler_kernel<16><<<blocks, 32 * kSampWarps, smem, s>>>(a);
     note_launches(1);
     return cudaGetLastError();
 }
