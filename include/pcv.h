@@ -120,10 +120,11 @@ int64_t pcv_amplitudes_workspace(int m, int n, int64_t n_out);
  * ways to give the first half of the photons a part of S, from the state
  * expansions of the two halves (at most C(n, n/2) terms per output; needs the
  * workspace pcv_amplitudes_workspace names, a smaller one takes the Glynn
- * kernels); else, with m <= 128 and enough outputs to fill the GPU, the shared-row-sum tile kernel (n <= 12), or for n >= 13 a
- * per-output choice between the tile kernel and Glynn's sum with
- * multiplicities (PCV_ALGO_MULT below), whichever issues fewer FP64
- * instructions for that output; otherwise the plain Glynn kernels. */
+ * kernels); else, from about 2e7 FP64 instructions of the plain kernels on,
+ * the shared-row-sum tile kernel with its sign vectors split over blocks, or
+ * for n >= 13 and m <= 128 a per-output choice between that kernel and Glynn's
+ * sum with multiplicities (PCV_ALGO_MULT below), whichever takes less time for
+ * that output; otherwise the plain Glynn kernels. */
 int pcv_amplitudes(const pcv_c64* U, int m, const uint8_t* input_occ,
                    const uint8_t* output_occ, int64_t n_out,
                    pcv_c64* amp, double* prob,
@@ -133,7 +134,8 @@ int pcv_amplitudes(const pcv_c64* U, int m, const uint8_t* input_occ,
  * `param` threads per permanent (1, 2, 4, 8, 16 or 32), PCV_ALGO_BLOCK with
  * `param` blocks per permanent (>= 1), PCV_ALGO_TILE (m <= 128; the row
  * sums y_r(d) = sum_j d_j U[r][c_j] of each sign vector are formed once per
- * block and shared by its 32..256 outputs), or PCV_ALGO_MULT with `param`
+ * block and shared by its 32..256 outputs, the products run on the integer
+ * pipe with 62-bit components, each term is rounded to FP64), or PCV_ALGO_MULT with `param`
  * warps per permanent (1..1024; 0 = chosen from n_out).
  * PCV_ALGO_MULT is Glynn's sum written over the multiplicities of a bunched
  * state (the same identity as above, with the sign vectors of the mu copies
@@ -174,9 +176,13 @@ int64_t pcv_amplitudes_batched_workspace(int n_circ, int64_t total_outputs);
 /* Amplitudes of many circuits of uneven size (Eq. eqperm per circuit).
  * A routing kernel sends each output either to the shared-row-sum tile
  * kernel or to Glynn's sum with multiplicities (PCV_ALGO_MULT), whichever
- * issues fewer FP64 instructions for it; a planning kernel sorts the circuits
+ * takes less time for it; a planning kernel sorts the circuits
  * by photon number (largest first) and expands them into tile items
- * (circuit, tile of 32..256 outputs) and single-output entries.  Two
+ * (circuit, tile of 32..256 outputs, part of the sign vectors: no item holds
+ * more than a twelfth of an SM's share of the tile work, given the workspace
+ * pcv_amplitudes_batched_workspace names; a workspace without room for the
+ * parts' sums, 12 bytes per output and 48 per circuit and more, keeps whole
+ * tiles) and single-output entries.  Two
  * persistent launches then pull from device counters until their queues are
  * empty: blocks take tile items, warps take entries.  No block waits on
  * another.

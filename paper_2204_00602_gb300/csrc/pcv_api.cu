@@ -76,6 +76,8 @@ constexpr int kSMs = 152;
 // launch's per-output routing (tile kernel or Glynn's sum with
 // multiplicities) applied to one circuit.
 constexpr int kAlgoRouted = 100;
+// The tile kernel with each tile's sign vectors split over blocks, any m.
+constexpr int kAlgoTileSplit = 101;
 constexpr int kRouteMinPhotons = 13;
 
 // Threads per permanent for the group kernel: enough threads in flight to
@@ -120,7 +122,8 @@ AmpChoice choose_amp(int m, int n, int64_t n_out, int algo, int param)
 {
     if (algo == PCV_ALGO_AUTO) {
         // shared row sums when there are enough outputs to give every SM a tile
-        if (m <= pcv::tile_max_modes() && n >= 1 && n_out >= (int64_t)kSMs * (256 / pcv::tile_splits(n)))
+        const int splits = n <= 10 ? 1 : n <= 13 ? 2 : n <= 16 ? 4 : 8;
+        if (m <= pcv::tile_max_modes() && n >= 1 && n_out >= (int64_t)kSMs * (256 / splits))
             return {n >= kRouteMinPhotons && n_out <= INT32_MAX ? kAlgoRouted : PCV_ALGO_TILE, 0};
         if (n <= 12 || (n <= 16 && n_out >= (int64_t)kSMs * 256)) return {PCV_ALGO_GROUP, auto_group(n, n_out)};
         return {PCV_ALGO_BLOCK, auto_splits(n, n_out)};
@@ -148,7 +151,7 @@ int check_choice(const AmpChoice& c, int n)
         if (n > 0 && (1ll << (n - 1)) < G) return fail(PCV_EINVAL, "threads per permanent %d exceed 2^(n-1)=%lld", G, 1ll << (n - 1));
         return PCV_OK;
     }
-    if (c.algo == kAlgoRouted) return PCV_OK;
+    if (c.algo == kAlgoRouted || c.algo == kAlgoTileSplit) return PCV_OK;
     if (c.algo == PCV_ALGO_MULT) {
         if (n < 1) return fail(PCV_EINVAL, "multiplicity kernel needs n >= 1");
         if (c.param < 1 || c.param > 1024) return fail(PCV_EINVAL, "warps per permanent %d outside [1, 1024]", c.param);
@@ -174,11 +177,41 @@ int64_t amp_workspace(const AmpChoice& c, int64_t n_out)
     return 0;
 }
 
+// PCV_ALGO_AUTO's choice among the Glynn kernels when the workspace holds it:
+// the tile kernel with split sequences, behind the per-output routing where
+// bunched outputs can be much cheaper (n >= kRouteMinPhotons, m <= 128).  Its
+// integer products cost 1.25 FP64 instructions per photon and lane, a warp 32
+// lanes however few outputs it has, against 6n - 2 of the plain kernels; below
+// kTileOverhead instructions in all the plain kernels' single launch is
+// quicker.  (256 outputs at m=324 n=18: 6.95 ms by the block kernel, 1.82 ms.)
+constexpr double kTileOverhead = 2e7;
+
+AmpChoice choose_glynn(int m, int n, int64_t n_out)
+{
+    const AmpChoice plain = choose_amp(m, n, n_out, PCV_ALGO_AUTO, 0);
+    if (n < 1 || n_out < 1 || n_out > INT32_MAX / 64 || plain.algo == kAlgoRouted) return plain;
+    const double steps = std::ldexp((double)n_out, n - 1);
+    const double tile = std::ldexp(1.25 * n * 32.0 * (double)((n_out + 31) / 32), n - 1);
+    if (steps * (6 * n - 2) < kTileOverhead || tile > steps * (6 * n - 2) || pcv::tile_split_workspace(m, n, n_out) < 0)
+        return plain;
+    if (n >= kRouteMinPhotons && m <= pcv::tile_max_modes()) return {kAlgoRouted, 0};
+    return {kAlgoTileSplit, 0};
+}
+
 // Workspace of PCV_ALGO_AUTO: what lets it take its first choice.  A smaller
 // one, down to the Glynn kernel's own need (often none), is accepted.
+int64_t glynn_workspace(const AmpChoice& c, int m, int n, int64_t n_out)
+{
+    if (c.algo == kAlgoRouted)
+        return (int64_t)align256(sizeof(pcv_batch_desc)) + pcv::batched_workspace_full(1, n_out);
+    if (c.algo == kAlgoTileSplit) return pcv::tile_split_workspace(m, n, n_out);
+    return amp_workspace(c, n_out);
+}
+
 int64_t auto_amp_workspace(int m, int n, int64_t n_out)
 {
-    const int64_t w = amp_workspace(choose_amp(m, n, n_out, PCV_ALGO_AUTO, 0), n_out);
+    const int64_t w = std::max(amp_workspace(choose_amp(m, n, n_out, PCV_ALGO_AUTO, 0), n_out),
+                               glynn_workspace(choose_glynn(m, n, n_out), m, n, n_out));
     return split_pays(m, n, n_out) ? std::max(w, pcv::split_workspace(m, n)) : w;
 }
 
@@ -405,6 +438,11 @@ int pcv_amplitudes_ex(const pcv_c64* U, int m, const uint8_t* input_occ,
         return e == cudaSuccess ? PCV_OK : cuda_fail(e, "split launch");
     }
     AmpChoice c = choose_amp(m, p.n, n_out, algo, param);
+    if (algo == PCV_ALGO_AUTO) {
+        const AmpChoice g = choose_glynn(m, p.n, n_out);
+        const int64_t w = glynn_workspace(g, m, p.n, n_out);
+        if (w == 0 || (workspace && workspace_bytes >= w && aligned(workspace, 256))) c = g;
+    }
     if ((rc = check_choice(c, p.n))) return rc;
     const int64_t need = amp_workspace(c, n_out);
     if (need > 0 && (!workspace || workspace_bytes < need))
@@ -422,9 +460,17 @@ int pcv_amplitudes_ex(const pcv_c64* U, int m, const uint8_t* input_occ,
         void* bws = (char*)workspace + align256(sizeof(pcv_batch_desc));
         pcv::stage_begin(pcv::kStagePlain, s);
         e = pcv::launch_store_desc(d, dd, s);
-        if (e == cudaSuccess) e = pcv::launch_glynn_batched(dd, 1, n_out, bws, sms, PCV_ALGO_AUTO, s);
+        if (e == cudaSuccess)
+            e = pcv::launch_glynn_batched(dd, 1, n_out, bws, workspace_bytes - (int64_t)align256(sizeof(pcv_batch_desc)), sms,
+                                          PCV_ALGO_AUTO, s);
         pcv::stage_end(pcv::kStagePlain, s);
         return e == cudaSuccess ? PCV_OK : cuda_fail(e, "routed launch");
+    }
+    if (c.algo == kAlgoTileSplit) {
+        pcv::stage_begin(pcv::kStagePlain, s);
+        cudaError_t e = pcv::launch_glynn_tile_split(make_desc(p, U, output_occ, n_out, amp, prob), workspace, s);
+        pcv::stage_end(pcv::kStagePlain, s);
+        return e == cudaSuccess ? PCV_OK : cuda_fail(e, "tile launch");
     }
     if (c.algo == PCV_ALGO_MULT) {
         const pcv_batch_desc d = make_desc(p, U, output_occ, n_out, amp, prob);
@@ -486,7 +532,7 @@ int pcv_amplitudes_multi(const pcv_c64* U, int B, int m, const uint8_t* input_oc
 int64_t pcv_amplitudes_batched_workspace(int n_circ, int64_t total_outputs)
 {
     if (n_circ < 0 || total_outputs < 0) return fail(PCV_EINVAL, "bad sizes");
-    return pcv::batched_workspace(n_circ, total_outputs);
+    return pcv::batched_workspace_full(n_circ, total_outputs);
 }
 
 int pcv_amplitudes_batched_ex(const pcv_batch_desc* descs, int n_circ, int64_t total_outputs, int algo,
@@ -509,7 +555,7 @@ int pcv_amplitudes_batched_ex(const pcv_batch_desc* descs, int n_circ, int64_t t
     if (e != cudaSuccess) return cuda_fail(e, "device query");
     cudaStream_t s = (cudaStream_t)stream;
     pcv::stage_begin(pcv::kStagePlain, s);
-    e = pcv::launch_glynn_batched(descs, n_circ, total_outputs, workspace, sms, algo, s);
+    e = pcv::launch_glynn_batched(descs, n_circ, total_outputs, workspace, workspace_bytes, sms, algo, s);
     pcv::stage_end(pcv::kStagePlain, s);
     return e == cudaSuccess ? PCV_OK : cuda_fail(e, "batched launch");
 }

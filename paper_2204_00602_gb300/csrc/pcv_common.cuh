@@ -123,17 +123,22 @@ cudaError_t launch_glynn_block(const Plan& p, const double2* U, const uint8_t* o
 int glynn_block_threads();
 
 // Shared-row-sum tile kernels (glynn_tile.cu)
-__host__ __device__ int tile_splits(int n);
 int tile_max_modes();
 cudaError_t launch_glynn_tile(const pcv_batch_desc& d, cudaStream_t s);
 cudaError_t launch_glynn_tile_multi(const pcv_batch_desc& d, int B, cudaStream_t s);
+// sign vectors of a tile split over several blocks: workspace (0: one part
+// per tile; -1: the modes do not fit), launch
+int64_t tile_split_workspace(int m, int n, int64_t n_out);
+cudaError_t launch_glynn_tile_split(const pcv_batch_desc& d, void* ws, cudaStream_t s);
+// the batched launch: least workspace, and with room for split sequences
 int64_t batched_workspace(int n_circ, int64_t total_outputs);
+int64_t batched_workspace_full(int n_circ, int64_t total_outputs);
 // copies a descriptor (passed by value) into device memory
 cudaError_t launch_store_desc(const pcv_batch_desc& d, pcv_batch_desc* out, cudaStream_t s);
 // route: PCV_ALGO_AUTO (per output, by FP64 instruction count), PCV_ALGO_TILE
 // or PCV_ALGO_MULT (every output to that kernel)
 cudaError_t launch_glynn_batched(const pcv_batch_desc* descs, int n_circ, int64_t total_outputs, void* ws,
-                                 int sms, int route, cudaStream_t s);
+                                 int64_t ws_bytes, int sms, int route, cudaStream_t s);
 
 // Glynn's sum with multiplicities (glynn_mult.cu).  side: 0 = fewer terms,
 // 1 = sign vectors on the output modes, 2 = on the input modes.

@@ -39,18 +39,20 @@ def index_range(N: int, rank: int, world: int) -> tuple[int, int]:
     return N * rank // world, N * (rank + 1) // world
 
 
-def _tile_splits(n: int) -> int:
-    return 1 if n <= 10 else 2 if n <= 13 else 4 if n <= 16 else 8
+def tile_cost(n: int) -> float:
+    """The tile kernel's time per output in FP64 instructions: its n - 1
+    integer-pipe products take 1.25 of them each, per sign vector."""
+    return 2.0 ** (n - 1) * (1.25 * (n - 1) + 1)
 
 
 def output_cost(m: int, n: int, input_occ, outputs: np.ndarray) -> np.ndarray:
-    """FP64 pipe instructions per output under the batched routing model:
+    """Time per output in FP64 instructions under the batched routing model:
     min(tile kernel, Glynn's sum with multiplicities on either side)."""
     t = np.asarray(input_occ, dtype=np.int64)
     tin = t[t > 0]
     d_in = len(tin)
     s = np.asarray(outputs, dtype=np.int64).reshape(-1, m)
-    tile = 2.0 ** (n - 1) * (4 * n - 2 + 2 * m / (256 // _tile_splits(n)))
+    tile = tile_cost(n)
 
     def terms(mu):                       # rows: multiplicities (zeros ignored)
         prod = np.prod(mu + 1, axis=-1).astype(np.float64)

@@ -47,18 +47,15 @@ def _events():
     return torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
 
 
-def _tile_splits(n: int) -> int:
-    return 1 if n <= 10 else 2 if n <= 13 else 4 if n <= 16 else 8
-
-
 def routed_fp64_instructions(m: int, n: int, outs: np.ndarray):
-    """FP64 pipe instructions under the batched launch's cost model
-    (single-photon input): the tile kernel's 2^{n-1} (4n - 2 + 2m/TILE) per
-    output, a tile block costing as much as TILE outputs however many are live,
-    or, for Glynn's sum with multiplicities, terms x (2q + 4n - 1) on the
-    cheaper side.  Returns (tile-only instructions, routed instructions,
-    outputs routed to the multiplicity kernel)."""
-    tile = 2.0 ** (n - 1) * (4 * n - 2 + 2 * m / (256 // _tile_splits(n)))
+    """Time in FP64 instructions under the batched launch's cost model
+    (single-photon input): the tile kernel's 2^{n-1} (1.25 (n - 1) + 1) per
+    output (its products run on the integer pipe), a warp costing as much as 32
+    outputs however many are live, or, for Glynn's sum with multiplicities,
+    terms x (2q + 4n - 1) on the cheaper side.  Returns (tile-only cost, routed
+    cost, outputs routed to the multiplicity kernel)."""
+    from .sharding import tile_cost
+    tile = tile_cost(n)
     s = outs.astype(np.int64)
     d_out = (s > 0).sum(axis=1)
     prod = np.prod(s + 1, axis=1).astype(np.float64)
@@ -69,10 +66,10 @@ def routed_fp64_instructions(m: int, n: int, outs: np.ndarray):
     cost_in = 2.0 ** (n - 1) * (2 * d_out + 4 * n - 1)  # sign side: the n input photons
     mult = np.minimum(cost_out, cost_in)
     to_mult = mult < tile
-    # a last, partly filled tile goes to the multiplicity kernel when its
-    # outputs cost less there than the whole tile block (as the routing kernel does)
+    # the outputs of a last, partly filled warp go to the multiplicity kernel when
+    # they cost less there than the whole warp (as the routing kernel does)
     tile_idx = np.flatnonzero(~to_mult)
-    tsz = 256 // _tile_splits(n)
+    tsz = 32
     r = len(tile_idx) % tsz
     if r and mult[tile_idx[-r:]].sum() < tile * tsz:
         to_mult[tile_idx[-r:]] = True
