@@ -1,21 +1,32 @@
 // BF16 GEMM on the 5th-generation tensor cores (tcgen05 + TMEM) with TMA
-// staging, for the surrogate MLP.  C[M x N] = A[M x K] . B[N x K]^T, A and B
-// bf16 row-major (K contiguous), FP32 accumulation in tensor memory, the same
-// fused epilogues as the mma.sync kernel in mlp.cu (plain, bias, bias+GELU,
-// GELU derivative).  No counterpart in the paper.
+// staging, for the surrogate MLP.  C[M x N] = A[M x K] . B[N x K]^T, FP32
+// accumulation in tensor memory, the same fused epilogues as the mma.sync
+// kernel in mlp.cu (plain, bias, bias+GELU, GELU derivative).  Either operand
+// is row-major with K contiguous, or given transposed (row-major with M or N
+// contiguous), so the weight gradient dY^T X and the input gradient dY W need
+// no transposed copies (12 transposes, 77 us of a training step of 4096 rows).
+// No counterpart in the paper.
 //
-// One CTA computes a 128 x 128 tile with 128 threads:
+// One CTA computes a 128 x BN tile with 128 threads:
 //   thread 0    TMA producer: 64-wide K blocks of A and B (128B swizzle) into a
-//               3-stage shared-memory ring, completion tracked by mbarriers;
-//   thread 32   MMA issuer: tcgen05.mma.cta_group::1.kind::f16 (M=128, N=128,
-//               K=16) from shared-memory descriptors into a 128-column TMEM
+//               ring of shared-memory stages, completion tracked by mbarriers;
+//   thread 32   MMA issuer: tcgen05.mma.cta_group::1.kind::f16 (M=128, N=BN,
+//               K=16) from shared-memory descriptors into a BN-column TMEM
 //               accumulator; tcgen05.commit frees each stage and finally
 //               signals the epilogue;
 //   all warps   epilogue: warp w reads TMEM lanes 32w..32w+31 (rows) with
 //               tcgen05.ld.32x32b, turns each 32 x 32 block around in shared
-//               memory and stores it row-contiguously.
-// Three stages (97 KB of shared memory) let two CTAs share an SM, so one
-// CTA's epilogue overlaps the other's main loop.
+//               memory and moves it four columns per lane (16-byte loads of
+//               `pre`, 16- and 8-byte stores), eight rows in flight.
+// What bounds it at the surrogate's sizes is latency, not the tensor cores: a
+// tile has 16 to 64 K blocks and an epilogue of erf and exp, and there are at
+// most about two tiles per SM.  So BN is the largest of 128, 64, 32 that still
+// gives every SM a tile (a weight gradient of 1024 x 1024 is 64 tiles of 128
+// columns), two CTAs share an SM with half the ring each when there are more
+// tiles than SMs, and otherwise one CTA has the whole ring (about 190 KB in
+// flight).  Training step of 4096 rows: GEMMs 400 us before.
+// A transposed operand's stage holds 64-column blocks of 64 K rows (128 bytes
+// each), 8 KB apart: the MN-major 128-byte-swizzle layout.
 // Out-of-range rows, columns and K are zero-filled by TMA and skipped on
 // store.  Every mbarrier wait gives up after a bounded number of polls and
 // raises an error flag the host reads; TMEM is always released.
@@ -24,6 +35,7 @@
 #include <cuda_bf16.h>
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <cstdio>
 #include <mutex>
 
@@ -34,15 +46,18 @@ namespace pcv {
 
 namespace {
 
-constexpr int TC_BM = 128, TC_BN = 128, TC_BK = 64, TC_STAGES = 3;   // 97 KB: two CTAs per SM
+constexpr int TC_BM = 128, TC_BK = 64;
+constexpr int TC_MAX_STAGES = 8;
+constexpr int kTcSms = 152;
 constexpr int TC_THREADS = 128;
-constexpr uint32_t TC_STAGE_BYTES = (TC_BM + TC_BN) * TC_BK * 2;     // 32 KB per stage
-constexpr uint32_t TC_TMEM_COLS = 128;
-constexpr long long TC_MAX_POLLS = 1ll << 22;                        // default bound of one mbarrier wait
+constexpr uint32_t TC_RING_ONE = 192 * 1024, TC_RING_TWO = 96 * 1024;   // ring bytes with one, two CTAs per SM
+constexpr long long TC_MAX_POLLS = 1ll << 22;                           // default bound of one mbarrier wait
 
 struct TcArgs {
     int M, N, K;
-    int mode;
+    int at, bt;                       // operand given transposed (M or N contiguous)
+    int stages;
+    int vec;                          // bias, outputs and pre allow 4-column accesses
     const float* bias;
     float* outf; int ldo;
     __nv_bfloat16* outb; int ldob;
@@ -63,22 +78,56 @@ __device__ __forceinline__ float gelu_grad_tc(float x)
     return 0.5f * (1.0f + erff(x * 0.70710678118654752f)) + x * 0.39894228040143268f * expf(-0.5f * x * x);
 }
 
+// Descriptor of an MN-major tile (128-byte swizzle): rows of one K, 64 MN
+// values each; 8 K rows 1024 B apart, 64-value MN blocks 8 KB apart.
+__device__ __forceinline__ uint64_t sdesc_mn_sw128(const void* p)
+{
+    uint64_t d = sdesc_sw128(p) & ~((uint64_t)0x3FFF << 16);
+    return d | ((uint64_t)(8192 >> 4) << 16);
+}
+
+// One element of the epilogue.
+template <int MODE>
+__device__ __forceinline__ void epilogue_one(const TcArgs& a, float x, int row, int col)
+{
+    if constexpr (MODE == 0) a.outf[(size_t)row * a.ldo + col] = x;
+    if constexpr (MODE == 2) a.outf[(size_t)row * a.ldo + col] = x + a.bias[col];
+    if constexpr (MODE == 1) {
+        x += a.bias[col];
+        if (a.outf) a.outf[(size_t)row * a.ldo + col] = x;
+        a.outb[(size_t)row * a.ldob + col] = __float2bfloat16_rn(gelu_tc(x));
+    }
+    if constexpr (MODE == 3)
+        a.outb[(size_t)row * a.ldob + col] = __float2bfloat16_rn(x * gelu_grad_tc(a.pre[(size_t)row * a.ldp + col]));
+}
+
+__device__ __forceinline__ uint2 pack_bf16(float4 x)
+{
+    const __nv_bfloat162 lo = __floats2bfloat162_rn(x.x, x.y), hi = __floats2bfloat162_rn(x.z, x.w);
+    uint2 r;
+    r.x = *reinterpret_cast<const uint32_t*>(&lo);
+    r.y = *reinterpret_cast<const uint32_t*>(&hi);
+    return r;
+}
+
+template <int BN, int MODE>
 __global__ void __launch_bounds__(TC_THREADS, 2)
 gemm_bf16_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, const TcArgs a)
 {
+    constexpr uint32_t kABytes = TC_BM * TC_BK * 2, kBBytes = BN * TC_BK * 2, kStage = kABytes + kBBytes;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
-    // 1024-byte aligned ring of stages: [A 128x64 | B 128x64] bf16 each
+    // 1024-byte aligned ring of stages: [A 128x64 | B BNx64] bf16 each
     unsigned char* ring = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    __shared__ __align__(8) uint64_t full_bar[TC_STAGES], empty_bar[TC_STAGES], done_bar, mma_done;
+    __shared__ __align__(8) uint64_t full_bar[TC_MAX_STAGES], empty_bar[TC_MAX_STAGES], done_bar, mma_done;
     __shared__ uint32_t tmem_base;
     __shared__ int s_fail;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int m0 = blockIdx.y * TC_BM, n0 = blockIdx.x * TC_BN;
-    const int nk = (a.K + TC_BK - 1) / TC_BK;
+    const int m0 = blockIdx.y * TC_BM, n0 = blockIdx.x * BN;
+    const int nk = (a.K + TC_BK - 1) / TC_BK, stages = a.stages;
 
     if (tid == 0) {
-        for (int s = 0; s < TC_STAGES; ++s) {
+        for (int s = 0; s < stages; ++s) {
             mbar_init(&full_bar[s], 1);
             mbar_init(&empty_bar[s], 1);
         }
@@ -89,7 +138,7 @@ gemm_bf16_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
         tcx::prefetch_tmap(&mapA);
         tcx::prefetch_tmap(&mapB);
     }
-    if (warp == 1) tcx::tmem_alloc(&tmem_base, TC_TMEM_COLS);
+    if (warp == 1) tcx::tmem_alloc(&tmem_base, BN);
     tcx::fence_before_sync();
     __syncthreads();
     tcx::fence_after_sync();
@@ -99,35 +148,51 @@ gemm_bf16_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
     if (tid == 0) {
         // ---------------- TMA producer
         int issued = 0;
-        for (int kt = 0; kt < nk && !s_fail; ++kt) {
-            const int s = kt % TC_STAGES;
-            if (kt >= TC_STAGES && !mbar_wait(&empty_bar[s], ((kt / TC_STAGES) - 1) & 1, polls)) { s_fail = 1; break; }
-            unsigned char* sa = ring + s * TC_STAGE_BYTES;
-            unsigned char* sb = sa + TC_BM * TC_BK * 2;
-            mbar_expect_tx(&full_bar[s], TC_STAGE_BYTES);
-            tma_load_2d(sa, &mapA, &full_bar[s], kt * TC_BK, m0);
-            tma_load_2d(sb, &mapB, &full_bar[s], kt * TC_BK, n0);
+        for (int kt = 0, st = 0, ph = 1; kt < nk && !s_fail; ++kt) {
+            if (kt >= stages && !mbar_wait(&empty_bar[st], ph, polls)) { s_fail = 1; break; }
+            unsigned char* sa = ring + st * kStage;
+            unsigned char* sb = sa + kABytes;
+            mbar_expect_tx(&full_bar[st], kStage);
+            if (a.at) {
+                tma_load_2d(sa, &mapA, &full_bar[st], m0, kt * TC_BK);
+                tma_load_2d(sa + 8192, &mapA, &full_bar[st], m0 + 64, kt * TC_BK);
+            } else {
+                tma_load_2d(sa, &mapA, &full_bar[st], kt * TC_BK, m0);
+            }
+            if (a.bt) {
+                for (int j = 0; j < BN; j += 64) tma_load_2d(sb + j * 128, &mapB, &full_bar[st], n0 + j, kt * TC_BK);
+            } else {
+                tma_load_2d(sb, &mapB, &full_bar[st], kt * TC_BK, n0);
+            }
             ++issued;
+            if (++st == stages) {
+                st = 0;
+                ph ^= 1;
+            }
         }
         // the loads issued land in this CTA's shared memory before it may exit
-        if (!tcx::wait_issued(full_bar, TC_STAGES, (uint32_t)issued) && !s_fail) s_fail = 4;
+        if (!tcx::wait_issued(full_bar, stages, (uint32_t)issued) && !s_fail) s_fail = 4;
     } else if (tid == 32) {
         // ---------------- MMA issuer
-        const uint32_t idesc = tcx::idesc_bf16(TC_BM, TC_BN);
+        const uint32_t idesc = tcx::idesc_bf16(TC_BM, BN) | (a.at ? 1u << 15 : 0u) | (a.bt ? 1u << 16 : 0u);
+        // 16 of K further: 32 B along a K-major row, 16 rows of 128 B of an MN-major tile (16-byte units)
+        const uint32_t astep = a.at ? 128 : 2, bstep = a.bt ? 128 : 2;
         bool all = true;
-        for (int kt = 0; kt < nk; ++kt) {
-            const int s = kt % TC_STAGES;
-            if (!mbar_wait(&full_bar[s], (kt / TC_STAGES) & 1, polls)) { s_fail = 2; all = false; break; }
+        for (int kt = 0, st = 0, ph = 0; kt < nk; ++kt) {
+            if (!mbar_wait(&full_bar[st], ph, polls)) { s_fail = 2; all = false; break; }
             tcx::fence_after_sync();
-            const unsigned char* sa = ring + s * TC_STAGE_BYTES;
-            const unsigned char* sb = sa + TC_BM * TC_BK * 2;
+            const unsigned char* sa = ring + st * kStage;
+            const unsigned char* sb = sa + kABytes;
+            const uint64_t ad = a.at ? sdesc_mn_sw128(sa) : sdesc_sw128(sa);
+            const uint64_t bd = a.bt ? sdesc_mn_sw128(sb) : sdesc_sw128(sb);
 #pragma unroll
-            for (int kk = 0; kk < TC_BK / 16; ++kk) {
-                const uint64_t ad = sdesc_sw128(sa + kk * 32);      // 16 bf16 = 32 B along K
-                const uint64_t bd = sdesc_sw128(sb + kk * 32);
-                tcx::mma_bf16(tmem, ad, bd, idesc, (kt > 0 || kk > 0) ? 1u : 0u);
+            for (int kk = 0; kk < TC_BK / 16; ++kk)
+                tcx::mma_bf16(tmem, ad + kk * astep, bd + kk * bstep, idesc, (kt > 0 || kk > 0) ? 1u : 0u);
+            tcx::mma_commit(&empty_bar[st]);
+            if (++st == stages) {
+                st = 0;
+                ph ^= 1;
             }
-            tcx::mma_commit(&empty_bar[s]);
         }
         // a complete accumulation goes to the epilogue; in every case the MMAs
         // issued finish before the tensor memory is released
@@ -143,10 +208,21 @@ gemm_bf16_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
     __syncwarp();
     if (ok) {
         // Each warp moves its 32 rows x 32 columns through a padded shared tile
-        // (the drained stage ring) so that global stores are row-contiguous.
-        float* stage = reinterpret_cast<float*>(ring) + warp * (32 * 33);
+        // (the drained stage ring): a row per lane in, four columns per lane out
+        // (8 lanes to a row).
+        constexpr int kRow = 36;
+        float* stage = reinterpret_cast<float*>(ring) + warp * (32 * kRow);
 #pragma unroll 1
-        for (int c0 = 0; c0 < TC_BN; c0 += 32) {
+        for (int c0 = 0; c0 < BN; c0 += 32) {
+            const int col = n0 + c0 + (lane & 7) * 4, row0 = m0 + warp * 32 + (lane >> 3);
+            const bool vec = a.vec && col + 4 <= a.N;
+            float4 pre[8];
+            if constexpr (MODE == 3) {
+#pragma unroll
+                for (int it = 0; it < 8; ++it)
+                    if (vec && row0 + 4 * it < a.M)
+                        pre[it] = *reinterpret_cast<const float4*>(a.pre + (size_t)(row0 + 4 * it) * a.ldp + col);
+            }
             uint32_t r[32];
             const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0;
             asm volatile(
@@ -160,42 +236,53 @@ gemm_bf16_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                 : "r"(taddr));
             asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
 #pragma unroll
-            for (int j = 0; j < 32; ++j) stage[lane * 33 + j] = __uint_as_float(r[j]);   // row = lane
+            for (int j = 0; j < 32; j += 4)                                              // row = lane
+                *reinterpret_cast<uint4*>(stage + lane * kRow + j) = make_uint4(r[j], r[j + 1], r[j + 2], r[j + 3]);
             __syncwarp();
-            const int col = n0 + c0 + lane;
-            if (col < a.N) {
-#pragma unroll 4
-                for (int rr = 0; rr < 32; ++rr) {
-                    const int row = m0 + warp * 32 + rr;
-                    if (row >= a.M) break;
-                    float x = stage[rr * 33 + lane];
-                    switch (a.mode) {
-                    case 0: a.outf[(size_t)row * a.ldo + col] = x; break;
-                    case 2: a.outf[(size_t)row * a.ldo + col] = x + a.bias[col]; break;
-                    case 1:
-                        x += a.bias[col];
-                        if (a.outf) a.outf[(size_t)row * a.ldo + col] = x;
-                        a.outb[(size_t)row * a.ldob + col] = __float2bfloat16_rn(gelu_tc(x));
-                        break;
-                    case 3:
-                        a.outb[(size_t)row * a.ldob + col] =
-                            __float2bfloat16_rn(x * gelu_grad_tc(a.pre[(size_t)row * a.ldp + col]));
-                        break;
-                    }
+            float4 bias = make_float4(0.f, 0.f, 0.f, 0.f);
+            if constexpr (MODE == 1 || MODE == 2)
+                if (vec) bias = *reinterpret_cast<const float4*>(a.bias + col);
+#pragma unroll
+            for (int it = 0; it < 8; ++it) {
+                const int row = row0 + 4 * it;
+                if (row >= a.M) continue;
+                float4 x = *reinterpret_cast<const float4*>(stage + ((lane >> 3) + 4 * it) * kRow + (lane & 7) * 4);
+                if (!vec) {
+                    const float v[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        if (col + e < a.N) epilogue_one<MODE>(a, v[e], row, col + e);
+                    continue;
                 }
+                if constexpr (MODE == 1 || MODE == 2) {
+                    x.x += bias.x;
+                    x.y += bias.y;
+                    x.z += bias.z;
+                    x.w += bias.w;
+                }
+                if constexpr (MODE == 3) {
+                    x.x *= gelu_grad_tc(pre[it].x);
+                    x.y *= gelu_grad_tc(pre[it].y);
+                    x.z *= gelu_grad_tc(pre[it].z);
+                    x.w *= gelu_grad_tc(pre[it].w);
+                } else if (MODE != 1 || a.outf) {
+                    *reinterpret_cast<float4*>(a.outf + (size_t)row * a.ldo + col) = x;
+                }
+                if constexpr (MODE == 1) x = make_float4(gelu_tc(x.x), gelu_tc(x.y), gelu_tc(x.z), gelu_tc(x.w));
+                if constexpr (MODE == 1 || MODE == 3)
+                    *reinterpret_cast<uint2*>(a.outb + (size_t)row * a.ldob + col) = pack_bf16(x);
             }
             __syncwarp();
         }
     }
     tcx::fence_before_sync();
     __syncthreads();
-    if (warp == 1) tcx::tmem_dealloc(tmem, TC_TMEM_COLS);
+    if (warp == 1) tcx::tmem_dealloc(tmem, BN);
     if (tid == 0 && s_fail && a.error) atomicExch(a.error, s_fail);
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
 std::once_flag g_encode_once;
-bool g_attr_done[64] = {};
 
 cudaError_t get_encode()
 {
@@ -209,12 +296,13 @@ cudaError_t get_encode()
     return g_encode ? cudaSuccess : cudaErrorNotSupported;
 }
 
-// 2-D bf16 tensor map over rows x K (row stride ld elements), box 64 x 128, 128B swizzle.
-cudaError_t make_map(CUtensorMap* map, const void* base, int rows, int K, int ld)
+// 2-D bf16 tensor map over `outer` rows of `inner` values (row stride ld), box
+// 64 x box_rows, 128B swizzle.
+cudaError_t make_map(CUtensorMap* map, const void* base, int inner, int outer, int ld, int box_rows)
 {
-    const cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)rows};
+    const cuuint64_t dims[2] = {(cuuint64_t)inner, (cuuint64_t)outer};
     const cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
-    const cuuint32_t box[2] = {(cuuint32_t)TC_BK, (cuuint32_t)TC_BM};
+    const cuuint32_t box[2] = {(cuuint32_t)TC_BK, (cuuint32_t)box_rows};
     const cuuint32_t estr[2] = {1, 1};
     const CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box,
                                 estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
@@ -222,49 +310,81 @@ cudaError_t make_map(CUtensorMap* map, const void* base, int rows, int K, int ld
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-}  // namespace
-
-size_t gemm_tc_smem() { return (size_t)TC_STAGES * TC_STAGE_BYTES + 1024; }
-
-cudaError_t launch_gemm_bf16_tc(const void* A, int lda, const void* B, int ldb, int M, int N, int K, int mode,
-                                const float* bias, float* outf, int ldo, void* outb, int ldob, const float* pre,
-                                int ldp, int* error, cudaStream_t s)
+template <int BN, int MODE>
+cudaError_t launch_tile(const CUtensorMap& ma, const CUtensorMap& mb, const TcArgs& a, size_t smem, cudaStream_t s)
 {
-    cudaError_t e = get_encode();
+    cudaError_t e = cudaFuncSetAttribute(gemm_bf16_tc_kernel<BN, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem);
     if (e != cudaSuccess) return e;
-    int dev = 0;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    if (dev >= 0 && dev < 64 && !g_attr_done[dev]) {
-        e = cudaFuncSetAttribute(gemm_bf16_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_tc_smem());
-        if (e != cudaSuccess) return e;
-        g_attr_done[dev] = true;
-    }
-    CUtensorMap ma, mb;
-    if ((e = make_map(&ma, A, M, K, lda)) != cudaSuccess) return e;
-    if ((e = make_map(&mb, B, N, K, ldb)) != cudaSuccess) return e;
-    TcArgs a;
-    a.M = M; a.N = N; a.K = K; a.mode = mode;
-    a.bias = bias; a.outf = outf; a.ldo = ldo; a.outb = (__nv_bfloat16*)outb; a.ldob = ldob; a.pre = pre; a.ldp = ldp;
-    a.error = error;
-    a.max_polls = wait_limit(TC_MAX_POLLS);
-    dim3 grid((N + TC_BN - 1) / TC_BN, (M + TC_BM - 1) / TC_BM);
-    gemm_bf16_tc_kernel<<<grid, TC_THREADS, gemm_tc_smem(), s>>>(ma, mb, a);
+    const dim3 grid((a.N + BN - 1) / BN, (a.M + TC_BM - 1) / TC_BM);
+    gemm_bf16_tc_kernel<BN, MODE><<<grid, TC_THREADS, smem, s>>>(ma, mb, a);
     note_launches(1);
     return cudaGetLastError();
 }
 
+template <int BN>
+cudaError_t launch_width(const CUtensorMap& ma, const CUtensorMap& mb, int mode, TcArgs a, int64_t tiles, cudaStream_t s)
+{
+    constexpr uint32_t stage = (TC_BM + BN) * TC_BK * 2;
+    const uint32_t ring = tiles > kTcSms ? TC_RING_TWO : TC_RING_ONE;
+    const int nk = (a.K + TC_BK - 1) / TC_BK;
+    a.stages = std::min<int>(std::min<int>(TC_MAX_STAGES, ring / stage), std::max(nk, 2));
+    const size_t smem = std::max<size_t>((size_t)a.stages * stage, 4 * 32 * 36 * sizeof(float)) + 1024;
+    switch (mode) {
+    case 0: return launch_tile<BN, 0>(ma, mb, a, smem, s);
+    case 1: return launch_tile<BN, 1>(ma, mb, a, smem, s);
+    case 2: return launch_tile<BN, 2>(ma, mb, a, smem, s);
+    default: return launch_tile<BN, 3>(ma, mb, a, smem, s);
+    }
+}
+
+bool aligned_to(const void* p, size_t n) { return (uintptr_t)p % n == 0; }
+
+}  // namespace
+
+cudaError_t launch_gemm_bf16_tc(const void* A, int lda, int at, const void* B, int ldb, int bt, int M, int N, int K,
+                                int mode, const float* bias, float* outf, int ldo, void* outb, int ldob,
+                                const float* pre, int ldp, int* error, cudaStream_t s)
+{
+    cudaError_t e = get_encode();
+    if (e != cudaSuccess) return e;
+    // the widest tile that still gives every SM one (a 32-wide tile cannot be
+    // transposed: its stage would hold half a 64-column block)
+    const int64_t rows = (M + TC_BM - 1) / TC_BM;
+    int bn = 128;
+    while (bn > (bt ? 64 : 32) && rows * ((N + bn - 1) / bn) < kTcSms) bn >>= 1;
+    CUtensorMap ma, mb;
+    e = at ? make_map(&ma, A, M, K, lda, TC_BK) : make_map(&ma, A, K, M, lda, TC_BM);
+    if (e != cudaSuccess) return e;
+    e = bt ? make_map(&mb, B, N, K, ldb, TC_BK) : make_map(&mb, B, K, N, ldb, bn);
+    if (e != cudaSuccess) return e;
+    TcArgs a;
+    a.M = M; a.N = N; a.K = K; a.at = at; a.bt = bt;
+    a.bias = bias; a.outf = outf; a.ldo = ldo; a.outb = (__nv_bfloat16*)outb; a.ldob = ldob; a.pre = pre; a.ldp = ldp;
+    a.error = error;
+    a.max_polls = wait_limit(TC_MAX_POLLS);
+    a.vec = (!outf || (ldo % 4 == 0 && aligned_to(outf, 16))) && (!outb || (ldob % 4 == 0 && aligned_to(outb, 8))) &&
+            (mode != 3 || (ldp % 4 == 0 && aligned_to(pre, 16))) && (mode == 0 || mode == 3 || aligned_to(bias, 16));
+    const int64_t tiles = rows * ((N + bn - 1) / bn);
+    if (bn == 128) return launch_width<128>(ma, mb, mode, a, tiles, s);
+    if (bn == 64) return launch_width<64>(ma, mb, mode, a, tiles, s);
+    return launch_width<32>(ma, mb, mode, a, tiles, s);
+}
+
 }  // namespace pcv
 
-extern "C" int pcv_gemm_bf16_tc(const void* A, int lda, const void* B, int ldb, int M, int N, int K, int mode,
-                                const float* bias, float* outf, int ldo, void* outb, int ldob, const float* pre,
-                                int ldp, int* error, void* stream)
+// Checks and launch of both entry points.
+static int gemm_tc(const void* A, int lda, int at, const void* B, int ldb, int bt, int M, int N, int K, int mode,
+                   const float* bias, float* outf, int ldo, void* outb, int ldob, const float* pre, int ldp, int* error,
+                   void* stream)
 {
     if (!A || !B || M < 1 || N < 1 || K < 16 || K % 8 != 0) {
         pcv::set_error("gemm_bf16_tc: sizes (K must be a positive multiple of 8)");
         return PCV_EINVAL;
     }
-    if (lda % 8 || ldb % 8 || lda < K || ldb < K || ((uintptr_t)A % 16) || ((uintptr_t)B % 16)) {
-        pcv::set_error("gemm_bf16_tc: leading dimensions must be multiples of 8 >= K and operands 16-byte aligned");
+    if (lda % 8 || ldb % 8 || lda < (at ? M : K) || ldb < (bt ? N : K) || ((uintptr_t)A % 16) || ((uintptr_t)B % 16)) {
+        pcv::set_error("gemm_bf16_tc: leading dimensions must be multiples of 8 >= K (>= M, N of a transposed operand) "
+                       "and operands 16-byte aligned");
         return PCV_EINVAL;
     }
     if (mode < 0 || mode > 3 || ((mode == 0 || mode == 2) && !outf) || ((mode == 1 || mode == 3) && !outb) ||
@@ -272,8 +392,8 @@ extern "C" int pcv_gemm_bf16_tc(const void* A, int lda, const void* B, int ldb, 
         pcv::set_error("gemm_bf16_tc: epilogue arguments");
         return PCV_EINVAL;
     }
-    cudaError_t e = pcv::launch_gemm_bf16_tc(A, lda, B, ldb, M, N, K, mode, bias, outf, ldo, outb, ldob, pre, ldp, error,
-                                             (cudaStream_t)stream);
+    cudaError_t e = pcv::launch_gemm_bf16_tc(A, lda, at, B, ldb, bt, M, N, K, mode, bias, outf, ldo, outb, ldob, pre, ldp,
+                                             error, (cudaStream_t)stream);
     if (e != cudaSuccess) {
         char buf[200];
         snprintf(buf, sizeof buf, "gemm_bf16_tc: %s", cudaGetErrorString(e));
@@ -281,4 +401,19 @@ extern "C" int pcv_gemm_bf16_tc(const void* A, int lda, const void* B, int ldb, 
         return PCV_ECUDA;
     }
     return PCV_OK;
+}
+
+extern "C" int pcv_gemm_bf16_tc(const void* A, int lda, const void* B, int ldb, int M, int N, int K, int mode,
+                                const float* bias, float* outf, int ldo, void* outb, int ldob, const float* pre,
+                                int ldp, int* error, void* stream)
+{
+    return gemm_tc(A, lda, 0, B, ldb, 0, M, N, K, mode, bias, outf, ldo, outb, ldob, pre, ldp, error, stream);
+}
+
+extern "C" int pcv_gemm_bf16_tc_t(const void* A, int lda, int a_transposed, const void* B, int ldb, int b_transposed,
+                                  int M, int N, int K, int mode, const float* bias, float* outf, int ldo, void* outb,
+                                  int ldob, const float* pre, int ldp, int* error, void* stream)
+{
+    return gemm_tc(A, lda, a_transposed != 0, B, ldb, b_transposed != 0, M, N, K, mode, bias, outf, ldo, outb, ldob, pre,
+                   ldp, error, stream);
 }

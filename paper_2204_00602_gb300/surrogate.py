@@ -71,7 +71,9 @@ class MLP:
         self.mb = [torch.zeros_like(b) for b in self.b]
         self.vb = [torch.zeros_like(b) for b in self.b]
         self.Wb = [_bf16(w.shape, self.dev) for w in self.W]                       # [out, in]
-        self.WTb = [_bf16((w.shape[1], w.shape[0]), self.dev) for w in self.W]     # [in, out]
+        # the tcgen05 GEMM reads transposed operands in place (widths a multiple of 8); else copies [in, out]
+        self.in_place = tensor_core == "tcgen05" and all(d % 8 == 0 for d in self.dims)
+        self.WTb = [] if self.in_place else [_bf16((w.shape[1], w.shape[0]), self.dev) for w in self.W]
         self.lr, self.betas, self.eps = lr, betas, eps
         self.step_count = 0
         self._mse_ws = torch.empty(abi.pcv_mse_workspace(), dtype=torch.uint8, device=self.dev)
@@ -86,6 +88,10 @@ class MLP:
     def refresh_bf16(self):
         for l in range(self.L):
             abi.pcv_f32_to_bf16(self.W[l], self.W[l].numel(), self.Wb[l], self.stream)
+            self._transpose_weights(l)
+
+    def _transpose_weights(self, l):
+        if not self.in_place:
             o, i = self.W[l].shape
             abi.pcv_transpose_bf16(self.Wb[l], o, i, i, self.WTb[l], o, self.stream)
 
@@ -103,6 +109,11 @@ class MLP:
                                  self.stream)
         else:
             abi.pcv_gemm_bf16(A, lda, B, ldb, M, N, K, mode, bias, outf, ldo, outb, ldob, pre, ldp, self.stream)
+
+    def gemm_nt(self, A, lda, at, B, ldb, bt, M, N, K, mode, outf, ldo, outb, ldob, pre, ldp):
+        """The same with operands read transposed in place (tcgen05 only)."""
+        abi.pcv_gemm_bf16_tc_t(A, lda, at, B, ldb, bt, M, N, K, mode, None, outf, ldo, outb, ldob, pre, ldp, self.error,
+                               self.stream)
 
     def check(self):
         """Raise if a tcgen05 pipeline wait gave up since the last check (host sync)."""
@@ -150,22 +161,31 @@ class MLP:
         for l in reversed(range(self.L)):
             o, i = self.W[l].shape
             if want_param_grad:
-                dYT = self._buf(f"dYT{l}", (o, B), torch.bfloat16)
-                XT = self._buf(f"XT{l}", (i, B), torch.bfloat16)
-                abi.pcv_transpose_bf16(dY, B, o, o, dYT, B, self.stream)
-                abi.pcv_transpose_bf16(self.acts[l], B, i, i, XT, B, self.stream)
                 gW = self._buf(f"gW{l}", (o, i), torch.float32)
-                self.gemm(dYT, B, XT, B, o, i, B, 0, None, gW, i, None, 0, None, 0)
+                if self.in_place:
+                    self.gemm_nt(dY, o, 1, self.acts[l], i, 1, o, i, B, 0, gW, i, None, 0, None, 0)
+                else:
+                    dYT = self._buf(f"dYT{l}", (o, B), torch.bfloat16)
+                    XT = self._buf(f"XT{l}", (i, B), torch.bfloat16)
+                    abi.pcv_transpose_bf16(dY, B, o, o, dYT, B, self.stream)
+                    abi.pcv_transpose_bf16(self.acts[l], B, i, i, XT, B, self.stream)
+                    self.gemm(dYT, B, XT, B, o, i, B, 0, None, gW, i, None, 0, None, 0)
                 gb = self._buf(f"gb{l}", (o,), torch.float32)
                 abi.pcv_colsum_bf16(dY, B, o, o, gb, self.stream)
                 self.gW[l], self.gb[l] = gW, gb
             if l > 0:
                 dprev = self._buf(f"dY{l - 1}", (B, i), torch.bfloat16)
-                self.gemm(dY, o, self.WTb[l], o, B, i, o, 3, None, None, 0, dprev, i, self.pres[l - 1], i)
+                if self.in_place:
+                    self.gemm_nt(dY, o, 0, self.Wb[l], i, 1, B, i, o, 3, None, 0, dprev, i, self.pres[l - 1], i)
+                else:
+                    self.gemm(dY, o, self.WTb[l], o, B, i, o, 3, None, None, 0, dprev, i, self.pres[l - 1], i)
                 dY = dprev
             elif want_input_grad:
                 dX0 = self._buf("dX0", (B, i), torch.float32)
-                self.gemm(dY, o, self.WTb[0], o, B, i, o, 0, None, dX0, i, None, 0, None, 0)
+                if self.in_place:
+                    self.gemm_nt(dY, o, 0, self.Wb[0], i, 1, B, i, o, 0, dX0, i, None, 0, None, 0)
+                else:
+                    self.gemm(dY, o, self.WTb[0], o, B, i, o, 0, None, dX0, i, None, 0, None, 0)
         return dX0
 
     def adam_step(self):
@@ -176,8 +196,7 @@ class MLP:
                          self.step_count, self.Wb[l], self.stream)
             abi.pcv_adam(self.b[l], self.mb[l], self.vb[l], self.gb[l], self.b[l].numel(), self.lr, b1, b2, self.eps,
                          self.step_count, None, self.stream)
-            o, i = self.W[l].shape
-            abi.pcv_transpose_bf16(self.Wb[l], o, i, i, self.WTb[l], o, self.stream)
+            self._transpose_weights(l)
 
     def loss(self, y: torch.Tensor, target: torch.Tensor, want_grad: bool = True):
         """MSE(y, target); returns (loss tensor [1] fp32, dy bf16 or None)."""
