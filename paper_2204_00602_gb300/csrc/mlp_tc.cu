@@ -110,13 +110,13 @@ __device__ __forceinline__ uint2 pack_bf16(float4 x)
     return r;
 }
 
-template <int BN, int MODE>
+template <int BN, int MODE, int KB>
 __global__ void __launch_bounds__(TC_THREADS, 2)
 gemm_bf16_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, const TcArgs a)
 {
-    constexpr uint32_t kABytes = TC_BM * TC_BK * 2, kBBytes = BN * TC_BK * 2, kStage = kABytes + kBBytes;
+    constexpr uint32_t kABytes = TC_BM * TC_BK * 2, kBBytes = BN * TC_BK * 2, kStage = KB * (kABytes + kBBytes);
     extern __shared__ __align__(1024) unsigned char smem_raw[];
-    // 1024-byte aligned ring of stages: [A 128x64 | B BNx64] bf16 each
+    // 1024-byte aligned ring of stages: KB blocks of A (128x64 bf16), then KB of B (BNx64)
     unsigned char* ring = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     __shared__ __align__(8) uint64_t full_bar[TC_MAX_STAGES], empty_bar[TC_MAX_STAGES], done_bar, mma_done;
     __shared__ uint32_t tmem_base;
@@ -124,7 +124,7 @@ gemm_bf16_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int m0 = blockIdx.y * TC_BM, n0 = blockIdx.x * BN;
-    const int nk = (a.K + TC_BK - 1) / TC_BK, stages = a.stages;
+    const int nk = (a.K + KB * TC_BK - 1) / (KB * TC_BK), stages = a.stages;
 
     if (tid == 0) {
         for (int s = 0; s < stages; ++s) {
@@ -145,24 +145,29 @@ gemm_bf16_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
     const uint32_t tmem = tmem_base;
     const long long polls = a.max_polls;
 
-    if (tid == 0) {
+    if (warp == 0 && tcx::elect_one()) {
         // ---------------- TMA producer
         int issued = 0;
         for (int kt = 0, st = 0, ph = 1; kt < nk && !s_fail; ++kt) {
             if (kt >= stages && !mbar_wait(&empty_bar[st], ph, polls)) { s_fail = 1; break; }
             unsigned char* sa = ring + st * kStage;
-            unsigned char* sb = sa + kABytes;
+            unsigned char* sb = sa + KB * kABytes;
             mbar_expect_tx(&full_bar[st], kStage);
-            if (a.at) {
-                tma_load_2d(sa, &mapA, &full_bar[st], m0, kt * TC_BK);
-                tma_load_2d(sa + 8192, &mapA, &full_bar[st], m0 + 64, kt * TC_BK);
-            } else {
-                tma_load_2d(sa, &mapA, &full_bar[st], kt * TC_BK, m0);
-            }
-            if (a.bt) {
-                for (int j = 0; j < BN; j += 64) tma_load_2d(sb + j * 128, &mapB, &full_bar[st], n0 + j, kt * TC_BK);
-            } else {
-                tma_load_2d(sb, &mapB, &full_bar[st], kt * TC_BK, n0);
+#pragma unroll
+            for (int h = 0; h < KB; ++h) {             // blocks beyond K are zero-filled
+                const int k0 = (kt * KB + h) * TC_BK;
+                if (a.at) {
+                    tma_load_2d(sa + h * kABytes, &mapA, &full_bar[st], m0, k0);
+                    tma_load_2d(sa + h * kABytes + 8192, &mapA, &full_bar[st], m0 + 64, k0);
+                } else {
+                    tma_load_2d(sa + h * kABytes, &mapA, &full_bar[st], k0, m0);
+                }
+                if (a.bt) {
+                    for (int j = 0; j < BN; j += 64)
+                        tma_load_2d(sb + h * kBBytes + j * 128, &mapB, &full_bar[st], n0 + j, k0);
+                } else {
+                    tma_load_2d(sb + h * kBBytes, &mapB, &full_bar[st], k0, n0);
+                }
             }
             ++issued;
             if (++st == stages) {
@@ -172,7 +177,7 @@ gemm_bf16_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
         }
         // the loads issued land in this CTA's shared memory before it may exit
         if (!tcx::wait_issued(full_bar, stages, (uint32_t)issued) && !s_fail) s_fail = 4;
-    } else if (tid == 32) {
+    } else if (warp == 1 && tcx::elect_one()) {
         // ---------------- MMA issuer
         const uint32_t idesc = tcx::idesc_bf16(TC_BM, BN) | (a.at ? 1u << 15 : 0u) | (a.bt ? 1u << 16 : 0u);
         // 16 of K further: 32 B along a K-major row, 16 rows of 128 B of an MN-major tile (16-byte units)
@@ -182,12 +187,15 @@ gemm_bf16_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
             if (!mbar_wait(&full_bar[st], ph, polls)) { s_fail = 2; all = false; break; }
             tcx::fence_after_sync();
             const unsigned char* sa = ring + st * kStage;
-            const unsigned char* sb = sa + kABytes;
+            const unsigned char* sb = sa + KB * kABytes;
             const uint64_t ad = a.at ? sdesc_mn_sw128(sa) : sdesc_sw128(sa);
             const uint64_t bd = a.bt ? sdesc_mn_sw128(sb) : sdesc_sw128(sb);
 #pragma unroll
-            for (int kk = 0; kk < TC_BK / 16; ++kk)
-                tcx::mma_bf16(tmem, ad + kk * astep, bd + kk * bstep, idesc, (kt > 0 || kk > 0) ? 1u : 0u);
+            for (int kk = 0; kk < KB * TC_BK / 16; ++kk) {
+                const int h = kk / (TC_BK / 16), j = kk % (TC_BK / 16);
+                tcx::mma_bf16(tmem, ad + h * (kABytes >> 4) + j * astep, bd + h * (kBBytes >> 4) + j * bstep, idesc,
+                              (kt > 0 || kk > 0) ? 1u : 0u);
+            }
             tcx::mma_commit(&empty_bar[st]);
             if (++st == stages) {
                 st = 0;
@@ -200,6 +208,12 @@ gemm_bf16_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
         tcx::mma_commit(&mma_done);
         if (!mbar_wait(&mma_done, 0, tcx::kCleanupPolls) && !s_fail) s_fail = 4;
     }
+
+    // The other lanes of the producer's and the issuer's warps park here: were
+    // they to poll done_bar meanwhile, the warp would alternate between the two
+    // paths and each K block's loads and MMAs would take about 400 cycles to
+    // issue (K = 4096: 28.8 us however wide the tile).
+    __syncwarp();
 
     // ---------------- epilogue (all warps)
     const bool ok = mbar_wait(&done_bar, 0, polls);
@@ -310,32 +324,40 @@ cudaError_t make_map(CUtensorMap* map, const void* base, int inner, int outer, i
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-template <int BN, int MODE>
+template <int BN, int MODE, int KB>
 cudaError_t launch_tile(const CUtensorMap& ma, const CUtensorMap& mb, const TcArgs& a, size_t smem, cudaStream_t s)
 {
-    cudaError_t e = cudaFuncSetAttribute(gemm_bf16_tc_kernel<BN, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(gemm_bf16_tc_kernel<BN, MODE, KB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
     const dim3 grid((a.N + BN - 1) / BN, (a.M + TC_BM - 1) / TC_BM);
-    gemm_bf16_tc_kernel<BN, MODE><<<grid, TC_THREADS, smem, s>>>(ma, mb, a);
+    gemm_bf16_tc_kernel<BN, MODE, KB><<<grid, TC_THREADS, smem, s>>>(ma, mb, a);
     note_launches(1);
     return cudaGetLastError();
 }
 
-template <int BN>
-cudaError_t launch_width(const CUtensorMap& ma, const CUtensorMap& mb, int mode, TcArgs a, int64_t tiles, cudaStream_t s)
+template <int BN, int KB>
+cudaError_t launch_depth(const CUtensorMap& ma, const CUtensorMap& mb, int mode, TcArgs a, uint32_t ring, cudaStream_t s)
 {
-    constexpr uint32_t stage = (TC_BM + BN) * TC_BK * 2;
-    const uint32_t ring = tiles > kTcSms ? TC_RING_TWO : TC_RING_ONE;
-    const int nk = (a.K + TC_BK - 1) / TC_BK;
+    constexpr uint32_t stage = KB * (TC_BM + BN) * TC_BK * 2;
+    const int nk = (a.K + KB * TC_BK - 1) / (KB * TC_BK);
     a.stages = std::min<int>(std::min<int>(TC_MAX_STAGES, ring / stage), std::max(nk, 2));
     const size_t smem = std::max<size_t>((size_t)a.stages * stage, 4 * 32 * 36 * sizeof(float)) + 1024;
     switch (mode) {
-    case 0: return launch_tile<BN, 0>(ma, mb, a, smem, s);
-    case 1: return launch_tile<BN, 1>(ma, mb, a, smem, s);
-    case 2: return launch_tile<BN, 2>(ma, mb, a, smem, s);
-    default: return launch_tile<BN, 3>(ma, mb, a, smem, s);
+    case 0: return launch_tile<BN, 0, KB>(ma, mb, a, smem, s);
+    case 1: return launch_tile<BN, 1, KB>(ma, mb, a, smem, s);
+    case 2: return launch_tile<BN, 2, KB>(ma, mb, a, smem, s);
+    default: return launch_tile<BN, 3, KB>(ma, mb, a, smem, s);
     }
+}
+
+template <int BN>
+cudaError_t launch_width(const CUtensorMap& ma, const CUtensorMap& mb, int mode, const TcArgs& a, int64_t tiles,
+                         cudaStream_t s)
+{
+    if (tiles > kTcSms) return launch_depth<BN, 1>(ma, mb, mode, a, TC_RING_TWO, s);
+    return a.K > 8 * TC_BK ? launch_depth<BN, 2>(ma, mb, mode, a, TC_RING_ONE, s)
+                           : launch_depth<BN, 1>(ma, mb, mode, a, TC_RING_ONE, s);
 }
 
 bool aligned_to(const void* p, size_t n) { return (uintptr_t)p % n == 0; }
