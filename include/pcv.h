@@ -534,6 +534,13 @@ int pcv_gemm_bf16_tc_t(const void* A, int lda, int a_transposed, const void* B, 
 int pcv_transpose_bf16(const void* in, int R, int C, int ldi, void* out, int ldo, void* stream);
 /* db[n] = sum_m dY[m][n] (bf16 in, fp32 out, fixed summation order). */
 int pcv_colsum_bf16(const void* dY, int M, int N, int ld, float* db, void* stream);
+/* The same for `count` matrices in one launch (jobs: host array). */
+typedef struct {
+    const void* dY;      /* M x N bf16, leading dimension ld */
+    float* db;           /* N sums (written)                 */
+    int32_t M, N, ld, reserved;
+} pcv_colsum_job;
+int pcv_colsum_bf16_multi(const pcv_colsum_job* jobs, int count, void* stream);
 /* X[b] = (sin phi_b, cos phi_b, 1, 0 ...) as bf16 rows of length ldx >= 2P+1;
  * the constant 1 carries the first layer's bias. */
 int pcv_phase_features(const double* phases, int B, int P, void* X, int ldx, void* stream);
@@ -549,6 +556,15 @@ int pcv_mse(const float* pred, const float* target, int64_t count, float* loss, 
  * bf16 copy of the updated weights to w_bf16 when it is not NULL. */
 int pcv_adam(float* w, float* m, float* v, const float* g, int64_t count, float lr, float beta1, float beta2,
              float eps, int step, void* w_bf16, void* stream);
+/* The same on `count` tensors in one launch (jobs: host array). */
+typedef struct {
+    float *w, *m, *v;
+    const float* g;
+    void* w_bf16;        /* or NULL */
+    int64_t count;
+} pcv_adam_job;
+int pcv_adam_multi(const pcv_adam_job* jobs, int count, float lr, float beta1, float beta2, float eps, int step,
+                   void* stream);
 int pcv_f32_to_bf16(const float* in, int64_t count, void* out, void* stream);
 /* Adam on FP64 parameters (the mesh phases of the optimisation loops). */
 int pcv_adam_f64(double* w, double* m, double* v, const double* g, int64_t count, double lr, double beta1,

@@ -25,7 +25,10 @@ __all__ = ["amplitudes", "amplitudes_batched", "BatchPlan", "distribution", "dis
 
 
 def _stream(device) -> int:
-    return torch.cuda.current_stream(device).cuda_stream
+    """The current stream's handle: what torch.cuda.current_stream(device).cuda_stream
+    returns, without making the Stream object (about 5 us of a 10 us call)."""
+    index = device.index if isinstance(device, torch.device) else torch.device(device).index
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device() if index is None else index)
 
 
 def _host_occ(occ, m: int) -> np.ndarray:

@@ -81,6 +81,8 @@ SIGNATURES = {
     "pcv_gemm_bf16_tc_t": (_i, [_vp, _i, _i, _vp, _i, _i, _i, _i, _i, _i, _vp, _vp, _i, _vp, _i, _vp, _i, _vp, _vp]),
     "pcv_gemm_bf16_tc": (_i, [_vp, _i, _vp, _i, _i, _i, _i, _i, _vp, _vp, _i, _vp, _i, _vp, _i, _vp, _vp]),
     "pcv_transpose_bf16": (_i, [_vp, _i, _i, _i, _vp, _i, _vp]),
+    "pcv_colsum_bf16_multi": (_i, [_vp, _i, _vp]),
+    "pcv_adam_multi": (_i, [_vp, _i, ctypes.c_float, ctypes.c_float, ctypes.c_float, ctypes.c_float, _i, _vp]),
     "pcv_colsum_bf16": (_i, [_vp, _i, _i, _i, _vp, _vp]),
     "pcv_phase_features": (_i, [_vp, _i, _i, _vp, _i, _vp]),
     "pcv_phase_features_grad": (_i, [_vp, _i, _i, _vp, _i, _vp, _vp]),
@@ -393,6 +395,27 @@ def pcv_mse_workspace() -> int:
 def pcv_mse(pred, target, count, loss, grad_pred_bf16, workspace, workspace_bytes, stream):
     return _call("pcv_mse", ptr(pred), ptr(target), count, ptr(loss), ptr(grad_pred_bf16), ptr(workspace),
                  workspace_bytes, stream)
+
+
+class pcv_colsum_job(ctypes.Structure):
+    _fields_ = [("dY", _vp), ("db", _vp), ("M", ctypes.c_int32), ("N", ctypes.c_int32), ("ld", ctypes.c_int32),
+                ("reserved", ctypes.c_int32)]
+
+
+def pcv_colsum_bf16_multi(jobs, stream):
+    """jobs: list of (dY, M, N, ld, db)."""
+    arr = (pcv_colsum_job * len(jobs))(*[(ptr(dY), ptr(db), M, N, ld, 0) for dY, M, N, ld, db in jobs])
+    return _call("pcv_colsum_bf16_multi", ctypes.addressof(arr), len(jobs), stream)
+
+
+class pcv_adam_job(ctypes.Structure):
+    _fields_ = [("w", _vp), ("m", _vp), ("v", _vp), ("g", _vp), ("w_bf16", _vp), ("count", _i64)]
+
+
+def pcv_adam_multi(jobs, lr, beta1, beta2, eps, step, stream):
+    """jobs: list of (w, m, v, g, w_bf16 or None)."""
+    arr = (pcv_adam_job * len(jobs))(*[(ptr(w), ptr(m), ptr(v), ptr(g), ptr(wb), w.numel()) for w, m, v, g, wb in jobs])
+    return _call("pcv_adam_multi", ctypes.addressof(arr), len(jobs), lr, beta1, beta2, eps, step, stream)
 
 
 def pcv_adam(w, m, v, g, count, lr, beta1, beta2, eps, step, w_bf16, stream):

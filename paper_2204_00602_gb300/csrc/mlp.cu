@@ -12,6 +12,7 @@
 
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cstdio>
 
 #include "pcv_common.cuh"
@@ -190,16 +191,27 @@ __global__ void transpose_bf16_kernel(const __nv_bfloat16* __restrict__ in, int 
 }
 
 // db[n] = sum_m dY[m][n] (bf16 input, fp32 sum in a fixed order: eight
-// interleaved chains per column, added in order).  8 columns per block, so
-// 1024 columns are 128 blocks, and 32 loads of a chain in flight: bound by the
-// loads' latency (4096 x 1024: 20 us with 32 columns per block and one load
-// at a time).
-__global__ void __launch_bounds__(64) colsum_bf16_kernel(const __nv_bfloat16* __restrict__ dY, int M, int N, int ld,
-                                                         float* __restrict__ db)
+// interleaved chains per column, added in order), for up to kColsumJobs
+// matrices in one launch.  8 columns per block and 32 loads of a chain in
+// flight: bound by the loads' latency (4096 x 1024 at first: 20 us, with 32
+// columns per block and one load at a time; a training step's four: 79 -> 33 us).
+constexpr int kColsumJobs = 8;
+struct ColsumArgs {
+    const __nv_bfloat16* dY[kColsumJobs];
+    float* db[kColsumJobs];
+    int M[kColsumJobs], N[kColsumJobs], ld[kColsumJobs];
+    int end[kColsumJobs];            // blocks up to and including this job
+};
+
+__global__ void __launch_bounds__(64) colsum_bf16_kernel(const __grid_constant__ ColsumArgs a)
 {
     constexpr int kAhead = 32;
     __shared__ float sh[8][9];
-    const int c = blockIdx.x * 8 + threadIdx.x;
+    int j = 0;
+    while ((int)blockIdx.x >= a.end[j]) ++j;
+    const __nv_bfloat16* __restrict__ dY = a.dY[j];
+    const int M = a.M[j], N = a.N[j], ld = a.ld[j];
+    const int c = ((int)blockIdx.x - (j ? a.end[j - 1] : 0)) * 8 + threadIdx.x;
     float s = 0.f;
     if (c < N) {
         int r = threadIdx.y;
@@ -217,20 +229,64 @@ __global__ void __launch_bounds__(64) colsum_bf16_kernel(const __nv_bfloat16* __
     if (threadIdx.y == 0 && c < N) {
         float t = 0.f;
         for (int y = 0; y < 8; ++y) t += sh[y][threadIdx.x];
-        db[c] = t;
+        a.db[j][c] = t;
     }
 }
 
-// x = [sin phi, cos phi, 1, 0...] (bf16, row length ldx)
-__global__ void features_kernel(const double* __restrict__ phases, int B, int P, __nv_bfloat16* __restrict__ X, int ldx)
+// Sine and cosine in FP64 from a table of 64 points of the circle: x = k h + r,
+// h = 2 pi / 64, |r| <= h / 2, then the addition theorem with Taylor's
+// polynomials in r (the next terms, r^9 / 9! and r^10 / 10!, are below 5e-18):
+// 18 FP64 instructions for both, where sin() and cos() take about 60 and bound
+// the kernel (4096 x 132 phases: 52 us).  Error below 3e-16, as a float the
+// same value but once in 1e8.
+__device__ __forceinline__ void sincos_table(double x, const double2* tab, double& s, double& c)
 {
-    const int b = blockIdx.y, j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= ldx) return;
-    float v = 0.f;
-    if (j < P) v = (float)sin(phases[(size_t)b * P + j]);
-    else if (j < 2 * P) v = (float)cos(phases[(size_t)b * P + j - P]);
-    else if (j == 2 * P) v = 1.f;
-    X[(size_t)b * ldx + j] = __float2bfloat16_rn(v);
+    if (!(fabs(x) < 1e6)) {
+        sincos(x, &s, &c);
+        return;
+    }
+    // k = rint(x / h): the sum's low mantissa bits
+    const double kShift = 6755399441055744.0;                         // 1.5 2^52
+    const double t = fma(x, 10.185916357881301489, kShift);
+    const int k = __double2loint(t);
+    const double kf = t - kShift;
+    double r = fma(-kf, 0.09817477042468103870, x);                   // h in two parts
+    r = fma(-kf, 3.827021247335479e-18, r);
+    const double q = r * r;
+    const double sr = fma(q * r, fma(q, fma(q, -1.0 / 5040, 1.0 / 120), -1.0 / 6), r);
+    const double cm = q * fma(q, fma(q, fma(q, 1.0 / 40320, -1.0 / 720), 1.0 / 24), -0.5);     // cos r - 1
+    const double2 e = tab[k & 63];
+    s = e.x + fma(e.x, cm, e.y * sr);
+    c = e.y + fma(e.y, cm, -(e.x * sr));
+}
+
+// x = [sin phi, cos phi, 1, 0...] (bf16, row length ldx).  A thread takes both
+// features of a phase; a block walks many rows, so its table is formed once.
+__global__ void __launch_bounds__(256) features_kernel(const double* __restrict__ phases, int B, int P,
+                                                       __nv_bfloat16* __restrict__ X, int ldx)
+{
+    __shared__ double2 tab[64];
+    if (threadIdx.x < 64) {
+        double s, c;
+        sincospi(threadIdx.x / 32.0, &s, &c);
+        tab[threadIdx.x] = make_double2(s, c);
+    }
+    __syncthreads();
+    const int64_t stride = (int64_t)gridDim.x * 256;
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < (int64_t)B * P; i += stride) {
+        const int64_t b = i / P;
+        const int j = (int)(i - b * P);
+        double s, c;
+        sincos_table(phases[i], tab, s, c);
+        X[b * ldx + j] = __float2bfloat16_rn((float)s);
+        X[b * ldx + P + j] = __float2bfloat16_rn((float)c);
+    }
+    const int pad = ldx - 2 * P;
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < (int64_t)B * pad; i += stride) {
+        const int64_t b = i / pad;
+        const int j = (int)(i - b * pad);
+        X[b * ldx + 2 * P + j] = __float2bfloat16_rn(j == 0 ? 1.f : 0.f);
+    }
 }
 
 // dL/dphi from dL/dx: d sin = cos, d cos = -sin
@@ -263,29 +319,74 @@ __global__ void mse_kernel(const float* __restrict__ pred, const float* __restri
     if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
 }
 
+// Sum of n <= 256 partials in index order.
 __global__ void sum_partials_kernel(const float* __restrict__ part, int n, float scale, float* out)
 {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
+    __shared__ float sh[256];
+    if (threadIdx.x < n) sh[threadIdx.x] = part[threadIdx.x];
+    __syncthreads();
+    if (threadIdx.x == 0) {
         float s = 0.f;
-        for (int i = 0; i < n; ++i) s += part[i];
+        for (int i = 0; i < n; ++i) s += sh[i];
         *out = s * scale;
     }
 }
 
-__global__ void adam_kernel(float* __restrict__ w, float* __restrict__ m, float* __restrict__ v, const float* __restrict__ g,
-                            int64_t count, float lr, float b1, float b2, float eps, float c1, float c2,
-                            __nv_bfloat16* __restrict__ wb)
+// Adam on up to kAdamJobs tensors in one launch (a training step of the
+// surrogate: eight tensors, 3 M weights; eight launches took 33 us), four
+// elements per thread where the pointers allow 16-byte accesses.
+constexpr int kAdamJobs = 16;
+struct AdamArgs {
+    float* w[kAdamJobs];
+    float* m[kAdamJobs];
+    float* v[kAdamJobs];
+    const float* g[kAdamJobs];
+    __nv_bfloat16* wb[kAdamJobs];
+    int64_t count[kAdamJobs];
+    int64_t end[kAdamJobs];          // blocks up to and including this job
+    int vec[kAdamJobs];
+    float lr, b1, b2, eps, c1, c2;
+};
+
+__device__ __forceinline__ float adam_one(const AdamArgs& a, float w, float& m, float& v, float g)
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= count) return;
-    const float gi = g[i];
-    const float mi = b1 * m[i] + (1.f - b1) * gi;
-    const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    const float wi = w[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-    w[i] = wi;
-    if (wb) wb[i] = __float2bfloat16_rn(wi);
+    const float mi = a.b1 * m + (1.f - a.b1) * g;
+    const float vi = a.b2 * v + (1.f - a.b2) * g * g;
+    m = mi;
+    v = vi;
+    return w - a.lr * (mi / a.c1) / (sqrtf(vi / a.c2) + a.eps);
+}
+
+__global__ void __launch_bounds__(256) adam_kernel(const __grid_constant__ AdamArgs a)
+{
+    int j = 0;
+    while ((int64_t)blockIdx.x >= a.end[j]) ++j;
+    const int64_t i = (((int64_t)blockIdx.x - (j ? a.end[j - 1] : 0)) * 256 + threadIdx.x) * 4;
+    const int64_t n = a.count[j];
+    float *w = a.w[j], *m = a.m[j], *v = a.v[j];
+    const float* g = a.g[j];
+    __nv_bfloat16* wb = a.wb[j];
+    if (a.vec[j] && i + 4 <= n) {
+        float4 w4 = *(float4*)(w + i), m4 = *(float4*)(m + i), v4 = *(float4*)(v + i);
+        const float4 g4 = *(const float4*)(g + i);
+        w4.x = adam_one(a, w4.x, m4.x, v4.x, g4.x);
+        w4.y = adam_one(a, w4.y, m4.y, v4.y, g4.y);
+        w4.z = adam_one(a, w4.z, m4.z, v4.z, g4.z);
+        w4.w = adam_one(a, w4.w, m4.w, v4.w, g4.w);
+        *(float4*)(w + i) = w4;
+        *(float4*)(m + i) = m4;
+        *(float4*)(v + i) = v4;
+        if (wb) {
+            __nv_bfloat162* o = (__nv_bfloat162*)(wb + i);
+            o[0] = __floats2bfloat162_rn(w4.x, w4.y);
+            o[1] = __floats2bfloat162_rn(w4.z, w4.w);
+        }
+        return;
+    }
+    for (int64_t q = i; q < min(n, i + 4); ++q) {
+        w[q] = adam_one(a, w[q], m[q], v[q], g[q]);
+        if (wb) wb[q] = __float2bfloat16_rn(w[q]);
+    }
 }
 
 __global__ void adam_f64_kernel(double* __restrict__ w, double* __restrict__ m, double* __restrict__ v,
@@ -308,10 +409,37 @@ __global__ void f32_to_bf16_kernel(const float* __restrict__ in, int64_t count, 
     if (i < count) out[i] = __float2bfloat16_rn(in[i]);
 }
 
-__global__ void log_f64_to_f32_kernel(const double* __restrict__ in, int64_t count, float* __restrict__ out)
+// out = (float)log(in).  FP64 bound, so the logarithm comes from a table: in =
+// 2^e m, c the reciprocal of the middle of m's 1/128 interval, r = m c - 1,
+// |r| <= 2^-8 + 2^-16, log in = e ln 2 - log c + log1p(r), the series up to r^6
+// (the next term is below 2^-58): 12 FP64 instructions against about 28 (1 M
+// values: 60 us before).  Near 1, where those terms cancel, and outside the
+// normal range: log().
+__global__ void __launch_bounds__(256) log_f64_to_f32_kernel(const double* __restrict__ in, int64_t count,
+                                                             float* __restrict__ out)
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < count) out[i] = (float)log(in[i]);
+    __shared__ double2 tab[128];                        // c, -log c
+    if (threadIdx.x < 128) {
+        const double c = 1.0 / (1.0 + (threadIdx.x + 0.5) / 128.0);
+        tab[threadIdx.x] = make_double2(c, -log(c));
+    }
+    __syncthreads();
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < count; i += (int64_t)gridDim.x * 256) {
+        const double x = in[i];
+        const int hi = __double2hiint(x), ef = (hi >> 20) & 0x7FF;
+        const double2 t = tab[(hi >> 13) & 127];
+        const double m = __hiloint2double((hi & 0xFFFFF) | 0x3FF00000, __double2loint(x));
+        const double e = __hiloint2double(0x43300000, (ef - 1023) ^ (int)0x80000000) - 4503601774854144.0;
+        const double r = fma(m, t.x, -1.0);
+        double q = fma(r, -1.0 / 6, 0.2);
+        q = fma(r, q, -0.25);
+        q = fma(r, q, 1.0 / 3);
+        q = fma(r, q, -0.5);
+        q = fma(r * r, q, r);
+        double y = fma(e, 0.69314718055994530942, t.y) + q;
+        if (hi < 0 || ef == 0 || ef == 0x7FF || fabs(y) < 0.01) y = log(x);
+        out[i] = (float)y;
+    }
 }
 
 __global__ void exp_f32_to_f64_kernel(const float* __restrict__ in, int64_t count, double* __restrict__ out)
@@ -331,7 +459,7 @@ cudaError_t launch_exp_f32_to_f64(const float* in, int64_t count, double* out, c
 
 cudaError_t launch_log_f64_to_f32(const double* in, int64_t count, float* out, cudaStream_t s)
 {
-    log_f64_to_f32_kernel<<<(unsigned)((count + 255) / 256), 256, 0, s>>>(in, count, out);
+    log_f64_to_f32_kernel<<<(unsigned)std::min<int64_t>(152 * 4, (count + 255) / 256), 256, 0, s>>>(in, count, out);
     note_launches(1);
     return cudaGetLastError();
 }
@@ -352,16 +480,34 @@ cudaError_t launch_transpose_bf16(const void* in, int R, int C, int ldi, void* o
     return cudaGetLastError();
 }
 
-cudaError_t launch_colsum_bf16(const void* dY, int M, int N, int ld, float* db, cudaStream_t s)
+cudaError_t launch_colsum_bf16(const pcv_colsum_job* jobs, int count, cudaStream_t s)
 {
-    colsum_bf16_kernel<<<(N + 7) / 8, dim3(8, 8), 0, s>>>((const __nv_bfloat16*)dY, M, N, ld, db);
-    note_launches(1);
-    return cudaGetLastError();
+    for (int j0 = 0; j0 < count; j0 += kColsumJobs) {
+        ColsumArgs a{};
+        int blocks = 0;
+        const int nj = std::min(kColsumJobs, count - j0);
+        for (int j = 0; j < nj; ++j) {
+            const pcv_colsum_job& q = jobs[j0 + j];
+            a.dY[j] = (const __nv_bfloat16*)q.dY;
+            a.db[j] = q.db;
+            a.M[j] = q.M;
+            a.N[j] = q.N;
+            a.ld[j] = q.ld;
+            blocks += (q.N + 7) / 8;
+            a.end[j] = blocks;
+        }
+        colsum_bf16_kernel<<<blocks, dim3(8, 8), 0, s>>>(a);
+        note_launches(1);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 cudaError_t launch_features(const double* phases, int B, int P, void* X, int ldx, cudaStream_t s)
 {
-    features_kernel<<<dim3((ldx + 127) / 128, B), 128, 0, s>>>(phases, B, P, (__nv_bfloat16*)X, ldx);
+    const int64_t blocks = std::min<int64_t>(152 * 2, ((int64_t)B * P + 255) / 256);
+    features_kernel<<<(unsigned)blocks, 256, 0, s>>>(phases, B, P, (__nv_bfloat16*)X, ldx);
     note_launches(1);
     return cudaGetLastError();
 }
@@ -382,19 +528,44 @@ cudaError_t launch_mse(const float* pred, const float* tgt, int64_t count, float
     note_launches(1);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    sum_partials_kernel<<<1, 32, 0, s>>>(part, 256, 1.f / (float)count, loss);
+    sum_partials_kernel<<<1, 256, 0, s>>>(part, 256, 1.f / (float)count, loss);
     note_launches(1);
     return cudaGetLastError();
 }
 
-cudaError_t launch_adam(float* w, float* m, float* v, const float* g, int64_t count, float lr, float b1, float b2,
-                        float eps, int step, void* wb, cudaStream_t s)
+cudaError_t launch_adam(const pcv_adam_job* jobs, int count, float lr, float b1, float b2, float eps, int step,
+                        cudaStream_t s)
 {
-    const float c1 = 1.f - powf(b1, (float)step), c2 = 1.f - powf(b2, (float)step);
-    adam_kernel<<<(unsigned)((count + 255) / 256), 256, 0, s>>>(w, m, v, g, count, lr, b1, b2, eps, c1, c2,
-                                                                 (__nv_bfloat16*)wb);
-    note_launches(1);
-    return cudaGetLastError();
+    for (int j0 = 0; j0 < count; j0 += kAdamJobs) {
+        AdamArgs a{};
+        a.lr = lr;
+        a.b1 = b1;
+        a.b2 = b2;
+        a.eps = eps;
+        a.c1 = 1.f - powf(b1, (float)step);
+        a.c2 = 1.f - powf(b2, (float)step);
+        int64_t blocks = 0;
+        const int nj = std::min(kAdamJobs, count - j0);
+        for (int j = 0; j < nj; ++j) {
+            const pcv_adam_job& q = jobs[j0 + j];
+            a.w[j] = q.w;
+            a.m[j] = q.m;
+            a.v[j] = q.v;
+            a.g[j] = q.g;
+            a.wb[j] = (__nv_bfloat16*)q.w_bf16;
+            a.count[j] = q.count;
+            a.vec[j] = ((uintptr_t)q.w | (uintptr_t)q.m | (uintptr_t)q.v | (uintptr_t)q.g) % 16 == 0 &&
+                       (uintptr_t)q.w_bf16 % 4 == 0;
+            blocks += (q.count + 1023) / 1024;
+            a.end[j] = blocks;
+        }
+        if (blocks > INT32_MAX) return cudaErrorInvalidConfiguration;
+        adam_kernel<<<(unsigned)blocks, 256, 0, s>>>(a);
+        note_launches(1);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 cudaError_t launch_adam_f64(double* w, double* m, double* v, const double* g, int64_t count, double lr, double b1,
@@ -464,7 +635,17 @@ int pcv_transpose_bf16(const void* in, int R, int C, int ldi, void* out, int ldo
 int pcv_colsum_bf16(const void* dY, int M, int N, int ld, float* db, void* stream)
 {
     if (!dY || !db || M < 1 || N < 1 || ld < N) return mlp_bad("colsum_bf16: bad arguments");
-    return mlp_ok(pcv::launch_colsum_bf16(dY, M, N, ld, db, (cudaStream_t)stream), "colsum_bf16");
+    const pcv_colsum_job j{dY, db, M, N, ld, 0};
+    return mlp_ok(pcv::launch_colsum_bf16(&j, 1, (cudaStream_t)stream), "colsum_bf16");
+}
+
+int pcv_colsum_bf16_multi(const pcv_colsum_job* jobs, int count, void* stream)
+{
+    if (count < 0 || (count > 0 && !jobs)) return mlp_bad("colsum_bf16_multi: bad arguments");
+    for (int j = 0; j < count; ++j)
+        if (!jobs[j].dY || !jobs[j].db || jobs[j].M < 1 || jobs[j].N < 1 || jobs[j].ld < jobs[j].N)
+            return mlp_bad("colsum_bf16_multi: bad job");
+    return mlp_ok(pcv::launch_colsum_bf16(jobs, count, (cudaStream_t)stream), "colsum_bf16_multi");
 }
 
 int pcv_phase_features(const double* phases, int B, int P, void* X, int ldx, void* stream)
@@ -494,7 +675,18 @@ int pcv_adam(float* w, float* m, float* v, const float* g, int64_t count, float 
              float eps, int step, void* w_bf16, void* stream)
 {
     if (!w || !m || !v || !g || count < 1 || step < 1) return mlp_bad("adam: bad arguments");
-    return mlp_ok(pcv::launch_adam(w, m, v, g, count, lr, beta1, beta2, eps, step, w_bf16, (cudaStream_t)stream), "adam");
+    const pcv_adam_job j{w, m, v, g, w_bf16, count};
+    return mlp_ok(pcv::launch_adam(&j, 1, lr, beta1, beta2, eps, step, (cudaStream_t)stream), "adam");
+}
+
+int pcv_adam_multi(const pcv_adam_job* jobs, int count, float lr, float beta1, float beta2, float eps, int step,
+                   void* stream)
+{
+    if (count < 0 || (count > 0 && !jobs) || step < 1) return mlp_bad("adam_multi: bad arguments");
+    for (int j = 0; j < count; ++j)
+        if (!jobs[j].w || !jobs[j].m || !jobs[j].v || !jobs[j].g || jobs[j].count < 1)
+            return mlp_bad("adam_multi: bad job");
+    return mlp_ok(pcv::launch_adam(jobs, count, lr, beta1, beta2, eps, step, (cudaStream_t)stream), "adam_multi");
 }
 
 int pcv_exp_f32_to_f64(const float* in, int64_t count, double* out, void* stream)

@@ -158,6 +158,7 @@ class MLP:
         self.gW, self.gb = [None] * self.L, [None] * self.L
         dY = dy_bf16
         dX0 = None
+        sums = []                            # bias gradients: the layers' column sums, one launch
         for l in reversed(range(self.L)):
             o, i = self.W[l].shape
             if want_param_grad:
@@ -171,7 +172,7 @@ class MLP:
                     abi.pcv_transpose_bf16(self.acts[l], B, i, i, XT, B, self.stream)
                     self.gemm(dYT, B, XT, B, o, i, B, 0, None, gW, i, None, 0, None, 0)
                 gb = self._buf(f"gb{l}", (o,), torch.float32)
-                abi.pcv_colsum_bf16(dY, B, o, o, gb, self.stream)
+                sums.append((dY, B, o, o, gb))
                 self.gW[l], self.gb[l] = gW, gb
             if l > 0:
                 dprev = self._buf(f"dY{l - 1}", (B, i), torch.bfloat16)
@@ -186,16 +187,16 @@ class MLP:
                     self.gemm_nt(dY, o, 0, self.Wb[0], i, 1, B, i, o, 0, dX0, i, None, 0, None, 0)
                 else:
                     self.gemm(dY, o, self.WTb[0], o, B, i, o, 0, None, dX0, i, None, 0, None, 0)
+        if sums:
+            abi.pcv_colsum_bf16_multi(sums, self.stream)
         return dX0
 
     def adam_step(self):
         self.step_count += 1
-        b1, b2 = self.betas
+        jobs = [(self.W[l], self.mW[l], self.vW[l], self.gW[l], self.Wb[l]) for l in range(self.L)]
+        jobs += [(self.b[l], self.mb[l], self.vb[l], self.gb[l], None) for l in range(self.L)]
+        abi.pcv_adam_multi(jobs, self.lr, *self.betas, self.eps, self.step_count, self.stream)
         for l in range(self.L):
-            abi.pcv_adam(self.W[l], self.mW[l], self.vW[l], self.gW[l], self.W[l].numel(), self.lr, b1, b2, self.eps,
-                         self.step_count, self.Wb[l], self.stream)
-            abi.pcv_adam(self.b[l], self.mb[l], self.vb[l], self.gb[l], self.b[l].numel(), self.lr, b1, b2, self.eps,
-                         self.step_count, None, self.stream)
             self._transpose_weights(l)
 
     def loss(self, y: torch.Tensor, target: torch.Tensor, want_grad: bool = True):
