@@ -246,7 +246,7 @@ struct SplitMultiArgs {
 
 // Glynn's sum of one output in Gray order, rows ascending, FP64 throughout.
 template <int NMAX>
-__device__ __noinline__ double2 glynn_row_sums(const double2* U, const SplitMultiArgs& a, const int* row)
+__device__ __forceinline__ double2 glynn_row_sums(const double2* U, const SplitMultiArgs& a, const int* row)
 {
     const int m = a.o.m, n = a.o.n, w1 = a.o.k1 + 1;
     double2 y[NMAX];
@@ -270,14 +270,16 @@ __device__ __noinline__ double2 glynn_row_sums(const double2* U, const SplitMult
 }
 
 template <int NMAX>
-__global__ void __launch_bounds__(kThreads) split_multi_kernel(const __grid_constant__ SplitMultiArgs a)
+__global__ void __launch_bounds__(kThreads, 2) split_multi_kernel(const __grid_constant__ SplitMultiArgs a)
 {
     extern __shared__ double2 s_tab[];   // per unitary F, G; one scratch level; one column; the counts
+    __shared__ int s_lost;
+    __shared__ uint16_t s_list[kThreads * kMulti];
     const int m = a.o.m, n = a.o.n, k1 = a.o.k1, k2 = a.o.k2, w1 = k1 + 1;
     double2* s_scratch = s_tab + kMulti * (a.n1 + a.n2);
     double2* s_u = s_scratch + a.ns;
     uint32_t* s_t = (uint32_t*)(s_u + m);
-    int* s_e = (int*)(s_t + (m + 1) * w1);   // per unitary and mode: exponent of the row's squared norm
+    int* s_e = (int*)(s_t + (m + 1) * w1);   // per unitary and mode: exponent of the row's squared norm, stride w1
     const int b0 = blockIdx.y * kMulti;
     count_table(s_t, m, k1);
     for (int q = threadIdx.x; q < kMulti * m; q += kThreads) {
@@ -287,7 +289,7 @@ __global__ void __launch_bounds__(kThreads) split_multi_kernel(const __grid_cons
             const double2 u = Ur[a.cols[j]];
             f = fma(u.x, u.x, fma(u.y, u.y, f));
         }
-        s_e[q] = f > 0.0 && isfinite(f) ? ilogb(f) : 0;
+        s_e[q / m * m * w1 + (m - 1 - q % m) * w1] = f > 0.0 && isfinite(f) ? ilogb(f) : 0;   // at the mode's table row
     }
     // both tables of each unitary, level by level; the last level lands in
     // place, the one before in the scratch, and so on back
@@ -347,52 +349,67 @@ __global__ void __launch_bounds__(kThreads) split_multi_kernel(const __grid_cons
     __syncthreads();
     const int64_t o0 = (int64_t)blockIdx.x * a.per_block;
     const int64_t o1 = min(a.o.n_out, o0 + a.per_block);
-    for (int64_t o = o0 + threadIdx.x; o < o1; o += kThreads) {
-        int row[NMAX];
-        uint32_t same;
-        double f;
-        const bool ok = decode_rows<NMAX>(a.o, o, row, same, f);
-        double2 acc[kMulti];
+    for (int64_t base = o0; base < o1; base += kThreads) {
+        if (threadIdx.x == 0) s_lost = 0;
+        __syncthreads();
+        const int64_t o = base + threadIdx.x;
+        if (o < o1) {
+            int row[NMAX];
+            uint32_t same;
+            double f;
+            const bool ok = decode_rows<NMAX>(a.o, o, row, same, f);
+            double2 acc[kMulti];
 #pragma unroll
-        for (int j = 0; j < kMulti; ++j) acc[j] = make_double2(0.0, 0.0);
-        if (ok) {
-            uint32_t mask = (1u << k1) - 1;
-            for (int64_t q = 0; q < a.o.masks; ++q) {
-                if (((mask & same) & ~(mask << 1)) == 0) {
-                    uint32_t rp = a.n1 - 1, rq = a.n2 - 1;
-                    split_ranks<NMAX>(s_t, row, n, k1, k2, mask, rp, rq);
-#pragma unroll
-                    for (int j = 0; j < kMulti; ++j) {
-                        const double2* F = s_tab + j * (a.n1 + a.n2);
-                        cmac(acc[j], F[rp], F[a.n1 + rq]);
-                    }
-                }
-                mask = next_mask(mask);
-            }
-        }
-        const double sc = sqrt(f) * a.o.norm_t;
-#pragma unroll
-        for (int j = 0; j < kMulti; ++j) {
-            if (b0 + j >= a.B) break;
-            double2 v = make_double2(0.0, 0.0);
+            for (int j = 0; j < kMulti; ++j) acc[j] = make_double2(0.0, 0.0);
             if (ok) {
+                uint32_t mask = (1u << k1) - 1;
+                for (int64_t q = 0; q < a.o.masks; ++q) {
+                    if (((mask & same) & ~(mask << 1)) == 0) {
+                        uint32_t rp = a.n1 - 1, rq = a.n2 - 1;
+                        split_ranks<NMAX>(s_t, row, n, k1, k2, mask, rp, rq);
+#pragma unroll
+                        for (int j = 0; j < kMulti; ++j) {
+                            const double2* F = s_tab + j * (a.n1 + a.n2);
+                            cmac(acc[j], F[rp], F[a.n1 + rq]);
+                        }
+                    }
+                    mask = next_mask(mask);
+                }
+            }
+            const double sc = sqrt(f) * a.o.norm_t;
+#pragma unroll
+            for (int j = 0; j < kMulti; ++j) {
+                if (b0 + j >= a.B) break;
+                const double2 v = ok ? make_double2(acc[j].x * sc, acc[j].y * sc) : make_double2(0.0, 0.0);
+                const int64_t at = (int64_t)(b0 + j) * a.o.n_out + o;
+                if (a.o.amp) a.o.amp[at] = v;
+                if (a.o.prob) a.o.prob[at] = fma(v.x, v.x, v.y * v.y);
+                if (!ok) continue;
                 const double w = fma(acc[j].x, acc[j].x, acc[j].y * acc[j].y) * f;      // |Perm|^2 / prod S!
                 int e = -60;
 #pragma unroll
                 for (int p = 0; p < NMAX; ++p)
-                    if (p < n) e += s_e[j * m + m - 1 - row[p] / w1];
-                if (w < scalbn(1.0, e)) {
-                    const double gs = ldexp(1.0 / sqrt(f) * a.o.norm_t, -(n - 1));
-                    const double2 g = glynn_row_sums<NMAX>(a.U + (size_t)(b0 + j) * m * m, a, row);
-                    v = make_double2(g.x * gs, g.y * gs);
-                } else {
-                    v = make_double2(acc[j].x * sc, acc[j].y * sc);
-                }
+                    if (p < n) e += s_e[j * m * w1 + row[p]];
+                if (w < scalbn(1.0, e)) s_list[atomicAdd(&s_lost, 1)] = (uint16_t)(threadIdx.x * kMulti + j);
             }
-            const int64_t at = (int64_t)(b0 + j) * a.o.n_out + o;
+        }
+        __syncthreads();
+        // the outputs lost in rounding, a thread each (their order does not matter)
+        for (int q = threadIdx.x; q < s_lost; q += kThreads) {
+            const int j = s_list[q] % kMulti;
+            const int64_t lo = base + s_list[q] / kMulti;
+            int row[NMAX];
+            uint32_t same;
+            double f;
+            decode_rows<NMAX>(a.o, lo, row, same, f);
+            const double gs = ldexp(1.0 / sqrt(f) * a.o.norm_t, -(n - 1));
+            const double2 g = glynn_row_sums<NMAX>(a.U + (size_t)(b0 + j) * m * m, a, row);
+            const double2 v = make_double2(g.x * gs, g.y * gs);
+            const int64_t at = (int64_t)(b0 + j) * a.o.n_out + lo;
             if (a.o.amp) a.o.amp[at] = v;
             if (a.o.prob) a.o.prob[at] = fma(v.x, v.x, v.y * v.y);
         }
+        __syncthreads();
     }
 }
 
@@ -427,7 +444,7 @@ size_t multi_smem(int m, int n)
     const int64_t n1 = mset_h(m, k1), n2 = mset_h(m, n - k1), ns = mset_h(m, k1 - 1);
     if (n1 < 0 || n1 > (1 << 20)) return SIZE_MAX;
     return (size_t)(kMulti * (n1 + n2) + ns + m) * sizeof(double2) + (size_t)(m + 1) * (k1 + 1) * sizeof(uint32_t) +
-           (size_t)kMulti * m * sizeof(int);
+           (size_t)kMulti * m * (k1 + 1) * sizeof(int);
 }
 
 SplitOut split_out(const pcv_batch_desc& d, double norm_t)
