@@ -214,18 +214,21 @@ int64_t pcv_distribution_tc_workspace(int m, int n);
  * default plan: for 2 <= n <= 10 and m >= 2 the single-pass plan of the
  * tensor-core products (= pcv_distribution_tc_workspace), otherwise the FP64
  * plan.  A smaller workspace (>= pcv_distribution_workspace_min) is accepted:
- * pcv_distribution then takes the FP64 products, in more passes if needed. */
+ * where it does not hold the state expansion (pcv_distribution_slos_workspace(
+ * 1, m, n) + 256 bytes) pcv_distribution takes the FP64 products, in more
+ * passes if needed. */
 int64_t pcv_distribution_workspace(int m, int n);
 int64_t pcv_distribution_workspace_min(int m, int n);
 
-/* The path pcv_distribution (PCV_ALGO_AUTO) takes for m modes, n photons
- * and a workspace of workspace_bytes: PCV_ALGO_FACTOR_TC when 2 <= n <= 10,
- * m >= 2 and workspace_bytes >= pcv_distribution_tc_workspace(m, n), else
- * PCV_ALGO_FACTOR, which here names the FP64 path: by state expansion (the
- * computation of PCV_ALGO_SLOS) when the workspace also holds its level
- * buffers (pcv_distribution_slos_workspace(1, m, n) + 256 bytes), else the
- * factorised sum with FP64 products, in as many passes as the workspace
- * asks for.  All give the same amplitudes to double precision.  Returns
+/* The plan whose workspace pcv_distribution (PCV_ALGO_AUTO) finds for m modes,
+ * n photons and workspace_bytes: PCV_ALGO_FACTOR_TC when 2 <= n <= 10, m >= 2
+ * and workspace_bytes >= pcv_distribution_tc_workspace(m, n), else
+ * PCV_ALGO_FACTOR.  Under either plan the call computes by state expansion
+ * (the method of PCV_ALGO_SLOS) when the workspace holds its level buffers
+ * (pcv_distribution_slos_workspace(1, m, n) + 256 bytes), which is never slower;
+ * else by the tensor-core products or by the factorised sum with FP64 products,
+ * in as many passes as the workspace asks for.  All give the same amplitudes to
+ * double precision.  Returns
  * the algorithm code, or PCV_EINVAL for sizes out of range.  No counterpart in
  * the paper. */
 int pcv_distribution_auto_algo(int m, int n, int64_t workspace_bytes);
@@ -234,14 +237,14 @@ int pcv_distribution_auto_algo(int m, int n, int64_t workspace_bytes);
  * distribution, Sec. 3.2.3, computed here from Eq. eqperm).
  *   prob  device, C(m+n-1,n) doubles (written) or NULL
  *   amp   device, C(m+n-1,n) pcv_c64 (written) or NULL; not both NULL
- * The algorithm factorises Glynn's sum: with sign vectors on the input
- * photons, every output shares the per-mode row sums
+ * The photons are added one at a time (PCV_ALGO_SLOS below) where the workspace
+ * holds two levels of that, as pcv_distribution_workspace bytes do.  Else the
+ * algorithm factorises Glynn's sum: with sign vectors on the input photons, every output shares the per-mode row sums
  * y_r(d) = sum_j d_j U[r][c_j], and a(S) = sum_d (sign, scale) prod_r y_r(d)^{s_r};
  * the product splits into the modes below and above m/2, so each output costs
  * one complex multiply-add per sign vector.  Those products run on the tensor
  * cores in exact integer arithmetic (PCV_ALGO_FACTOR_TC below) when the input
- * has 2..10 photons and the workspace holds that plan, else the call takes the
- * FP64 path; pcv_distribution_auto_algo tells which. */
+ * has 2..10 photons and the workspace holds that plan, else in FP64. */
 int pcv_distribution(const pcv_c64* U, int m, const uint8_t* input_occ,
                      double* prob, pcv_c64* amp,
                      void* workspace, int64_t workspace_bytes, void* stream);

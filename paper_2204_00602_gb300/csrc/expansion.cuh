@@ -65,6 +65,50 @@ __device__ __forceinline__ int next_mode(const I* t, int w1, int m, int v, int r
         ++v;
     }
 }
+
+// State i of S_{m,k} (count table mc, row length w1): term(r, rank) for every
+// occupied mode r, rank that of the state without one photon of r among the
+// prev_n states of S_{m,k-1}.  Returns sqrt(prod s!).
+template <int KMAX, typename I, typename F>
+__device__ __forceinline__ double expand_state(const I* mc, int w1, int m, int k, I i, I prev_n, const double* sqrtfact,
+                                               F&& term)
+{
+    int l[KMAX];                               // sorted mode list
+    {
+        int v = 0;
+#pragma unroll
+        for (int p = 0; p < KMAX; ++p) {
+            if (p >= k) break;
+            v = next_mode<I>(mc, w1, m, v, k - 1 - p, i);
+            l[p] = v;
+        }
+    }
+    auto t = [&](int mode, int j) { return mc[(m - mode - 1) * w1 + j]; };
+    // prev_n - 1 minus the terms of the list without position p: `pre` those
+    // before it, `suf` those after it (moved up by one)
+    I pre = prev_n - 1, suf = 0;
+#pragma unroll
+    for (int q = 1; q < KMAX; ++q)
+        if (q < k) suf += t(l[q], k - q);
+    double sfac = 1.0;
+    int mult = 0;
+#pragma unroll
+    for (int p = 0; p < KMAX; ++p) {
+        if (p >= k) break;
+        const int r = l[p];
+        mult = (p > 0 && l[p > 0 ? p - 1 : 0] == r) ? mult + 1 : 1;
+        const int nxt = p + 1 < k ? l[p + 1 < KMAX ? p + 1 : p] : -1;
+        if (nxt != r) {                        // one term per occupied mode, at its last copy
+            term(r, (I)(pre - suf));
+            if (mult > 1) sfac *= sqrtfact[mult];
+        }
+        if (p + 1 < k) {
+            pre -= t(r, k - 1 - p);
+            suf -= t(nxt, k - 1 - p);
+        }
+    }
+    return sfac;
+}
 #endif
 
 }  // namespace pcv

@@ -237,13 +237,24 @@ __global__ void multiset_table_kernel(int64_t* t, int amax, int kmax)
 {
     const int a = blockIdx.x * blockDim.x + threadIdx.x;
     if (a > amax) return;
-    unsigned __int128 c = 1;                  // C(a+k-1, k) by the multiplicative recurrence
+    // C(a+k-1, k) by the multiplicative recurrence: in 32 bits while the product
+    // fits (a 128-bit division takes some hundred instructions, and this kernel
+    // is the first of most calls), then in 64, then in 128
+    uint64_t c = 1;
     bool sat = false;
     t[a * (kmax + 1)] = 1;
     for (int k = 1; k <= kmax; ++k) {
         if (!sat) {
-            c = c * (unsigned __int128)(a + k - 1) / (unsigned __int128)k;
-            if (c > (unsigned __int128)INT64_MAX) sat = true;
+            const uint64_t f = (uint64_t)(a + k - 1);
+            if (c * f <= UINT32_MAX && c <= UINT32_MAX) {
+                c = (uint32_t)(c * f) / (uint32_t)k;
+            } else if (c < (1ull << 48)) {       // f < 2^11: the product is below 2^59
+                c = c * f / (uint64_t)k;
+            } else {
+                const unsigned __int128 w = (unsigned __int128)c * f / (unsigned __int128)k;
+                sat = w > (unsigned __int128)INT64_MAX;
+                c = (uint64_t)w;
+            }
         }
         t[a * (kmax + 1) + k] = sat ? INT64_MAX : (int64_t)c;
     }

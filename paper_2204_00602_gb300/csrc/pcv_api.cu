@@ -620,14 +620,27 @@ static int64_t tc_ws_bytes(int m, int n)
     return pcv::dist_plan_tc(p, true, &dp);
 }
 
-// PCV_ALGO_AUTO for one full distribution: the tensor-core products when the
-// input has 2..10 photons over m >= 2 modes and the workspace holds their
-// single-pass plan, else the FP64 products (which accept any workspace down to
+// PCV_ALGO_AUTO for one full distribution: the tensor-core plan when the input
+// has 2..10 photons over m >= 2 modes and the workspace holds its single pass,
+// else the FP64 path (which accepts any workspace down to
 // pcv_distribution_workspace_min).
 static int auto_dist_algo(int m, int n, int64_t workspace_bytes)
 {
     const int64_t tc = tc_ws_bytes(m, n);
     return (tc >= 0 && workspace_bytes >= tc) ? PCV_ALGO_FACTOR_TC : PCV_ALGO_FACTOR;
+}
+
+// Either plan of AUTO is computed by state expansion where the workspace holds
+// its two levels (it does wherever it holds the tensor-core plan, but for the
+// space's limits in fp64_expand_ws): n multiply-adds per output at most instead
+// of 2^(n-1).  Measured over m = 6..64, n = 3..10, 56 to 20 M outputs, the
+// products against the expansion: m=6 n=3 66 and 31 us, m=13 n=7 167 and 62,
+// m=16 n=8 196 and 101, m=10 n=10 249 and 83, m=24 n=7 314 and 198, m=20 n=10
+// 2397 and 2202; there is no size on the other side.
+static bool auto_expands(int m, int n, int64_t workspace_bytes)
+{
+    const int64_t x = fp64_expand_ws(1, m, n);
+    return x >= 0 && workspace_bytes >= x;
 }
 
 int64_t pcv_distribution_workspace(int m, int n)
@@ -689,10 +702,9 @@ static int distribution_fp64(const pcv_c64* U, int B, int m, const uint8_t* inpu
     if (B > 1 && (lo != 0 || hi != N)) return fail(PCV_EINVAL, "output ranges take one unitary");
     const int64_t xws = expand ? fp64_expand_ws(B, m, p.n) : -1;
     if (xws >= 0 && workspace_bytes >= xws) {
-        cudaError_t e = cudaMemsetAsync(workspace, 0, 16, s);             // the call's status word
-        if (e != cudaSuccess) return cuda_fail(e, "status word");
         pcv::stage_begin(pcv::kStagePlain, s);
-        e = pcv::launch_slos(p, B, (const double2*)U, lo, hi, prob, (double2*)amp, (char*)workspace + 256, s);
+        cudaError_t e = pcv::launch_slos(p, B, (const double2*)U, lo, hi, prob, (double2*)amp, (char*)workspace + 256,
+                                         workspace, s);
         pcv::stage_end(pcv::kStagePlain, s);
         return e == cudaSuccess ? PCV_OK : cuda_fail(e, "state expansion");
     }
@@ -745,7 +757,7 @@ int pcv_distribution_slos(const pcv_c64* U, int B, int m, const uint8_t* input_o
         return fail(PCV_ENOMEM, "workspace of %lld bytes (256-byte aligned) needed, %lld given", (long long)need,
                     (long long)workspace_bytes);
     pcv::stage_begin(pcv::kStagePlain, s);
-    cudaError_t e = pcv::launch_slos(p, B, (const double2*)U, 0, N, prob, (double2*)amp, workspace, s);
+    cudaError_t e = pcv::launch_slos(p, B, (const double2*)U, 0, N, prob, (double2*)amp, workspace, nullptr, s);
     pcv::stage_end(pcv::kStagePlain, s);
     return e == cudaSuccess ? PCV_OK : cuda_fail(e, "state expansion");
 }
@@ -797,11 +809,12 @@ int pcv_distribution_ex(const pcv_c64* U, int m, const uint8_t* input_occ,
                         void* workspace, int64_t workspace_bytes, void* stream)
 {
     const bool choose = algo == PCV_ALGO_AUTO;
+    int n = 0;
     if (choose && m >= 1 && m <= PCV_MAX_MODES && input_occ) {
-        int n = 0;
         for (int i = 0; i < m; ++i) n += input_occ[i];
         algo = auto_dist_algo(m, n, workspace ? workspace_bytes : 0);
     }
+    if (choose && algo == PCV_ALGO_FACTOR_TC && auto_expands(m, n, workspace_bytes)) algo = PCV_ALGO_AUTO;
     if (algo == PCV_ALGO_FACTOR_TC)
         return distribution_tc(U, m, input_occ, 0, -1, prob, amp, workspace, workspace_bytes, stream);
     if (algo == PCV_ALGO_SLOS)
@@ -882,7 +895,7 @@ int pcv_distribution_range(const pcv_c64* U, int m, const uint8_t* input_occ, in
         return end <= N ? PCV_OK : fail(PCV_EINVAL, "output range [%lld, %lld) outside [0, %lld]", (long long)begin,
                                         (long long)end, (long long)N);
     }
-    if (auto_dist_algo(m, n, workspace ? workspace_bytes : 0) == PCV_ALGO_FACTOR_TC)
+    if (auto_dist_algo(m, n, workspace ? workspace_bytes : 0) == PCV_ALGO_FACTOR_TC && !auto_expands(m, n, workspace_bytes))
         return distribution_tc(U, m, input_occ, begin, end, prob, amp, workspace, workspace_bytes, stream);
     return distribution_fp64(U, 1, m, input_occ, begin, end, prob, amp, true, workspace, workspace_bytes, stream);
 }

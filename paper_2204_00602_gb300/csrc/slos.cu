@@ -24,6 +24,7 @@
 // template bound), and with a batch a thread unranks its state once for
 // kGroup batch entries.
 
+#include <algorithm>
 #include <cmath>
 
 #include "expansion.cuh"
@@ -102,50 +103,17 @@ __global__ void __launch_bounds__(kThreads) expand_kernel(const __grid_constant_
 
     const int64_t i = a.lo + (int64_t)blockIdx.x * kThreads + threadIdx.x;
     if (i >= a.hi) return;
-    int l[KMAX];                               // sorted mode list of state i
-    {
-        I idx = (I)i;
-        int v = 0;
-#pragma unroll
-        for (int p = 0; p < KMAX; ++p) {
-            if (p >= k) break;
-            v = next_mode<I>(s_mc, w1, m, v, k - 1 - p, idx);
-            l[p] = v;
-        }
-    }
-    auto t = [&](int mode, int j) { return s_mc[(m - mode - 1) * w1 + j]; };
-    // |S_{m,k-1}| - 1 minus the terms of the list without position p: `pre`
-    // those before it, `suf` those after it (moved up by one)
-    I pre = (I)(a.prev_count - 1), suf = 0;
-#pragma unroll
-    for (int q = 1; q < KMAX; ++q)
-        if (q < k) suf += t(l[q], k - q);
     double2 acc[GROUP];
 #pragma unroll
     for (int j = 0; j < GROUP; ++j) acc[j] = make_double2(0.0, 0.0);
-    double sfac = 1.0;                         // sqrt(prod s!)
-    int mult = 0;
+    const double sfac = expand_state<KMAX, I>(s_mc, w1, m, k, (I)i, (I)a.prev_count, a.sqrtfact, [&](int r, I rk) {
 #pragma unroll
-    for (int p = 0; p < KMAX; ++p) {
-        if (p >= k) break;
-        const int r = l[p];
-        mult = (p > 0 && l[p > 0 ? p - 1 : 0] == r) ? mult + 1 : 1;
-        const int nxt = p + 1 < k ? l[p + 1 < KMAX ? p + 1 : p] : -1;
-        if (nxt != r) {                        // one term per occupied mode, at its last copy
-            const I rk = pre - suf;
-#pragma unroll
-            for (int j = 0; j < GROUP; ++j) {
-                const double2 u = s_u[j * m + r];
-                if (k == 1) acc[j] = u;
-                else cmac(acc[j], u, a.prev[s_parent[j] * a.prev_stride + rk]);
-            }
-            if (mult > 1) sfac *= a.sqrtfact[mult];
+        for (int j = 0; j < GROUP; ++j) {
+            const double2 u = s_u[j * m + r];
+            if (k == 1) acc[j] = u;
+            else cmac(acc[j], u, a.prev[s_parent[j] * a.prev_stride + rk]);
         }
-        if (p + 1 < k) {
-            pre -= t(r, k - 1 - p);
-            suf -= t(nxt, k - 1 - p);
-        }
-    }
+    });
 #pragma unroll
     for (int j = 0; j < GROUP; ++j) {
         const int b = b0 + j;
@@ -186,6 +154,74 @@ cudaError_t launch_group(const ExpandArgs& a, cudaStream_t s)
     if (a.k <= 4) return launch_one<4, GROUP, uint32_t>(a, s);
     if (a.k <= 8) return launch_one<8, GROUP, uint32_t>(a, s);
     return launch_one<16, GROUP, uint32_t>(a, s);
+}
+
+// Small problems: every level of a batch entry in one block, the levels below
+// the last in shared memory, one launch in all (the count table and the call's
+// status word included).  Level by level the launches bound such a call: m=6
+// n=3 took 65 us with the ten launches of the tensor-core plan, 31 with one
+// (most of it the host's call).
+struct SmallArgs {
+    const double2* U;          // [B][m][m]
+    int m, n;
+    int col[16];
+    uint32_t count[17];        // states of level k
+    uint32_t even;             // entries of the even levels' buffer
+    int64_t lo, hi;            // outputs, at [b][o - lo]
+    double2* amp;
+    double* prob;
+    int64_t out_stride;
+    double norm_t;
+    int64_t* status;           // two words zeroed, or null
+    double sqrtfact[17];
+};
+
+template <int KMAX>
+__global__ void __launch_bounds__(kThreads) expand_small_kernel(const __grid_constant__ SmallArgs a)
+{
+    extern __shared__ double2 s_lev[];         // even levels, odd levels, U's columns [n][m], the counts
+    const int m = a.m, n = a.n, w1 = n + 1, b = blockIdx.x;
+    uint32_t odd = 1;
+    for (int k = 1; k < n; k += 2) odd = max(odd, a.count[k]);
+    double2* s_u = s_lev + a.even + odd;
+    uint32_t* s_mc = (uint32_t*)(s_u + n * m);
+    if (a.status && b == 0 && threadIdx.x < 2) a.status[threadIdx.x] = 0;
+    for (int q = threadIdx.x; q < n * m; q += kThreads)
+        s_u[q] = a.U[((size_t)b * m + q % m) * m + a.col[q / m]];
+    for (int w = threadIdx.x; w <= m; w += kThreads) {
+        uint64_t c = 1;
+        s_mc[w * w1] = 1;
+        for (int j = 1; j <= n; ++j) {
+            c = c * (uint64_t)(w + j - 1) / (uint64_t)j;
+            s_mc[w * w1 + j] = (uint32_t)c;
+        }
+    }
+    __syncthreads();
+    for (int k = 1; k <= n; ++k) {
+        const bool last = k == n;
+        const double2* prev = s_lev + (k & 1 ? 0 : a.even);
+        double2* cur = s_lev + (k & 1 ? a.even : 0);
+        const double2* u = s_u + (k - 1) * m;
+        const int64_t hi = last ? a.hi : (int64_t)a.count[k];
+        for (int64_t i = (last ? a.lo : 0) + threadIdx.x; i < hi; i += kThreads) {
+            double2 acc = make_double2(0.0, 0.0);
+            const double sf = expand_state<KMAX, uint32_t>(s_mc, w1, m, k, (uint32_t)i, a.count[k - 1], a.sqrtfact,
+                                                           [&](int r, uint32_t rk) {
+                                                               if (k == 1) acc = u[r];
+                                                               else cmac(acc, u[r], prev[rk]);
+                                                           });
+            if (!last) {
+                cur[i] = acc;
+                continue;
+            }
+            const double sc = sf * a.norm_t;
+            const double2 v = make_double2(acc.x * sc, acc.y * sc);
+            const size_t o = (size_t)b * a.out_stride + (i - a.lo);
+            if (a.amp) a.amp[o] = v;
+            if (a.prob) a.prob[o] = fma(v.x, v.x, v.y * v.y);
+        }
+        __syncthreads();
+    }
 }
 
 int64_t mset_s(int w, int k)
@@ -250,6 +286,33 @@ cudaError_t build_cum_table(const int64_t* mc, int m, int kmax, int64_t* cum, cu
     return cudaGetLastError();
 }
 
+namespace {
+
+// Shared memory of expand_small_kernel, or 0 where the launches per level are
+// the better form: one SM would need more time for the multiply-adds (2 cycles
+// each) than n launches take (about 4,800 cycles each).
+size_t small_smem(int m, int n, SmallArgs* a)
+{
+    if (n < 1 || n > 16 || m > 256) return 0;
+    double terms = 0.0;
+    int64_t even = 1, odd = 1;
+    for (int k = 0; k <= n; ++k) {
+        const int64_t c = mset_s(m, k);
+        if (c < 0 || c > 100000) return 0;
+        a->count[k] = (uint32_t)c;
+        if (k < n) {
+            terms += (double)m * (double)c;
+            (k & 1 ? odd : even) = std::max(k & 1 ? odd : even, c);
+        }
+    }
+    a->even = (uint32_t)even;
+    if (2.0 * terms > 4800.0 * n) return 0;
+    const size_t b = (size_t)(even + odd + (int64_t)n * m) * sizeof(double2) + (size_t)(m + 1) * (n + 1) * sizeof(uint32_t);
+    return b <= 100 * 1024 ? b : 0;
+}
+
+}  // namespace
+
 // Workspace: the count table, then two level buffers of the largest
 // intermediate level per batch entry.
 int64_t slos_workspace(int B, int m, int n)
@@ -266,9 +329,41 @@ int64_t slos_workspace(int B, int m, int n)
 }
 
 cudaError_t launch_slos(const Plan& p, int B, const double2* U, int64_t lo, int64_t hi, double* prob, double2* amp,
-                        void* ws, cudaStream_t s)
+                        void* ws, void* status, cudaStream_t s)
 {
     const int m = p.m, n = p.n;
+    if (!amp && !prob) return cudaErrorInvalidValue;
+    SmallArgs sm;
+    if (const size_t smem = small_smem(m, n, &sm)) {
+        ExpandArgs d;
+        expand_defaults(&d);
+        sm.U = U;
+        sm.m = m;
+        sm.n = n;
+        for (int j = 0; j < n; ++j) sm.col[j] = p.cols[j];
+        sm.lo = lo;
+        sm.hi = hi;
+        sm.amp = amp;
+        sm.prob = prob;
+        sm.out_stride = hi - lo;
+        sm.norm_t = p.norm_t;
+        sm.status = (int64_t*)status;
+        for (int j = 0; j <= 16; ++j) sm.sqrtfact[j] = d.sqrtfact[j];
+        auto go = [&](auto kernel) {
+            cudaError_t e = cudaSuccess;
+            if (smem > 48 * 1024)
+                e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
+            kernel<<<B, kThreads, smem, s>>>(sm);
+            note_launches(1);
+            return cudaGetLastError();
+        };
+        return n <= 4 ? go(expand_small_kernel<4>) : n <= 8 ? go(expand_small_kernel<8>) : go(expand_small_kernel<16>);
+    }
+    if (status) {
+        const cudaError_t e = cudaMemsetAsync(status, 0, 16, s);
+        if (e != cudaSuccess) return e;
+    }
     int64_t half = 1;
     for (int k = 0; k < n; ++k) {
         const int64_t c = mset_s(m, k);
@@ -279,7 +374,6 @@ cudaError_t launch_slos(const Plan& p, int B, const double2* U, int64_t lo, int6
     double2* buf[2];
     buf[0] = (double2*)w;               w += al256((size_t)B * half * sizeof(double2));
     buf[1] = (double2*)w;
-    if (!amp && !prob) return cudaErrorInvalidValue;
     cudaError_t e = build_multiset_table(mc, m, n, s);
     if (e != cudaSuccess) return e;
     ExpandArgs a;
