@@ -3,10 +3,11 @@
 One step = every amplitude and probability of the 20,030,010 outputs of a
 Haar-random 20x20 unitary with photons in modes 0..9 (Eq. eqperm, Sec. 4.2),
 computed by the CUDA library through its C ABI entry point pcv_distribution.
-At this size that call takes the factorised Glynn sum with its complex
-products on the tensor cores as exact integer digit products (--algo auto,
-the default, = factor_tc here); --algo factor runs the same sum with FP64
-products, which the JSON line also reports as context.
+At this size that call expands the state photon by photon, its sums in fixed
+point on the integer pipe (--algo auto, the default, = slos here); --algo
+factor_tc runs the factorised Glynn sum with its complex products on the
+tensor cores as exact integer digit products, --algo factor the same sum with
+FP64 products.  The JSON line reports both as context.
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
                     [--algo auto|factor_tc|factor|group|slos]
@@ -95,14 +96,13 @@ def parse():
     return args
 
 
-def measured_bf16_peak() -> float:
-    """Dense BF16 TFLOP/s measured on the GB300s (burst), else the
-    recipe's fallback figure."""
+def measured_peak(key: str, fallback: float) -> float:
+    """A rate measured on GB300 (MEASURED_PEAKS.json), else the fallback figure."""
     try:
         with open(os.path.join(os.path.dirname(os.path.abspath(__file__)), "MEASURED_PEAKS.json")) as f:
-            return float(json.load(f)["bf16_tflops"])
+            return float(json.load(f)[key])
     except Exception:
-        return 1900.0
+        return fallback
 
 
 def rank_unitary_seed(rank: int) -> int:
@@ -239,7 +239,11 @@ def run_ours(args):
     # the path pcv_distribution takes with this workspace (the roofline's kernel)
     kind = args.algo
     if args.algo == "auto":
-        kind = "factor_tc" if abi.pcv_distribution_auto_algo(M, N_PH, ws_bytes) == pcv.PCV_ALGO_FACTOR_TC else "factor"
+        if ws_bytes >= abi.pcv_distribution_slos_workspace(1, M, N_PH) + 256:
+            kind = "slos"
+        else:
+            tc = abi.pcv_distribution_auto_algo(M, N_PH, ws_bytes) == pcv.PCV_ALGO_FACTOR_TC
+            kind = "factor_tc" if tc else "factor"
     flush = torch.empty(L2_FLUSH_BYTES // 4, dtype=torch.float32, device=dev)
 
     def dist_call(Uc, out):
@@ -388,26 +392,36 @@ def run_ours(args):
         # multisets of size k over M modes with d distinct modes: C(M, d) C(k-1, d-1)
         flops_per_call = sum(8 * d * math.comb(M, d) * math.comb(k - 1, d - 1)
                              for k in range(1, N_PH + 1) for d in range(1, min(k, M) + 1))
-        kname = "slos_level_kernel (state expansion)"
-        launches_per_call = N_PH
+        kname = "expand_fixed_kernel (state expansion, sums of 30-bit halves on the integer pipe)"
+        launches_per_call = N_PH + 2
     achieved = flops_per_call * calls / (ms * 1e-3) / 1e12 if ms > 0 and flops_per_call else None
     peak_src = f"derived: {sms} SMs x 2 DFMA/clk x 2 flop x {sm_max:.0f} MHz (FP64 ALU)"
     bound = "alu"
     if kind == "factor_tc":
-        peak_tflops, bound = measured_bf16_peak(), "tensor"
+        peak_tflops, bound = measured_peak("bf16_tflops", 1900.0), "tensor"
         peak_src = "MEASURED_PEAKS.json bf16_tflops (burst cuBLAS bf16 GEMM, measured)"
+    unit, fp64_equivalent = "TFLOP/s", None
+    if kind == "slos":
+        # the sums leave the FP64 pipe, so what remains as a roof is memory: results written once, every
+        # level below the last written and read once
+        fp64_equivalent = {"tflops": achieved, "frac_of_fp64_peak": achieved / peak_tflops if achieved else None,
+                           "note": "8 flops per state and occupied mode; computed as integer multiply-adds"}
+        moved = 24 * (hi - lo) + 32 * sum(pcv.num_outputs(M, k) for k in range(1, N_PH))
+        achieved = moved * calls / (ms * 1e-3) / 1e9 if ms > 0 else None
+        peak_tflops, bound, unit = measured_peak("hbm_gbs", 6800.0), "hbm", "GB/s"
+        peak_src = "MEASURED_PEAKS.json hbm_gbs (STREAM-style copy, measured)"
     traffic, traffic_note = recorded_traffic(kind, M, N_PH)
-    roof = {"bound": bound, "kernel": kname, "achieved": achieved, "peak": peak_tflops, "unit": "TFLOP/s",
+    roof = {"bound": bound, "kernel": kname, "achieved": achieved, "peak": peak_tflops, "unit": unit,
             "frac": achieved / peak_tflops if achieved else None,
             "peak_source": peak_src,
             "fp64_probe_tflops": probe_tflops,
             "traffic": traffic, "traffic_source": traffic_note,
-            "launches_per_step": launches_per_call,
+            "launches_per_step": launches_per_call, "fp64_equivalent": fp64_equivalent,
             "stage_ms_per_step": {k: (v[0] / v[1] if v[1] else None) for k, v in stages.items()}}
 
     # context: the FP64 factorised path (its product kernel against the FP64 peak)
     fp64_ctx = None
-    if kind == "factor_tc" and not args.no_e2e:
+    if args.algo in ("auto", "factor_tc") and kind != "factor" and not args.no_e2e:
         ws_f = pcv.workspace(pcv.distribution_workspace_bytes(M, N_PH, pcv.PCV_ALGO_FACTOR), dev)
         for _ in range(2):
             pcv.distribution(U, t, algo=pcv.PCV_ALGO_FACTOR, ws=ws_f, out=(prob, amp))
@@ -433,6 +447,32 @@ def run_ours(args):
                     "product_kernel_tflops": ach, "fp64_peak_tflops": fp64_peak,
                     "frac_of_fp64_peak": ach / fp64_peak if ach else None}
         del ws_f
+
+    # context: the factorised sum with its products on the tensor cores
+    tc_ctx = None
+    if args.algo == "auto" and kind == "slos" and not args.no_e2e:
+        ws_t = pcv.workspace(pcv.distribution_workspace_bytes(M, N_PH, pcv.PCV_ALGO_FACTOR_TC), dev)
+        for _ in range(2):
+            pcv.distribution(U, t, algo=pcv.PCV_ALGO_FACTOR_TC, ws=ws_t, out=(prob, amp))
+        torch.cuda.synchronize()
+        abi.pcv_profile_read()
+        abi.pcv_profile_enable(True)
+        tsteps = min(args.steps, 100)                     # ~2.4 ms each
+        t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        t0.record(stream)
+        for _ in range(tsteps):
+            pcv.distribution(U, t, algo=pcv.PCV_ALGO_FACTOR_TC, ws=ws_t, out=(prob, amp))
+        t1.record(stream)
+        torch.cuda.synchronize()
+        abi.pcv_profile_enable(False)
+        abi.pcv_distribution_status(ws_t, stream.cuda_stream)
+        pms, pcalls = abi.pcv_profile_read()["dist_products"]
+        ms_t = t0.elapsed_time(t1) / tsteps
+        ach = Ntot * (2 ** (N_PH - 1)) * 3 * 36 * 2 * pcalls / (pms * 1e-3) / 1e12 if pms > 0 else None
+        tc_ctx = {"algo": "factorised Glynn, exact-digit BF16 products on the tensor cores (tc_product_kernel)",
+                  "ms_per_step": ms_t, "value": Ntot / (ms_t * 1e-3), "unit": "amplitudes/s",
+                  "product_kernel_tflops": ach, "frac_of_bf16_peak": ach / measured_peak("bf16_tflops", 1900.0) if ach else None}
+        del ws_t
 
     # context: the same workload by photon-by-photon state expansion (not the Glynn path)
     alt = None
@@ -463,7 +503,8 @@ def run_ours(args):
         "scaling": "strong" if args.shard else "weak",
         "vs_baseline": None,
         "dtype": "f64",
-        "dtype_note": None if kind != "factor_tc" else
+        "dtype_note": "FP64 inputs and results; the sums over a level run as exact fixed-point sums of 57- by 59-bit "
+        "products" if kind == "slos" else None if kind != "factor_tc" else
         "FP64 tables, scaling and results; the complex products run as exact integer digit products "
         "on the bf16 tensor cores (no rounding; agreement with the FP64 path to 1e-11)",
         "data": "synthetic",
@@ -474,6 +515,7 @@ def run_ours(args):
         "e2e": e2e, "gpu_launches": launches, "roofline": roof, "cpu_baseline": cpu, "clocks": clk,
         "state_expansion": alt,
         "fp64_factor_path": fp64_ctx,
+        "factor_tc_path": tc_ctx,
         "wall_s_timed_region": wall,
     }
     print(json.dumps(line), flush=True)

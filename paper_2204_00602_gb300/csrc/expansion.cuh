@@ -52,6 +52,14 @@ struct ExpandArgs {
 void expand_defaults(ExpandArgs* a);
 cudaError_t launch_expand(const ExpandArgs& a, cudaStream_t s);
 
+// The same levels of one unitary in fixed point (expansion_fixed.cu); count[k]:
+// the states of level k, buf: two levels, header: 256 bytes.
+constexpr int64_t kFixedMinStates = 200000;
+bool expand_fixed_applies(int m, int n, int64_t largest, int64_t states);
+cudaError_t launch_expand_fixed(const Plan& p, const double2* U, const int64_t* count, int64_t lo, int64_t hi,
+                                double* prob, double2* amp, const int64_t* mc, void* header, double2* const* buf,
+                                int64_t* status, cudaStream_t s);
+
 #ifdef __CUDACC__
 // Sorted mode list of index i of S_{m,k}, from the shared or global table t
 // (row length w1): t[a * w1 + j] = MC(a, j).
@@ -66,9 +74,9 @@ __device__ __forceinline__ int next_mode(const I* t, int w1, int m, int v, int r
     }
 }
 
-// State i of S_{m,k} (count table mc, row length w1): term(r, rank) for every
-// occupied mode r, rank that of the state without one photon of r among the
-// prev_n states of S_{m,k-1}.  Returns sqrt(prod s!).
+// State i of S_{m,k} (count table mc, row length w1): term(r, rank, photons) for
+// every occupied mode r, rank that of the state without one photon of r among
+// the prev_n states of S_{m,k-1}.  Returns sqrt(prod s!) (1 without the table).
 template <int KMAX, typename I, typename F>
 __device__ __forceinline__ double expand_state(const I* mc, int w1, int m, int k, I i, I prev_n, const double* sqrtfact,
                                                F&& term)
@@ -99,8 +107,8 @@ __device__ __forceinline__ double expand_state(const I* mc, int w1, int m, int k
         mult = (p > 0 && l[p > 0 ? p - 1 : 0] == r) ? mult + 1 : 1;
         const int nxt = p + 1 < k ? l[p + 1 < KMAX ? p + 1 : p] : -1;
         if (nxt != r) {                        // one term per occupied mode, at its last copy
-            term(r, (I)(pre - suf));
-            if (mult > 1) sfac *= sqrtfact[mult];
+            term(r, (I)(pre - suf), mult);
+            if (mult > 1 && sqrtfact) sfac *= sqrtfact[mult];
         }
         if (p + 1 < k) {
             pre -= t(r, k - 1 - p);

@@ -1,0 +1,282 @@
+// State expansion of one large distribution on the integer pipe (the sums of
+// slos.cu, n <= 12).
+//
+// What bounds it: the sums of slos.cu are bound by the FP64 pipe, which takes a
+// warp instruction per 16 cycles and SM: 64 cycles for the four DFMA of a
+// complex term.  Sixteen wide integer multiply-adds of 30-bit halves give the
+// same term in about 16, without any rounding inside a sum.  m=20 n=10: 2203 to
+// 1421 us (relative error against 64 bits 7.6e-16 to 6.3e-16), m=12 n=12: 294 to
+// 265 us (1.2e-15 to 9.2e-16).
+//
+// Numbers.  The kernels carry B_k(s) of slos.cu (not C_k: all B_k(s) are of one
+// size, so one scale serves a level) as X = B_k(s) 2^S_k, components at most
+// 2^59, split as h 2^30 + l with |l| <= 2^29.  The factors U[r][c] sqrt(j), j the
+// photons in mode r, are fixed-point numbers of scale 2^(57 - e), 2^e at least
+// the 2-norm of column c.  With M the largest component of level k-1 and
+// sum_r sqrt(s_r) |U_r| <= sqrt(k) |U|, a component of level k is below
+// 2^57 M sqrt(2 k) before it is shifted back to 59 bits: the shift follows from
+// M, which every level leaves in the header, so nothing can overflow and at most
+// 4 of the 59 bits stay unused.  Sums of half products: with 12 terms the cross
+// sum is below 24 2^58 + 2^59 < 2^63, the others are smaller.
+//
+// A level rounds once, to 2^-53 of the level's typical amplitude or less.  The
+// error is one of absolute size, as that of Glynn's sum, so inputs whose outputs
+// differ by many orders of magnitude by construction keep the FP64 sums: where a
+// column has an entry that is neither zero nor at least 2^-20 of its norm, or a
+// norm outside 2^-40 .. 2^40, or an entry that is not finite, the same launches
+// run the FP64 form of slos.cu (the first kernel decides, on the device).
+
+#include <algorithm>
+#include <cmath>
+
+#include "expansion.cuh"
+
+namespace pcv {
+namespace {
+
+constexpr int kThreads = 256;
+constexpr int kMaxN = 12;
+constexpr int kUBits = 57, kXBits = 59;
+constexpr unsigned kBlocks = 152 * 8;          // a block takes several tiles: its table of factors is built once
+
+struct FixedHeader {
+    int fp64;                  // the FP64 form runs
+    int colexp[kMaxN];         // e of photon j's column
+    unsigned top[kMaxN + 1];   // level k: max |component| >> 29
+    int scale[kMaxN + 1];      // S_k
+};
+
+struct FixedArgs {
+    const double2* U;          // [m][m]
+    int m, n, k;
+    int col[kMaxN];
+    const int64_t* mc;         // [m + 1][n + 1]
+    int64_t lo, hi;            // states written
+    uint32_t prev_count;
+    const int4* prev;
+    int4* cur;                 // or null: the last level
+    double2* amp;              // last level, at [i - lo]
+    double* prob;
+    double norm_t;
+    FixedHeader* hdr;
+    int64_t* status;           // setup: two words zeroed, or null
+    double sqrtfact[kMaxN + 1];
+};
+
+// One warp per photon: its column's norm, and whether the fixed-point form applies.
+__global__ void fixed_setup_kernel(const __grid_constant__ FixedArgs a)
+{
+    const int j = threadIdx.x / 32, lane = threadIdx.x & 31;
+    __shared__ int s_bad[kMaxN];
+    double sum = 0.0, least = INFINITY;
+    for (int r = lane; r < a.m; r += 32) {
+        const double2 u = a.U[(size_t)r * a.m + a.col[j]];
+        sum = fma(u.x, u.x, fma(u.y, u.y, sum));
+        const double c = fmax(fabs(u.x), fabs(u.y));
+        if (c > 0.0) least = fmin(least, c);
+    }
+    for (int d = 16; d; d >>= 1) {
+        sum += __shfl_xor_sync(0xffffffffu, sum, d);
+        least = fmin(least, __shfl_xor_sync(0xffffffffu, least, d));
+    }
+    const double norm = sqrt(sum);
+    // written so that a NaN fails
+    const bool ok = norm >= 0x1p-40 && norm <= 0x1p40 && least >= 0x1p-20 * norm;
+    if (lane == 0) {
+        s_bad[j] = !ok;
+        int e = 0;
+        if (ok) {
+            frexp(norm * (1.0 - 0x1p-20), &e);     // a norm of 1 but for rounding counts as 1
+        }
+        a.hdr->colexp[j] = e;
+    }
+    if (threadIdx.x <= kMaxN) a.hdr->top[threadIdx.x] = 0;
+    if (a.status && threadIdx.x < 2) a.status[threadIdx.x] = 0;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int bad = 0;
+        for (int q = 0; q < a.n; ++q) bad |= s_bad[q];
+        a.hdr->fp64 = bad;
+    }
+}
+
+__device__ __forceinline__ void wide_mad(long long& acc, int x, int y)
+{
+    asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc) : "r"(x), "r"(y));
+}
+
+__device__ __forceinline__ void split30(long long x, int& h, int& l)
+{
+    l = (int)((uint32_t)x << 2) >> 2;
+    h = (int)((x - l) >> 30);
+}
+
+struct Sum30 {                                  // hh 2^60 + hl 2^30 + ll
+    long long hh = 0, hl = 0, ll = 0;
+    __device__ __forceinline__ void add(int xh, int xl, int yh, int yl)
+    {
+        wide_mad(hh, xh, yh);
+        wide_mad(hl, xh, yl);
+        wide_mad(hl, xl, yh);
+        wide_mad(ll, xl, yl);
+    }
+    // the sum / 2^(30 + sh), rounded, 0 < sh <= 30
+    __device__ __forceinline__ long long value(int sh) const
+    {
+        const long long v = hl + (ll >> 30);
+        return (hh << (30 - sh)) + ((v + (1ll << (sh - 1))) >> sh);
+    }
+};
+
+template <int KMAX>
+__global__ void __launch_bounds__(kThreads) expand_fixed_kernel(const __grid_constant__ FixedArgs a)
+{
+    extern __shared__ int4 s_f[];               // [m][k] factors (FP64 form: [m] entries of U), then the count table
+    const int m = a.m, k = a.k, w1 = k + 1;
+    uint32_t* s_mc = (uint32_t*)(s_f + m * k);
+    __shared__ unsigned s_top;
+    const bool last = !a.cur, fp64 = a.hdr->fp64;
+    for (int q = threadIdx.x; q < (m + 1) * w1; q += kThreads)
+        s_mc[q] = (uint32_t)a.mc[(q / w1) * (a.n + 1) + q % w1];
+    if (threadIdx.x == 0) s_top = 0;
+
+    if (fp64) {
+        double2* s_u = (double2*)s_f;
+        const double2* prev = (const double2*)a.prev;
+        for (int r = threadIdx.x; r < m; r += kThreads) s_u[r] = a.U[(size_t)r * m + a.col[k - 1]];
+        __syncthreads();
+        for (int64_t i = a.lo + (int64_t)blockIdx.x * kThreads + threadIdx.x; i < a.hi; i += (int64_t)gridDim.x * kThreads) {
+            double2 acc = make_double2(0.0, 0.0);
+            const double sf = expand_state<KMAX, uint32_t>(s_mc, w1, m, k, (uint32_t)i, a.prev_count, a.sqrtfact,
+                                                           [&](int r, uint32_t rk, int) {
+                                                               if (k == 1) acc = s_u[r];
+                                                               else cmac(acc, s_u[r], prev[rk]);
+                                                           });
+            if (!last) {
+                ((double2*)a.cur)[i] = acc;
+                continue;
+            }
+            const double sc = sf * a.norm_t;
+            const double2 v = make_double2(acc.x * sc, acc.y * sc);
+            if (a.amp) a.amp[i - a.lo] = v;
+            if (a.prob) a.prob[i - a.lo] = fma(v.x, v.x, v.y * v.y);
+        }
+        return;
+    }
+
+    const int e = a.hdr->colexp[k - 1];
+    for (int q = threadIdx.x; q < m * k; q += kThreads) {
+        const double2 u = a.U[(size_t)(q / k) * m + a.col[k - 1]];
+        const double f = ldexp(sqrt((double)(q % k + 1)), kUBits - e);
+        int4 y;
+        split30(__double2ll_rn(u.x * f), y.x, y.y);
+        split30(__double2ll_rn(u.y * f), y.z, y.w);
+        s_f[q] = y;
+    }
+    // The shift back to kXBits bits; the last level keeps three bits more, as it is not multiplied again.
+    int sh = 0, scale = kUBits - e;
+    if (k > 1) {
+        const double bound = ((double)a.hdr->top[k - 1] + 1.0) * sqrt(2.0 * k) * (1.0 + 0x1p-18);   // of M sqrt(2k), in 2^29
+        sh = min(max(ilogb(bound) + 1 + 29 + kUBits - kXBits - 30 - (last ? 3 : 0), 1), 30);
+        scale += a.hdr->scale[k - 1] - 30 - sh;
+    }
+    if (!last && blockIdx.x == 0 && threadIdx.x == 0) a.hdr->scale[k] = scale;
+    const double back = ldexp(a.norm_t, -scale);
+    __syncthreads();
+
+    unsigned top = 0;
+    for (int64_t i = a.lo + (int64_t)blockIdx.x * kThreads + threadIdx.x; i < a.hi; i += (int64_t)gridDim.x * kThreads) {
+        Sum30 re, im;
+        long long x, y;
+        if (k == 1) {
+            const int4 u = s_f[i];
+            x = ((long long)u.x << 30) + u.y;
+            y = ((long long)u.z << 30) + u.w;
+        } else {
+            expand_state<KMAX, uint32_t>(s_mc, w1, m, k, (uint32_t)i, a.prev_count, nullptr,
+                                         [&](int r, uint32_t rk, int mult) {
+                                             const int4 u = s_f[r * k + mult - 1], c = a.prev[rk];
+                                             re.add(u.x, u.y, c.x, c.y);
+                                             re.add(-u.z, -u.w, c.z, c.w);
+                                             im.add(u.x, u.y, c.z, c.w);
+                                             im.add(u.z, u.w, c.x, c.y);
+                                         });
+            x = re.value(sh);
+            y = im.value(sh);
+        }
+        if (!last) {
+            int4 c;
+            split30(x, c.x, c.y);
+            split30(y, c.z, c.w);
+            a.cur[i] = c;
+            top = max(top, (unsigned)max(llabs(x) >> 29, llabs(y) >> 29));
+            continue;
+        }
+        const double2 v = make_double2((double)x * back, (double)y * back);
+        if (a.amp) a.amp[i - a.lo] = v;
+        if (a.prob) a.prob[i - a.lo] = fma(v.x, v.x, v.y * v.y);
+    }
+    if (last) return;
+    top = __reduce_max_sync(0xffffffffu, top);
+    if ((threadIdx.x & 31) == 0) atomicMax(&s_top, top);
+    __syncthreads();
+    if (threadIdx.x == 0) atomicMax(&a.hdr->top[k], s_top);
+}
+
+template <int KMAX>
+cudaError_t launch_level(const FixedArgs& a, cudaStream_t s)
+{
+    const size_t smem = (size_t)a.m * a.k * sizeof(int4) + (size_t)(a.m + 1) * (a.k + 1) * sizeof(uint32_t);
+    const int64_t tiles = (a.hi - a.lo + kThreads - 1) / kThreads;
+    expand_fixed_kernel<KMAX><<<(unsigned)std::min<int64_t>(tiles, kBlocks), kThreads, smem, s>>>(a);
+    note_launches(1);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+// By the size of the problem alone, so that a range of outputs takes the form
+// of the whole.  states: of all levels; tables of factors and counts up to 44 KB.
+bool expand_fixed_applies(int m, int n, int64_t largest, int64_t states)
+{
+    return n >= 2 && n <= kMaxN && m * n <= 2048 && largest <= (int64_t)UINT32_MAX && states >= kFixedMinStates;
+}
+
+static_assert(sizeof(FixedHeader) <= 256, "the header fits the table that the FP64 form leaves unused");
+
+cudaError_t launch_expand_fixed(const Plan& p, const double2* U, const int64_t* count, int64_t lo, int64_t hi,
+                                double* prob, double2* amp, const int64_t* mc, void* header, double2* const* buf,
+                                int64_t* status, cudaStream_t s)
+{
+    ExpandArgs d;
+    expand_defaults(&d);
+    FixedArgs a{};
+    a.U = U;
+    a.m = p.m;
+    a.n = p.n;
+    a.mc = mc;
+    a.norm_t = p.norm_t;
+    a.hdr = (FixedHeader*)header;
+    a.status = status;
+    for (int j = 0; j < p.n; ++j) a.col[j] = p.cols[j];
+    for (int j = 0; j <= kMaxN; ++j) a.sqrtfact[j] = d.sqrtfact[j];
+    fixed_setup_kernel<<<1, 32 * p.n, 0, s>>>(a);
+    note_launches(1);
+    cudaError_t e = cudaGetLastError();
+    for (int k = 1; k <= p.n && e == cudaSuccess; ++k) {
+        const bool last = k == p.n;
+        a.k = k;
+        a.lo = last ? lo : 0;
+        a.hi = last ? hi : count[k];
+        if (a.hi <= a.lo) break;
+        a.prev_count = (uint32_t)count[k - 1];
+        a.prev = (const int4*)buf[(k - 1) & 1];
+        a.cur = last ? nullptr : (int4*)buf[k & 1];
+        a.amp = last ? amp : nullptr;
+        a.prob = last ? prob : nullptr;
+        e = k <= 4 ? launch_level<4>(a, s) : k <= 8 ? launch_level<8>(a, s) : launch_level<kMaxN>(a, s);
+    }
+    return e;
+}
+
+}  // namespace pcv

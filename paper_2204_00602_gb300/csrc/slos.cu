@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(kThreads) expand_kernel(const __grid_constant_
     double2 acc[GROUP];
 #pragma unroll
     for (int j = 0; j < GROUP; ++j) acc[j] = make_double2(0.0, 0.0);
-    const double sfac = expand_state<KMAX, I>(s_mc, w1, m, k, (I)i, (I)a.prev_count, a.sqrtfact, [&](int r, I rk) {
+    const double sfac = expand_state<KMAX, I>(s_mc, w1, m, k, (I)i, (I)a.prev_count, a.sqrtfact, [&](int r, I rk, int) {
 #pragma unroll
         for (int j = 0; j < GROUP; ++j) {
             const double2 u = s_u[j * m + r];
@@ -206,7 +206,7 @@ __global__ void __launch_bounds__(kThreads) expand_small_kernel(const __grid_con
         for (int64_t i = (last ? a.lo : 0) + threadIdx.x; i < hi; i += kThreads) {
             double2 acc = make_double2(0.0, 0.0);
             const double sf = expand_state<KMAX, uint32_t>(s_mc, w1, m, k, (uint32_t)i, a.count[k - 1], a.sqrtfact,
-                                                           [&](int r, uint32_t rk) {
+                                                           [&](int r, uint32_t rk, int) {
                                                                if (k == 1) acc = u[r];
                                                                else cmac(acc, u[r], prev[rk]);
                                                            });
@@ -360,22 +360,27 @@ cudaError_t launch_slos(const Plan& p, int B, const double2* U, int64_t lo, int6
         };
         return n <= 4 ? go(expand_small_kernel<4>) : n <= 8 ? go(expand_small_kernel<8>) : go(expand_small_kernel<16>);
     }
-    if (status) {
+    int64_t half = 1, states = 0;
+    int64_t count[PCV_MAX_PHOTONS + 1];
+    for (int k = 0; k <= n; ++k) {
+        count[k] = mset_s(m, k);
+        if (k < n) half = std::max(half, count[k]);
+        states += count[k] < kFixedMinStates ? count[k] : kFixedMinStates;
+    }
+    const bool fixed = B == 1 && hi > lo && expand_fixed_applies(m, n, std::max(half, count[n]), states);
+    if (status && !fixed) {
         const cudaError_t e = cudaMemsetAsync(status, 0, 16, s);
         if (e != cudaSuccess) return e;
     }
-    int64_t half = 1;
-    for (int k = 0; k < n; ++k) {
-        const int64_t c = mset_s(m, k);
-        half = c > half ? c : half;
-    }
     char* w = (char*)ws;
-    int64_t* mc = (int64_t*)w;          w += 2 * al256((size_t)(m + 1) * (n + 1) * sizeof(int64_t));
+    int64_t* mc = (int64_t*)w;          w += al256((size_t)(m + 1) * (n + 1) * sizeof(int64_t));
+    void* header = w;                   w += al256((size_t)(m + 1) * (n + 1) * sizeof(int64_t));
     double2* buf[2];
     buf[0] = (double2*)w;               w += al256((size_t)B * half * sizeof(double2));
     buf[1] = (double2*)w;
     cudaError_t e = build_multiset_table(mc, m, n, s);
     if (e != cudaSuccess) return e;
+    if (fixed) return launch_expand_fixed(p, U, count, lo, hi, prob, amp, mc, header, buf, (int64_t*)status, s);
     ExpandArgs a;
     expand_defaults(&a);
     a.source = kExpandBatch;
@@ -390,10 +395,10 @@ cudaError_t launch_slos(const Plan& p, int B, const double2* U, int64_t lo, int6
         const bool last = k == n;
         a.k = k;
         a.col[0] = p.cols[k - 1];
-        a.count = mset_s(m, k);
+        a.count = count[k];
         a.lo = last ? lo : 0;
         a.hi = last ? hi : a.count;
-        a.prev_count = mset_s(m, k - 1);
+        a.prev_count = count[k - 1];
         a.prev = buf[(k - 1) & 1];
         a.cur = last ? nullptr : buf[k & 1];
         a.amp = last ? amp : nullptr;
