@@ -87,7 +87,8 @@ __device__ __forceinline__ double expand_state(const I* mc, int w1, int m, int k
 #pragma unroll
         for (int p = 0; p < KMAX; ++p) {
             if (p >= k) break;
-            v = next_mode<I>(mc, w1, m, v, k - 1 - p, i);
+            // below the last position every mode counts for one state
+            v = p + 1 < k ? next_mode<I>(mc, w1, m, v, k - 1 - p, i) : v + (int)i;
             l[p] = v;
         }
     }
