@@ -37,7 +37,7 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kMaxN = 12;
 constexpr int kUBits = 57, kXBits = 59;
-constexpr unsigned kBlocks = 152 * 8;          // a block takes several tiles: its table of factors is built once
+constexpr unsigned kBlocks = 152 * 3;          // one wave: a block takes several tiles, its table of factors is built once
 
 struct FixedHeader {
     int fp64;                  // the FP64 form runs
@@ -52,6 +52,7 @@ struct FixedArgs {
     int col[kMaxN];
     const int64_t* mc;         // [m + 1][n + 1]
     int64_t lo, hi;            // states written
+    int steps;                 // of 32 states in a warp's run (K >= 5)
     uint32_t prev_count;
     const int4* prev;
     int4* cur;                 // or null: the last level
@@ -128,42 +129,48 @@ struct Sum30 {                                  // hh 2^60 + hl 2^30 + ll
     }
 };
 
-template <int KMAX>
-__global__ void __launch_bounds__(kThreads) expand_fixed_kernel(const __grid_constant__ FixedArgs a)
+// The FP64 form of a level: the sums of slos.cu.  Not inlined, so that it costs
+// the fixed-point form no registers.
+__device__ __noinline__ void fp64_level(const FixedArgs& a, double2* s_u, const uint32_t* s_mc)
 {
-    extern __shared__ int4 s_f[];               // [m][k] factors (FP64 form: [m] entries of U), then the count table
-    const int m = a.m, k = a.k, w1 = k + 1;
-    uint32_t* s_mc = (uint32_t*)(s_f + m * k);
-    __shared__ unsigned s_top;
-    const bool last = !a.cur, fp64 = a.hdr->fp64;
+    const int m = a.m, k = a.k;
+    const double2* prev = (const double2*)a.prev;
+    for (int r = threadIdx.x; r < m; r += kThreads) s_u[r] = a.U[(size_t)r * m + a.col[k - 1]];
+    __syncthreads();
+    for (int64_t i = a.lo + (int64_t)blockIdx.x * kThreads + threadIdx.x; i < a.hi; i += (int64_t)gridDim.x * kThreads) {
+        double2 acc = make_double2(0.0, 0.0);
+        const double sf = expand_state<kMaxN, uint32_t>(s_mc, k + 1, m, k, (uint32_t)i, a.prev_count, a.sqrtfact,
+                                                        [&](int r, uint32_t rk, int) {
+                                                            if (k == 1) acc = s_u[r];
+                                                            else cmac(acc, s_u[r], prev[rk]);
+                                                        });
+        if (a.cur) {
+            ((double2*)a.cur)[i] = acc;
+            continue;
+        }
+        const double sc = sf * a.norm_t;
+        const double2 v = make_double2(acc.x * sc, acc.y * sc);
+        if (a.amp) a.amp[i - a.lo] = v;
+        if (a.prob) a.prob[i - a.lo] = fma(v.x, v.x, v.y * v.y);
+    }
+}
+
+// What a block needs before its states: the tables, the shift and the scale.
+struct LevelSetup {
+    bool fp64;
+    int sh;
+    double back;
+};
+
+__device__ __forceinline__ LevelSetup level_setup(const FixedArgs& a, int k, int4* s_f, uint32_t* s_mc, unsigned& s_top)
+{
+    const int m = a.m, w1 = k + 1;
+    LevelSetup o{};
+    o.fp64 = a.hdr->fp64;
     for (int q = threadIdx.x; q < (m + 1) * w1; q += kThreads)
         s_mc[q] = (uint32_t)a.mc[(q / w1) * (a.n + 1) + q % w1];
     if (threadIdx.x == 0) s_top = 0;
-
-    if (fp64) {
-        double2* s_u = (double2*)s_f;
-        const double2* prev = (const double2*)a.prev;
-        for (int r = threadIdx.x; r < m; r += kThreads) s_u[r] = a.U[(size_t)r * m + a.col[k - 1]];
-        __syncthreads();
-        for (int64_t i = a.lo + (int64_t)blockIdx.x * kThreads + threadIdx.x; i < a.hi; i += (int64_t)gridDim.x * kThreads) {
-            double2 acc = make_double2(0.0, 0.0);
-            const double sf = expand_state<KMAX, uint32_t>(s_mc, w1, m, k, (uint32_t)i, a.prev_count, a.sqrtfact,
-                                                           [&](int r, uint32_t rk, int) {
-                                                               if (k == 1) acc = s_u[r];
-                                                               else cmac(acc, s_u[r], prev[rk]);
-                                                           });
-            if (!last) {
-                ((double2*)a.cur)[i] = acc;
-                continue;
-            }
-            const double sc = sf * a.norm_t;
-            const double2 v = make_double2(acc.x * sc, acc.y * sc);
-            if (a.amp) a.amp[i - a.lo] = v;
-            if (a.prob) a.prob[i - a.lo] = fma(v.x, v.x, v.y * v.y);
-        }
-        return;
-    }
-
+    if (o.fp64) return o;
     const int e = a.hdr->colexp[k - 1];
     for (int q = threadIdx.x; q < m * k; q += kThreads) {
         const double2 u = a.U[(size_t)(q / k) * m + a.col[k - 1]];
@@ -174,61 +181,190 @@ __global__ void __launch_bounds__(kThreads) expand_fixed_kernel(const __grid_con
         s_f[q] = y;
     }
     // The shift back to kXBits bits; the last level keeps three bits more, as it is not multiplied again.
-    int sh = 0, scale = kUBits - e;
+    const bool last = !a.cur;
+    int scale = kUBits - e;
     if (k > 1) {
         const double bound = ((double)a.hdr->top[k - 1] + 1.0) * sqrt(2.0 * k) * (1.0 + 0x1p-18);   // of M sqrt(2k), in 2^29
-        sh = min(max(ilogb(bound) + 1 + 29 + kUBits - kXBits - 30 - (last ? 3 : 0), 1), 30);
-        scale += a.hdr->scale[k - 1] - 30 - sh;
+        o.sh = min(max(ilogb(bound) + 1 + 29 + kUBits - kXBits - 30 - (last ? 3 : 0), 1), 30);
+        scale += a.hdr->scale[k - 1] - 30 - o.sh;
     }
     if (!last && blockIdx.x == 0 && threadIdx.x == 0) a.hdr->scale[k] = scale;
-    const double back = ldexp(a.norm_t, -scale);
+    o.back = ldexp(a.norm_t, -scale);
     __syncthreads();
+    return o;
+}
 
-    unsigned top = 0;
-    for (int64_t i = a.lo + (int64_t)blockIdx.x * kThreads + threadIdx.x; i < a.hi; i += (int64_t)gridDim.x * kThreads) {
-        Sum30 re, im;
-        long long x, y;
-        if (k == 1) {
-            const int4 u = s_f[i];
-            x = ((long long)u.x << 30) + u.y;
-            y = ((long long)u.z << 30) + u.w;
-        } else {
-            expand_state<KMAX, uint32_t>(s_mc, w1, m, k, (uint32_t)i, a.prev_count, nullptr,
-                                         [&](int r, uint32_t rk, int mult) {
-                                             const int4 u = s_f[r * k + mult - 1], c = a.prev[rk];
-                                             re.add(u.x, u.y, c.x, c.y);
-                                             re.add(-u.z, -u.w, c.z, c.w);
-                                             im.add(u.x, u.y, c.z, c.w);
-                                             im.add(u.z, u.w, c.x, c.y);
-                                         });
-            x = re.value(sh);
-            y = im.value(sh);
-        }
-        if (!last) {
-            int4 c;
-            split30(x, c.x, c.y);
-            split30(y, c.z, c.w);
-            a.cur[i] = c;
-            top = max(top, (unsigned)max(llabs(x) >> 29, llabs(y) >> 29));
-            continue;
-        }
-        const double2 v = make_double2((double)x * back, (double)y * back);
-        if (a.amp) a.amp[i - a.lo] = v;
-        if (a.prob) a.prob[i - a.lo] = fma(v.x, v.x, v.y * v.y);
+__device__ __forceinline__ void add_term(Sum30& re, Sum30& im, const int4 u, const int4 c)
+{
+    re.add(u.x, u.y, c.x, c.y);
+    re.add(-u.z, -u.w, c.z, c.w);
+    im.add(u.x, u.y, c.z, c.w);
+    im.add(u.z, u.w, c.x, c.y);
+}
+
+// State i of the level, x + i y: to the next level, or as an output.
+__device__ __forceinline__ void store_state(const FixedArgs& a, int64_t i, long long x, long long y, double back,
+                                            unsigned& top)
+{
+    if (a.cur) {
+        int4 c;
+        split30(x, c.x, c.y);
+        split30(y, c.z, c.w);
+        a.cur[i] = c;
+        top = max(top, (unsigned)max(llabs(x) >> 29, llabs(y) >> 29));
+        return;
     }
-    if (last) return;
+    const double2 v = make_double2((double)x * back, (double)y * back);
+    if (a.amp) a.amp[i - a.lo] = v;
+    if (a.prob) a.prob[i - a.lo] = fma(v.x, v.x, v.y * v.y);
+}
+
+__device__ __forceinline__ void publish_top(const FixedArgs& a, int k, unsigned top, unsigned& s_top)
+{
+    if (!a.cur) return;
     top = __reduce_max_sync(0xffffffffu, top);
     if ((threadIdx.x & 31) == 0) atomicMax(&s_top, top);
     __syncthreads();
     if (threadIdx.x == 0) atomicMax(&a.hdr->top[k], s_top);
 }
 
-template <int KMAX>
-cudaError_t launch_level(const FixedArgs& a, cudaStream_t s)
+// Levels 1 to 4: a thread per state.
+__global__ void __launch_bounds__(kThreads) expand_fixed_low_kernel(const __grid_constant__ FixedArgs a)
+{
+    extern __shared__ int4 s_f[];               // [m][k] factors (FP64 form: [m] entries of U), then the count table
+    const int m = a.m, k = a.k;
+    uint32_t* s_mc = (uint32_t*)(s_f + m * k);
+    __shared__ unsigned s_top;
+    const LevelSetup o = level_setup(a, k, s_f, s_mc, s_top);
+    if (o.fp64) return fp64_level(a, (double2*)s_f, s_mc);
+    unsigned top = 0;
+    for (int64_t i = a.lo + (int64_t)blockIdx.x * kThreads + threadIdx.x; i < a.hi; i += (int64_t)gridDim.x * kThreads) {
+        Sum30 re, im;
+        if (k == 1) {
+            const int4 u = s_f[i];
+            store_state(a, i, ((long long)u.x << 30) + u.y, ((long long)u.z << 30) + u.w, o.back, top);
+            continue;
+        }
+        expand_state<4, uint32_t>(s_mc, k + 1, m, k, (uint32_t)i, a.prev_count, nullptr, [&](int r, uint32_t rk, int mult) {
+            add_term(re, im, s_f[r * k + mult - 1], a.prev[rk]);
+        });
+        store_state(a, i, re.value(o.sh), im.value(o.sh), o.back, top);
+    }
+    publish_top(a, k, top, s_top);
+}
+
+// Level K >= 5: a warp takes runs of 32 `a.steps` consecutive states.  A thread
+// goes through its run 32 states at a time and keeps its first K - 4 photons
+// while only the last four change (113 states on average at m=20 n=10): their
+// modes, factors and the part of their terms' ranks that the last four do not
+// touch; a rank is then one subtraction.
+template <int K>
+__global__ void __launch_bounds__(kThreads, 3) expand_fixed_kernel(const __grid_constant__ FixedArgs a)
+{
+    constexpr int P = K - 4, W = K + 1;
+    extern __shared__ int4 s_f[];
+    const int m = a.m;
+    uint32_t* s_mc = (uint32_t*)(s_f + m * K);
+    __shared__ unsigned s_top;
+    const LevelSetup o = level_setup(a, K, s_f, s_mc, s_top);
+    if (o.fp64) return fp64_level(a, (double2*)s_f, s_mc);
+
+    // multisets of size j above mode l
+    auto above = [&](int l, int j) { return s_mc[(m - 1 - l) * W + j]; };
+    // the next position's mode from v on, `rest` photons behind it
+    auto next = [&](int v, int rest, uint32_t& idx) {
+        const uint32_t* q = s_mc + (m - v) * W + rest;
+        for (uint32_t c = *q; idx >= c; c = *q) {
+            idx -= c;
+            q -= W;
+            ++v;
+        }
+        return v;
+    };
+
+    const uint32_t run = 32u * (uint32_t)a.steps;
+    const uint32_t total = (uint32_t)(a.hi - a.lo), runs = (total + run - 1) / run;
+    unsigned top = 0;
+    for (uint32_t c = blockIdx.x * (kThreads / 32) + threadIdx.x / 32; c < runs; c += gridDim.x * (kThreads / 32)) {
+        uint32_t base[P], off = 0, size = 0, after = 0;
+        int fac[P], lp = 0, lm = 0;             // factor of a term, -1 where the mode's run goes on
+        const uint32_t end = min(total - c * run, run);
+        for (uint32_t d = threadIdx.x & 31; d < end; d += 32) {
+            const uint32_t out = c * run + d;
+            off += 32;
+            if (off >= size) {                  // the first photons of this state
+                int l[P];
+                uint32_t idx = (uint32_t)a.lo + out;
+                int v = 0;
+#pragma unroll
+                for (int p = 0; p < P; ++p) l[p] = v = next(v, K - 1 - p, idx);
+                off = idx;
+                size = s_mc[(m - v) * W + 4];
+                uint32_t suf = 0;
+                after = a.prev_count - 1;
+#pragma unroll
+                for (int p = 1; p < P; ++p) suf += above(l[p], K - p);
+#pragma unroll
+                for (int p = 0; p < P; ++p) {
+                    lm = p > 0 && l[p > 0 ? p - 1 : 0] == l[p] ? lm + 1 : 1;
+                    base[p] = after - suf;
+                    fac[p] = p + 1 < P && l[p + 1 < P ? p + 1 : p] == l[p] ? -1 : l[p] * K + lm - 1;
+                    after -= above(l[p], K - 1 - p);
+                    if (p + 1 < P) suf -= above(l[p + 1 < P ? p + 1 : p], K - 1 - p);
+                }
+                lp = v;
+            }
+            int x[4];
+            {
+                uint32_t idx = off;
+                x[0] = next(lp, 3, idx);
+                x[1] = next(x[0], 2, idx);
+                x[2] = next(x[1], 1, idx);
+                x[3] = x[2] + (int)idx;
+            }
+            uint32_t suf = above(x[1], 3) + above(x[2], 2) + above(x[3], 1);
+            const uint32_t all = suf + above(x[0], 4);
+            Sum30 re, im;
+#pragma unroll
+            for (int p = 0; p < P; ++p)
+                if (p + 1 < P ? fac[p] >= 0 : x[0] != lp) add_term(re, im, s_f[fac[p]], a.prev[base[p] - all]);
+            uint32_t pre = after;
+            int mult = lm, before = lp;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                mult = x[q] == before ? mult + 1 : 1;
+                before = x[q];
+                if (q == 3 || x[q < 3 ? q + 1 : q] != x[q]) add_term(re, im, s_f[x[q] * K + mult - 1], a.prev[pre - suf]);
+                if (q < 3) {
+                    pre -= above(x[q], 3 - q);
+                    suf -= above(x[q < 3 ? q + 1 : q], 3 - q);
+                }
+            }
+            store_state(a, a.lo + out, re.value(o.sh), im.value(o.sh), o.back, top);
+        }
+    }
+    publish_top(a, K, top, s_top);
+}
+
+cudaError_t launch_level(FixedArgs a, cudaStream_t s)
 {
     const size_t smem = (size_t)a.m * a.k * sizeof(int4) + (size_t)(a.m + 1) * (a.k + 1) * sizeof(uint32_t);
-    const int64_t tiles = (a.hi - a.lo + kThreads - 1) / kThreads;
-    expand_fixed_kernel<KMAX><<<(unsigned)std::min<int64_t>(tiles, kBlocks), kThreads, smem, s>>>(a);
+    // Runs of up to 16 x 32 states while every warp slot still gets four of them.
+    const int64_t n = a.hi - a.lo;
+    a.steps = (int)std::min<int64_t>(16, std::max<int64_t>(1, n / (32 * 4 * 8 * (int64_t)kBlocks)));
+    const int64_t per_block = (int64_t)kThreads * (a.k <= 4 ? 1 : a.steps);
+    const unsigned grid = (unsigned)std::min<int64_t>((n + per_block - 1) / per_block, kBlocks);
+    switch (a.k) {
+    case 5: expand_fixed_kernel<5><<<grid, kThreads, smem, s>>>(a); break;
+    case 6: expand_fixed_kernel<6><<<grid, kThreads, smem, s>>>(a); break;
+    case 7: expand_fixed_kernel<7><<<grid, kThreads, smem, s>>>(a); break;
+    case 8: expand_fixed_kernel<8><<<grid, kThreads, smem, s>>>(a); break;
+    case 9: expand_fixed_kernel<9><<<grid, kThreads, smem, s>>>(a); break;
+    case 10: expand_fixed_kernel<10><<<grid, kThreads, smem, s>>>(a); break;
+    case 11: expand_fixed_kernel<11><<<grid, kThreads, smem, s>>>(a); break;
+    case 12: expand_fixed_kernel<12><<<grid, kThreads, smem, s>>>(a); break;
+    default: expand_fixed_low_kernel<<<grid, kThreads, smem, s>>>(a); break;
+    }
     note_launches(1);
     return cudaGetLastError();
 }
@@ -274,7 +410,7 @@ cudaError_t launch_expand_fixed(const Plan& p, const double2* U, const int64_t* 
         a.cur = last ? nullptr : (int4*)buf[k & 1];
         a.amp = last ? amp : nullptr;
         a.prob = last ? prob : nullptr;
-        e = k <= 4 ? launch_level<4>(a, s) : k <= 8 ? launch_level<8>(a, s) : launch_level<kMaxN>(a, s);
+        e = launch_level(a, s);
     }
     return e;
 }
