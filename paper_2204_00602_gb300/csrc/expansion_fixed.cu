@@ -3,10 +3,14 @@
 //
 // What bounds it: the sums of slos.cu are bound by the FP64 pipe, which takes a
 // warp instruction per 16 cycles and SM: 64 cycles for the four DFMA of a
-// complex term.  Sixteen wide integer multiply-adds of 30-bit halves give the
-// same term in about 16, without any rounding inside a sum.  m=20 n=10: 2203 to
-// 1421 us (relative error against 64 bits 7.6e-16 to 6.3e-16), m=12 n=12: 294 to
-// 265 us (1.2e-15 to 9.2e-16).
+// complex term.  Sixteen wide integer multiply-adds of 30-bit halves (fixed30.cuh)
+// give the same term in about 16, without any rounding inside a sum; unranking
+// then takes as long again, so a thread keeps the first photons of its state.
+// m=20 n=10: 2203 us in FP64, 1383 in fixed point, 1118 with the first photons
+// kept (relative error against 64 bits 7.6e-16 and 6.3e-16); m=12 n=12: 294, 262,
+// 209 and, with the levels' starts overlapped, 168 us (1.2e-15 and 9.5e-16).
+// Now (ncu, m=18 n=9): multiplier pipe 49 %, 24 warps an SM, latency of the
+// multiply-add chains and of the gathers.
 //
 // Numbers.  The kernels carry B_k(s) of slos.cu (not C_k: all B_k(s) are of one
 // size, so one scale serves a level) as X = B_k(s) 2^S_k, components at most
@@ -30,6 +34,7 @@
 #include <cmath>
 
 #include "expansion.cuh"
+#include "fixed30.cuh"
 
 namespace pcv {
 namespace {
@@ -101,34 +106,6 @@ __global__ void fixed_setup_kernel(const __grid_constant__ FixedArgs a)
     }
 }
 
-__device__ __forceinline__ void wide_mad(long long& acc, int x, int y)
-{
-    asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc) : "r"(x), "r"(y));
-}
-
-__device__ __forceinline__ void split30(long long x, int& h, int& l)
-{
-    l = (int)((uint32_t)x << 2) >> 2;
-    h = (int)((x - l) >> 30);
-}
-
-struct Sum30 {                                  // hh 2^60 + hl 2^30 + ll
-    long long hh = 0, hl = 0, ll = 0;
-    __device__ __forceinline__ void add(int xh, int xl, int yh, int yl)
-    {
-        wide_mad(hh, xh, yh);
-        wide_mad(hl, xh, yl);
-        wide_mad(hl, xl, yh);
-        wide_mad(ll, xl, yl);
-    }
-    // the sum / 2^(30 + sh), rounded, 0 < sh <= 30
-    __device__ __forceinline__ long long value(int sh) const
-    {
-        const long long v = hl + (ll >> 30);
-        return (hh << (30 - sh)) + ((v + (1ll << (sh - 1))) >> sh);
-    }
-};
-
 // The FP64 form of a level: the sums of slos.cu.  Not inlined, so that it costs
 // the fixed-point form no registers.
 __device__ __noinline__ void fp64_level(const FixedArgs& a, double2* s_u, const uint32_t* s_mc)
@@ -166,20 +143,22 @@ __device__ __forceinline__ LevelSetup level_setup(const FixedArgs& a, int k, int
 {
     const int m = a.m, w1 = k + 1;
     LevelSetup o{};
+    if (k == 1) level_below_done();            // the first kernel's header; from level 2 on it is complete
     o.fp64 = a.hdr->fp64;
     for (int q = threadIdx.x; q < (m + 1) * w1; q += kThreads)
         s_mc[q] = (uint32_t)a.mc[(q / w1) * (a.n + 1) + q % w1];
     if (threadIdx.x == 0) s_top = 0;
-    if (o.fp64) return o;
+    if (o.fp64) {
+        if (k > 1) level_below_done();
+        return o;
+    }
     const int e = a.hdr->colexp[k - 1];
     for (int q = threadIdx.x; q < m * k; q += kThreads) {
         const double2 u = a.U[(size_t)(q / k) * m + a.col[k - 1]];
         const double f = ldexp(sqrt((double)(q % k + 1)), kUBits - e);
-        int4 y;
-        split30(__double2ll_rn(u.x * f), y.x, y.y);
-        split30(__double2ll_rn(u.y * f), y.z, y.w);
-        s_f[q] = y;
+        s_f[q] = split30(__double2ll_rn(u.x * f), __double2ll_rn(u.y * f));
     }
+    if (k > 1) level_below_done();
     // The shift back to kXBits bits; the last level keeps three bits more, as it is not multiplied again.
     const bool last = !a.cur;
     int scale = kUBits - e;
@@ -194,23 +173,12 @@ __device__ __forceinline__ LevelSetup level_setup(const FixedArgs& a, int k, int
     return o;
 }
 
-__device__ __forceinline__ void add_term(Sum30& re, Sum30& im, const int4 u, const int4 c)
-{
-    re.add(u.x, u.y, c.x, c.y);
-    re.add(-u.z, -u.w, c.z, c.w);
-    im.add(u.x, u.y, c.z, c.w);
-    im.add(u.z, u.w, c.x, c.y);
-}
-
 // State i of the level, x + i y: to the next level, or as an output.
 __device__ __forceinline__ void store_state(const FixedArgs& a, int64_t i, long long x, long long y, double back,
                                             unsigned& top)
 {
     if (a.cur) {
-        int4 c;
-        split30(x, c.x, c.y);
-        split30(y, c.z, c.w);
-        a.cur[i] = c;
+        a.cur[i] = split30(x, y);
         top = max(top, (unsigned)max(llabs(x) >> 29, llabs(y) >> 29));
         return;
     }
@@ -242,7 +210,7 @@ __global__ void __launch_bounds__(kThreads) expand_fixed_low_kernel(const __grid
         Sum30 re, im;
         if (k == 1) {
             const int4 u = s_f[i];
-            store_state(a, i, ((long long)u.x << 30) + u.y, ((long long)u.z << 30) + u.w, o.back, top);
+            store_state(a, i, join30(u.x, u.y), join30(u.z, u.w), o.back, top);
             continue;
         }
         expand_state<4, uint32_t>(s_mc, k + 1, m, k, (uint32_t)i, a.prev_count, nullptr, [&](int r, uint32_t rk, int mult) {
@@ -354,25 +322,26 @@ cudaError_t launch_level(FixedArgs a, cudaStream_t s)
     a.steps = (int)std::min<int64_t>(16, std::max<int64_t>(1, n / (32 * 4 * 8 * (int64_t)kBlocks)));
     const int64_t per_block = (int64_t)kThreads * (a.k <= 4 ? 1 : a.steps);
     const unsigned grid = (unsigned)std::min<int64_t>((n + per_block - 1) / per_block, kBlocks);
+    auto go = [&](void (*kernel)(const FixedArgs)) { return launch_level_kernel(kernel, dim3(grid), kThreads, smem, s, a); };
     switch (a.k) {
-    case 5: expand_fixed_kernel<5><<<grid, kThreads, smem, s>>>(a); break;
-    case 6: expand_fixed_kernel<6><<<grid, kThreads, smem, s>>>(a); break;
-    case 7: expand_fixed_kernel<7><<<grid, kThreads, smem, s>>>(a); break;
-    case 8: expand_fixed_kernel<8><<<grid, kThreads, smem, s>>>(a); break;
-    case 9: expand_fixed_kernel<9><<<grid, kThreads, smem, s>>>(a); break;
-    case 10: expand_fixed_kernel<10><<<grid, kThreads, smem, s>>>(a); break;
-    case 11: expand_fixed_kernel<11><<<grid, kThreads, smem, s>>>(a); break;
-    case 12: expand_fixed_kernel<12><<<grid, kThreads, smem, s>>>(a); break;
-    default: expand_fixed_low_kernel<<<grid, kThreads, smem, s>>>(a); break;
+    case 5: return go(expand_fixed_kernel<5>);
+    case 6: return go(expand_fixed_kernel<6>);
+    case 7: return go(expand_fixed_kernel<7>);
+    case 8: return go(expand_fixed_kernel<8>);
+    case 9: return go(expand_fixed_kernel<9>);
+    case 10: return go(expand_fixed_kernel<10>);
+    case 11: return go(expand_fixed_kernel<11>);
+    case 12: return go(expand_fixed_kernel<12>);
+    default: return go(expand_fixed_low_kernel);
     }
-    note_launches(1);
-    return cudaGetLastError();
 }
 
 }  // namespace
 
 // By the size of the problem alone, so that a range of outputs takes the form
-// of the whole.  states: of all levels; tables of factors and counts up to 44 KB.
+// of the whole.  The line (both with plain launches): fixed point against FP64 at m=20 n=6 (0.23 M states in
+// all) 57 and 50 us, m=46 n=4 (0.25 M) 49 and 36, m=30 n=5 (0.32 M) 54 and 50,
+// m=24 n=6 (0.59 M) 69 and 70, m=16 n=8 (0.74 M) 88 and 96, m=16 n=9 140 and 195.  states: of all levels; tables of factors and counts up to 44 KB.
 bool expand_fixed_applies(int m, int n, int64_t largest, int64_t states)
 {
     return n >= 2 && n <= kMaxN && m * n <= 2048 && largest <= (int64_t)UINT32_MAX && states >= kFixedMinStates;

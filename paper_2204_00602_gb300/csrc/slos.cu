@@ -65,6 +65,7 @@ __global__ void __launch_bounds__(kThreads) expand_kernel(const __grid_constant_
     __shared__ double s_norm[GROUP];
     __shared__ int s_col[GROUP];
     const int b0 = blockIdx.y * GROUP;
+    if (k == 1) level_below_done();
     if (threadIdx.x < GROUP) {
         const int b = min(b0 + (int)threadIdx.x, a.B - 1);
         int64_t parent = b;
@@ -100,6 +101,7 @@ __global__ void __launch_bounds__(kThreads) expand_kernel(const __grid_constant_
         s_u[q] = a.U[ub + (size_t)r * m + s_col[j]];
     }
     __syncthreads();
+    if (k > 1) level_below_done();
 
     const int64_t i = a.lo + (int64_t)blockIdx.x * kThreads + threadIdx.x;
     if (i >= a.hi) return;
@@ -143,9 +145,7 @@ cudaError_t launch_one(const ExpandArgs& a, cudaStream_t s)
         if (e != cudaSuccess) return e;
     }
     const dim3 grid((unsigned)((a.hi - a.lo + kThreads - 1) / kThreads), (unsigned)((a.B + GROUP - 1) / GROUP));
-    expand_kernel<KMAX, GROUP, I><<<grid, kThreads, smem, s>>>(a);
-    note_launches(1);
-    return cudaGetLastError();
+    return launch_level_kernel(expand_kernel<KMAX, GROUP, I>, grid, kThreads, smem, s, a);
 }
 
 template <int GROUP>

@@ -1,5 +1,5 @@
 """GPU: the fixed-point state expansion of large single distributions against
-the oracle at the bounds of its register lists (4, 8, 12 photons), for bunched
+the oracle at the bounds of its register lists (4, 8, 12 photons) and beside them, for bunched
 inputs, matrices that are not unitary and ranges; and its FP64 form, which
 matrices with entries of very different size, or none that is finite, take,
 against the batched FP64 expansion.  Tolerances: 1e-10 relative with the RMS
@@ -28,9 +28,9 @@ def dev(a):
 
 
 @pytest.mark.parametrize("m,n,t,form", [
-    (640, 2, None, "haar"), (46, 4, [1] * 4, "haar"), (24, 6, [3, 0, 2, 1], "haar"), (20, 7, None, "scaled"),
-    (14, 8, None, "gauss"), (12, 9, [9], "haar"), (9, 12, None, "haar"), (10, 12, [12], "haar"),
-    (10, 11, [4, 4, 3], "scaled")])
+    (998, 2, None, "haar"), (58, 4, [1] * 4, "haar"), (34, 5, [2, 1, 1, 1], "gauss"), (24, 6, [3, 0, 2, 1], "haar"),
+    (20, 7, None, "scaled"), (16, 8, None, "gauss"), (14, 9, [9], "haar"), (12, 10, None, "haar"),
+    (10, 12, [4] + [1] * 8, "haar"), (10, 12, [12], "haar"), (11, 11, [4, 4, 3], "scaled")])
 def test_matches_oracle(pcv, m, n, t, form):
     full = np.zeros(m, np.uint8)
     if t is None:
@@ -65,7 +65,7 @@ def test_matches_oracle(pcv, m, n, t, form):
 
 @pytest.mark.parametrize("form", ["coupling", "zero_column", "nan", "inf", "huge"])
 def test_fp64_form(pcv, form):
-    m, n = 16, 7
+    m, n = 19, 7
     t = pin.single_photon_input(m, n)
     U = pin.haar_unitary(m, 9790)
     if form == "coupling":                     # weakly coupled modes: outputs down to 1e-60
