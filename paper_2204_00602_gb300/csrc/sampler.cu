@@ -22,7 +22,10 @@
 //                          whole sample, 4 FP64 instructions each, where the
 //                          Glynn sums of the steps take about 14 n 2^{n-1}
 //                          (n = 14: 0.46 M against 1.6 M), and no sign
-//                          cancellation.  Two neighbouring levels live in
+//                          cancellation.  From n = 10 on the levels are in
+//                          fixed point on the integer pipe (16,384 samples of
+//                          n = 14: 17.3 to 10.8 ms; the FP64 pipe took 12.5 of
+//                          it).  Two neighbouring levels live in
 //                          shared memory (n = 14: 103 KB, two samples per SM;
 //                          n = 15: 206 KB), which ends the form at n = 15;
 //   sampler_kernel         n = 16: one Glynn sum per step (below), one warp
@@ -32,6 +35,11 @@
 
 #include <algorithm>
 
+#include <cfloat>
+#include <cmath>
+#include <type_traits>
+
+#include "fixed30.cuh"
 #include "pcv_common.cuh"
 
 namespace pcv {
@@ -102,12 +110,12 @@ __host__ __device__ inline int subset_level(int n, int odd)
     return best;
 }
 
-// Shared memory of one sample: two levels, the drawn row, the weights, the
-// sample's columns and rows.
+// Shared memory of one sample: two levels, the drawn row, the sub-permanents of
+// the step, the weights, the sample's columns and rows.
 __host__ __device__ inline size_t subset_bytes(int m, int n)
 {
-    return (size_t)(subset_level(n, 0) + subset_level(n, 1) + n) * sizeof(double2) +
-           (size_t)(m + (m & 1)) * sizeof(double) + 2 * 16 * sizeof(int);      // a multiple of 16
+    return (size_t)(subset_level(n, 0) + subset_level(n, 1) + 2 * n) * sizeof(double2) +
+           (size_t)(m + (m & 1)) * sizeof(double) + 3 * 16 * sizeof(int);      // a multiple of 16
 }
 
 constexpr int kBinom = 17;
@@ -115,11 +123,15 @@ constexpr int kBinom = 17;
 // Position of the lowest bit (15 for none: a valid row of the tables).
 __device__ __forceinline__ int low_bit(uint32_t x) { return (__ffs((int)x) - 1) & 15; }
 
-// A group of T threads per sample (T = 32: several samples per block).
-template <int T>
+// A group of T threads per sample (T = 32: several samples per block).  FIXED:
+// the levels in fixed point (fixed30.cuh), components at most 2^59.  A drawn row
+// is scaled by a power of two to 57 bits of its norm |a|, and with M the largest
+// component of level k - 1 a component of level k is below 2^57 M sqrt(2 k), which
+// gives the shift back; powers of two cancel in a draw, so no scale is kept.
+template <int T, bool FIXED>
 __global__ void subset_sampler_kernel(const __grid_constant__ SampArgs a)
 {
-    extern __shared__ double2 s_mem[];
+    extern __shared__ int4 s_mem[];
     __shared__ int s_c[kBinom][kBinom];        // C(t, j)
     for (int q = threadIdx.x; q < kBinom * kBinom; q += blockDim.x) {
         const int t = q / kBinom, j = q % kBinom;
@@ -137,23 +149,32 @@ __global__ void subset_sampler_kernel(const __grid_constant__ SampArgs a)
         else __syncthreads();
     };
     const int n_even = subset_level(n, 0), n_odd = subset_level(n, 1);
-    double2* base = (double2*)((char*)s_mem + (size_t)grp * subset_bytes(m, n));
-    double2* s_a = base + n_even + n_odd;      // A[r_k][.], the drawn row
-    double* s_w = (double*)(s_a + n);
+    using Level = std::conditional_t<FIXED, int4, double2>;
+    Level* base = (Level*)((char*)s_mem + (size_t)grp * subset_bytes(m, n));
+    Level* s_a = base + n_even + n_odd;         // A[r_k][.], the drawn row
+    double2* s_g = (double2*)(s_a + n);        // entries 0 .. k of level k in FP64
+    double* s_w = (double*)(s_g + n);
     int* s_pc = (int*)(s_w + m + (m & 1));               // input mode of each permuted photon
     int* s_rows = s_pc + 16;
+    unsigned* s_top = (unsigned*)(s_rows + 16);          // of the odd and even levels: max |component| >> 29
+    unsigned* s_nan = s_top + 2;                         // a drawn row is not finite
+    if (tid == 0) *s_nan = 0;
     if (tid < n) s_pc[tid] = a.cols[min((int)a.perm[smp * n + tid], n - 1)];   // clamp keeps reads in bounds
     sync();
     for (int k = 1; k <= n; ++k) {
         // weights: sub-permanent of {0..k-1} \ l is entry k-1-l of level k-1
-        const double2* f = base + ((k - 1) & 1 ? n_even : 0);      // level k - 1: even levels first, then odd
+        const Level* f = base + ((k - 1) & 1 ? n_even : 0);         // level k - 1: even levels first, then odd
+        if (tid == 0) s_top[k & 1] = 0;
         for (int i = tid; i < m; i += T) {
             const double2* Ui = a.U + (size_t)i * m;
             double2 s = make_double2(0.0, 0.0);
             if (k == 1) s = __ldg(Ui + s_pc[0]);
             else
-                for (int l = 0; l < k; ++l) cmac(s, __ldg(Ui + s_pc[l]), f[k - 1 - l]);
-            s_w[i] = fma(s.x, s.x, s.y * s.y);
+                for (int l = 0; l < k; ++l) {
+                    if constexpr (FIXED) cmac(s, __ldg(Ui + s_pc[l]), s_g[k - 1 - l]);
+                    else cmac(s, __ldg(Ui + s_pc[l]), f[k - 1 - l]);
+                }
+            s_w[i] = FIXED && *s_nan ? NAN : fma(s.x, s.x, s.y * s.y);
         }
         sync();
         if (tid < 32) {
@@ -162,14 +183,29 @@ __global__ void subset_sampler_kernel(const __grid_constant__ SampArgs a)
             for (int c = 0; c < 4; ++c) wloc[c] = tid + 32 * c < m ? s_w[tid + 32 * c] : 0.0;
             const int r = draw_mode(wloc, m, a.uni[smp * n + k - 1]);
             if (tid == 0) s_rows[k - 1] = r;
-            if (tid < n) s_a[tid] = __ldg(a.U + (size_t)r * m + s_pc[tid]);
+            const double2 u = tid < n ? __ldg(a.U + (size_t)r * m + s_pc[tid]) : make_double2(0.0, 0.0);
+            if constexpr (FIXED) {
+                double sum = fma(u.x, u.x, u.y * u.y);
+                for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+                if (!(sum <= DBL_MAX) && tid == 0) *s_nan = 1;
+                int e = 0;                         // 2^e at least the row's norm
+                if (sum > 0.0 && sum <= DBL_MAX) frexp(sqrt(sum) * (1.0 - 0x1p-20), &e);
+                const double sc = ldexp(1.0, 57 - e);
+                if (tid < n) s_a[tid] = split30(__double2ll_rn(u.x * sc), __double2ll_rn(u.y * sc));
+            } else if (tid < n) {
+                s_a[tid] = u;
+            }
         }
         sync();
         if (k == n) break;
         // level k: contiguous runs of subsets (increasing masks) per thread.
         // The rank of S is sum_i C(s_i, i + 1) over its elements in order;
         // without s_j the elements after it move down one place.
-        double2* cur = base + (k & 1 ? n_even : 0);
+        Level* cur = base + (k & 1 ? n_even : 0);
+        int sh = 1;
+        if (FIXED && k > 1)
+            sh = min(max(ilogbf(((float)s_top[(k - 1) & 1] + 1.0f) * sqrtf(2.0f * k) * 1.0001f) - 2, 1), 30);
+        unsigned top = 0;
         const int cnt = s_c[n][k];
         const int below = s_c[n][k - 1];       // entries of level k - 1
         const int per = (cnt + T - 1) / T;
@@ -187,21 +223,38 @@ __global__ void subset_sampler_kernel(const __grid_constant__ SampArgs a)
             int suf = 0;                       // sum over the elements not yet passed, one place down
             uint32_t x = mask;
             for (int i = 0; i < k; ++i, x &= x - 1) suf += s_c[low_bit(x)][i];
+            Sum30 re, im;
             double2 acc = make_double2(0.0, 0.0);
             int pre = 0;
             x = mask;
-            for (int i = 0; i < k; ++i, x &= x - 1) {
+            for (int i = 0; i < k && k > 1; ++i, x &= x - 1) {
                 const int l = low_bit(x);
                 suf -= s_c[l][i];
-                if (k == 1) acc = s_a[l];
-                else cmac(acc, s_a[l], f[min((uint32_t)(pre + suf), (uint32_t)(below - 1))]);
+                const Level c = f[min((uint32_t)(pre + suf), (uint32_t)(below - 1))];
+                if constexpr (FIXED) add_term(re, im, s_a[l], c);
+                else cmac(acc, s_a[l], c);
                 pre += s_c[l][i + 1];
             }
-            if (q < cnt) cur[q] = acc;
+            if (q < cnt) {
+                const Level row = s_a[low_bit(mask)];
+                if constexpr (FIXED) {
+                    const long long vx = k == 1 ? join30(row.x, row.y) : re.value(sh);
+                    const long long vy = k == 1 ? join30(row.z, row.w) : im.value(sh);
+                    cur[q] = split30(vx, vy);
+                    if (q <= k) s_g[q] = make_double2((double)vx, (double)vy);
+                    top = max(top, (unsigned)max(llabs(vx) >> 29, llabs(vy) >> 29));
+                } else {
+                    cur[q] = k == 1 ? row : acc;
+                }
+            }
             if (q + 1 < cnt) {
                 const uint32_t c = mask & (0u - mask), r = mask + c;
                 mask = r | (((mask ^ r) >> 2) >> (__ffs(mask) - 1));
             }
+        }
+        if constexpr (FIXED) {
+            top = __reduce_max_sync(0xffffffffu, top);
+            if ((tid & 31) == 0) atomicMax(&s_top[k & 1], top);
         }
         sync();
     }
@@ -360,10 +413,17 @@ cudaError_t launch_sampler(const Plan& p, const double2* U, const uint8_t* perm,
             }
             return r;
         };
-        if (p.n <= 8) return go(subset_sampler_kernel<32>, 256, 8);
-        if (p.n <= 11) return go(subset_sampler_kernel<32>, 64, 2);
-        if (p.n <= 14) return go(subset_sampler_kernel<128>, 128, 1);
-        return go(subset_sampler_kernel<256>, 256, 1);
+        // Fixed point and threads, measured on 16,384 samples of n = 14 (m = 60):
+        // FP64 with 128 threads 17.3 ms, fixed point with 128, 256, 512 threads
+        // 14.4, 11.4, 10.8; n = 12: 4.0, and 2.6, 3.4, 5.7; n = 13: 7.8, and 5.4, 5.2,
+        // 7.9; n = 15 (4,096): 9.4 with 256, and 11.3, 7.8, 6.3.  n = 8 (60,000, a warp
+        // each): 1.60 in FP64 and 1.96, n = 10 (50,000): 3.10 and 2.41.
+        if (p.n <= 8) return go(subset_sampler_kernel<32, false>, 256, 8);
+        if (p.n <= 9) return go(subset_sampler_kernel<32, false>, 64, 2);
+        if (p.n <= 11) return go(subset_sampler_kernel<32, true>, 64, 2);
+        if (p.n <= 12) return go(subset_sampler_kernel<128, true>, 128, 1);
+        if (p.n <= 13) return go(subset_sampler_kernel<256, true>, 256, 1);
+        return go(subset_sampler_kernel<512, true>, 512, 1);
     }
     const size_t smem = (size_t)p.m * p.n * sizeof(double2);
     const unsigned blocks = (unsigned)((count + kSampWarps - 1) / kSampWarps);
