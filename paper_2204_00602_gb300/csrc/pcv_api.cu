@@ -634,9 +634,10 @@ static int auto_dist_algo(int m, int n, int64_t workspace_bytes)
 // its two levels (it does wherever it holds the tensor-core plan, but for the
 // space's limits in fp64_expand_ws): n multiply-adds per output at most instead
 // of 2^(n-1).  Measured over m = 6..64, n = 3..10, 56 to 20 M outputs, the
-// products against the expansion: m=6 n=3 66 and 31 us, m=13 n=7 167 and 62,
-// m=16 n=8 196 and 101, m=10 n=10 249 and 83, m=24 n=7 314 and 198, m=20 n=10
-// 2397 and 2202; there is no size on the other side.
+// products against the expansion: m=6 n=3 65 and 30 us, m=13 n=7 168 and 56,
+// m=16 n=8 196 and 65, m=20 n=10 2399 and 1118; also with its FP64 levels alone
+// (m=10 n=10 249 and 83, m=24 n=7 314 and 198, m=20 n=10 2397 and 2202) there
+// was no size on the other side.
 static bool auto_expands(int m, int n, int64_t workspace_bytes)
 {
     const int64_t x = fp64_expand_ws(1, m, n);
