@@ -121,10 +121,11 @@ int64_t pcv_amplitudes_workspace(int m, int n, int64_t n_out);
  * expansions of the two halves (at most C(n, n/2) terms per output; needs the
  * workspace pcv_amplitudes_workspace names, a smaller one takes the Glynn
  * kernels); else, from about 2e7 FP64 instructions of the plain kernels on,
- * the shared-row-sum tile kernel with its sign vectors split over blocks, or
- * for n >= 13 and m <= 128 a per-output choice between that kernel and Glynn's
- * sum with multiplicities (PCV_ALGO_MULT below), whichever takes less time for
- * that output; otherwise the plain Glynn kernels. */
+ * the shared-row-sum tile kernel with its sign vectors split over blocks, or,
+ * with m <= 128, n >= 13 and enough outputs to give every SM a tile, a
+ * per-output choice between that kernel and Glynn's sum with multiplicities
+ * (PCV_ALGO_MULT below), whichever takes less time for that output; otherwise
+ * the plain Glynn kernels. */
 int pcv_amplitudes(const pcv_c64* U, int m, const uint8_t* input_occ,
                    const uint8_t* output_occ, int64_t n_out,
                    pcv_c64* amp, double* prob,

@@ -178,12 +178,15 @@ int64_t amp_workspace(const AmpChoice& c, int64_t n_out)
 }
 
 // PCV_ALGO_AUTO's choice among the Glynn kernels when the workspace holds it:
-// the tile kernel with split sequences, behind the per-output routing where
-// bunched outputs can be much cheaper (n >= kRouteMinPhotons, m <= 128).  Its
-// integer products cost 1.25 FP64 instructions per photon and lane, a warp 32
-// lanes however few outputs it has, against 6n - 2 of the plain kernels; below
-// kTileOverhead instructions in all the plain kernels' single launch is
-// quicker.  (256 outputs at m=324 n=18: 6.95 ms by the block kernel, 1.82 ms.)
+// the tile kernel with split sequences.  Its integer products cost 1.25 FP64
+// instructions per photon and lane, a warp 32 lanes however few outputs it has,
+// against 6n - 2 of the plain kernels; below kTileOverhead instructions in all
+// the plain kernels' single launch is quicker.  (256 outputs at m=324 n=18: 6.95
+// ms by the block kernel, 1.82 ms.)  Too few outputs for choose_amp's per-output
+// routing stay out of it here too: its multiplicity kernel gives a permanent one
+// warp (33 outputs at m=24 n=18 took 20.7 ms against 1.4 by the block kernel, 7
+// bunched ones at m=40 n=18 7.8 against 0.7), and its weighted terms cost bits
+// (64 bunched outputs at m=15 n=15: rms error 1.7e-14, the block kernel 3.8e-15).
 constexpr double kTileOverhead = 2e7;
 
 AmpChoice choose_glynn(int m, int n, int64_t n_out)
@@ -194,7 +197,6 @@ AmpChoice choose_glynn(int m, int n, int64_t n_out)
     const double tile = std::ldexp(1.25 * n * 32.0 * (double)((n_out + 31) / 32), n - 1);
     if (steps * (6 * n - 2) < kTileOverhead || tile > steps * (6 * n - 2) || pcv::tile_split_workspace(m, n, n_out) < 0)
         return plain;
-    if (n >= kRouteMinPhotons && m <= pcv::tile_max_modes()) return {kAlgoRouted, 0};
     return {kAlgoTileSplit, 0};
 }
 
