@@ -226,12 +226,15 @@ int64_t pcv_distribution_workspace_min(int m, int n);
  * and workspace_bytes >= pcv_distribution_tc_workspace(m, n), else
  * PCV_ALGO_FACTOR.  Under either plan the call computes by state expansion
  * (the method of PCV_ALGO_SLOS) when the workspace holds its level buffers
- * (pcv_distribution_slos_workspace(1, m, n) + 256 bytes), which is never slower;
- * else by the tensor-core products or by the factorised sum with FP64 products,
- * in as many passes as the workspace asks for.  All give the same amplitudes to
- * double precision.  Returns
- * the algorithm code, or PCV_EINVAL for sizes out of range.  No counterpart in
- * the paper. */
+ * (pcv_distribution_slos_workspace(1, m, n) + 256 bytes), the faster of the two
+ * at every size measured; else by the tensor-core products or by the factorised
+ * sum with FP64 products, in as many passes as the workspace asks for.  All
+ * give the same amplitudes up to an absolute error of some 2^-53 of the
+ * distribution's largest amplitudes (Glynn's sums cancel to that, and the
+ * expansion of one unitary with 0.5 M states or more sums in fixed point);
+ * amplitudes far below that have no correct digits, unless PCV_ALGO_SLOS is
+ * asked for by name.  Returns the algorithm code, or PCV_EINVAL for sizes out
+ * of range.  No counterpart in the paper. */
 int pcv_distribution_auto_algo(int m, int n, int64_t workspace_bytes);
 
 /* Every output of S_{m,n} in canonical order (the SLOS back-end's full
@@ -317,7 +320,9 @@ int pcv_distribution_batched(const pcv_c64* U, int B, int m, const uint8_t* inpu
  *     B_k(s) = sum_{r: s_r >= 1} U[r][c_k] sqrt(s_r) B_{k-1}(s - e_r),  B_0 = 1,
  * and a(S) = B_n(S) / sqrt(prod t!) gives Eq. eqperm's amplitudes in canonical
  * order; level k keeps C(m+k-1, k) complex values.  Layouts as
- * pcv_distribution_batched (U [B][m][m], outputs [B][C(m+n-1,n)]). */
+ * pcv_distribution_batched (U [B][m][m], outputs [B][C(m+n-1,n)]).  FP64 at
+ * every size: an output's error is relative to the sum of its own terms'
+ * magnitudes, however small it is beside the others. */
 int64_t pcv_distribution_slos_workspace(int B, int m, int n);
 int pcv_distribution_slos(const pcv_c64* U, int B, int m, const uint8_t* input_occ,
                           double* prob, pcv_c64* amp,

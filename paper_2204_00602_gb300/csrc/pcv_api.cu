@@ -184,9 +184,9 @@ int64_t amp_workspace(const AmpChoice& c, int64_t n_out)
 // the plain kernels' single launch is quicker.  (256 outputs at m=324 n=18: 6.95
 // ms by the block kernel, 1.82 ms.)  Too few outputs for choose_amp's per-output
 // routing stay out of it here too: its multiplicity kernel gives a permanent one
-// warp (33 outputs at m=24 n=18 took 20.7 ms against 1.4 by the block kernel, 7
-// bunched ones at m=40 n=18 7.8 against 0.7), and its weighted terms cost bits
-// (64 bunched outputs at m=15 n=15: rms error 1.7e-14, the block kernel 3.8e-15).
+// warp (33 outputs at m=24 n=18: 20.7 ms, the block kernel 1.38, split tiles 0.50;
+// 7 bunched ones at m=40 n=18: 7.75, 0.70 and 0.35), and its weighted terms cost
+// bits (64 bunched outputs at m=15 n=15: rms errors 1.7e-14, 3.8e-15 and 1.1e-15).
 constexpr double kTileOverhead = 2e7;
 
 AmpChoice choose_glynn(int m, int n, int64_t n_out)
@@ -706,8 +706,8 @@ static int distribution_fp64(const pcv_c64* U, int B, int m, const uint8_t* inpu
     const int64_t xws = expand ? fp64_expand_ws(B, m, p.n) : -1;
     if (xws >= 0 && workspace_bytes >= xws) {
         pcv::stage_begin(pcv::kStagePlain, s);
-        cudaError_t e = pcv::launch_slos(p, B, (const double2*)U, lo, hi, prob, (double2*)amp, (char*)workspace + 256,
-                                         workspace, s);
+        cudaError_t e = pcv::launch_slos(p, B, (const double2*)U, lo, hi, true, prob, (double2*)amp,
+                                         (char*)workspace + 256, workspace, s);
         pcv::stage_end(pcv::kStagePlain, s);
         return e == cudaSuccess ? PCV_OK : cuda_fail(e, "state expansion");
     }
@@ -760,7 +760,7 @@ int pcv_distribution_slos(const pcv_c64* U, int B, int m, const uint8_t* input_o
         return fail(PCV_ENOMEM, "workspace of %lld bytes (256-byte aligned) needed, %lld given", (long long)need,
                     (long long)workspace_bytes);
     pcv::stage_begin(pcv::kStagePlain, s);
-    cudaError_t e = pcv::launch_slos(p, B, (const double2*)U, 0, N, prob, (double2*)amp, workspace, nullptr, s);
+    cudaError_t e = pcv::launch_slos(p, B, (const double2*)U, 0, N, false, prob, (double2*)amp, workspace, nullptr, s);
     pcv::stage_end(pcv::kStagePlain, s);
     return e == cudaSuccess ? PCV_OK : cuda_fail(e, "state expansion");
 }

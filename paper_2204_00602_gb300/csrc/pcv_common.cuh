@@ -216,11 +216,12 @@ cudaError_t launch_source(const SourcePlan& p, int m, int n, const int* modes, c
                           double beta, double gamma, double* prob, void* ws, cudaStream_t s);
 
 // Photon-by-photon state expansion (slos.cu)
-// outputs [lo, hi) of every batch entry, at [b][o - lo]; status: 16 bytes
-// zeroed on the stream, or null
+// outputs [lo, hi) of every batch entry, at [b][o - lo]; fixed: levels in fixed
+// point allowed (an error of one absolute size per level) where they are the
+// faster form; status: 16 bytes zeroed on the stream, or null
 int64_t slos_workspace(int B, int m, int n);
-cudaError_t launch_slos(const Plan& p, int B, const double2* U, int64_t lo, int64_t hi, double* prob, double2* amp,
-                        void* ws, void* status, cudaStream_t s);
+cudaError_t launch_slos(const Plan& p, int B, const double2* U, int64_t lo, int64_t hi, bool fixed, double* prob,
+                        double2* amp, void* ws, void* status, cudaStream_t s);
 
 // Adjoint of the full distribution by the state expansion
 // (expansion_grad.cu).  The plan's total is -1 where it does not apply (n = 0,

@@ -328,8 +328,8 @@ int64_t slos_workspace(int B, int m, int n)
                      2 * al256((size_t)B * half * sizeof(double2)));
 }
 
-cudaError_t launch_slos(const Plan& p, int B, const double2* U, int64_t lo, int64_t hi, double* prob, double2* amp,
-                        void* ws, void* status, cudaStream_t s)
+cudaError_t launch_slos(const Plan& p, int B, const double2* U, int64_t lo, int64_t hi, bool fixed, double* prob,
+                        double2* amp, void* ws, void* status, cudaStream_t s)
 {
     const int m = p.m, n = p.n;
     if (!amp && !prob) return cudaErrorInvalidValue;
@@ -367,7 +367,7 @@ cudaError_t launch_slos(const Plan& p, int B, const double2* U, int64_t lo, int6
         if (k < n) half = std::max(half, count[k]);
         states += count[k] < kFixedMinStates ? count[k] : kFixedMinStates;
     }
-    const bool fixed = B == 1 && hi > lo && expand_fixed_applies(m, n, std::max(half, count[n]), states);
+    fixed = fixed && B == 1 && hi > lo && expand_fixed_applies(m, n, std::max(half, count[n]), states);
     if (status && !fixed) {
         const cudaError_t e = cudaMemsetAsync(status, 0, 16, s);
         if (e != cudaSuccess) return e;
