@@ -233,8 +233,10 @@ int64_t pcv_distribution_workspace_min(int m, int n);
  * distribution's largest amplitudes (Glynn's sums cancel to that, and the
  * expansion of one unitary with 0.5 M states or more sums in fixed point);
  * amplitudes far below that have no correct digits, unless PCV_ALGO_SLOS is
- * asked for by name.  Returns the algorithm code, or PCV_EINVAL for sizes out
- * of range.  No counterpart in the paper. */
+ * asked for by name (the default keeps FP64 sums where a mode holds all photons
+ * with an amplitude below 2^-42 of the input columns' norms).  Returns the
+ * algorithm code, or PCV_EINVAL for sizes out of range.  No counterpart in the
+ * paper. */
 int pcv_distribution_auto_algo(int m, int n, int64_t workspace_bytes);
 
 /* Every output of S_{m,n} in canonical order (the SLOS back-end's full

@@ -27,8 +27,15 @@
 // error is one of absolute size, as that of Glynn's sum, so inputs whose outputs
 // differ by many orders of magnitude by construction keep the FP64 sums: where a
 // column has an entry that is neither zero nor at least 2^-20 of its norm, or a
-// norm outside 2^-40 .. 2^40, or an entry that is not finite, the same launches
-// run the FP64 form of slos.cu (the first kernel decides, on the device).
+// norm outside 2^-40 .. 2^40, or an entry that is not finite, or where a mode
+// takes all n photons with an amplitude B_n = sqrt(n!) prod_j |U[r][c_j]| below
+// 2^-42 of the norms' product (a zero entry counts as the least other one of its
+// row: weak couplings between few modes have zeros beside them), the same
+// launches run the FP64 form of slos.cu (the first kernel decides, on the
+// device).  Single entries do not tell: U = I + 1e-3 Haar at m=19 n=7 has none
+// below 2^-17, and 190,797 of its 480,700 amplitudes came out as zero.  The least
+// such amplitude of Haar matrices, 300 draws each: m=20 n=10 2^-22 in the median
+// and 2^-32 at worst, m=28 n=12 2^-28 and 2^-41.
 
 #include <algorithm>
 #include <cmath>
@@ -66,20 +73,27 @@ struct FixedArgs {
     double norm_t;
     FixedHeader* hdr;
     int64_t* status;           // setup: two words zeroed, or null
+    float most_bits;           // setup: least log2 of a mode's prod_j |U[r][c_j]| / norm_j, negated
     double sqrtfact[kMaxN + 1];
 };
 
-// One warp per photon: its column's norm, and whether the fixed-point form applies.
+constexpr float kRowBits = 42.0f;
+
+// One warp per photon: its column's norm; then the rows, a thread each: whether
+// the fixed-point form applies.
 __global__ void fixed_setup_kernel(const __grid_constant__ FixedArgs a)
 {
     const int j = threadIdx.x / 32, lane = threadIdx.x & 31;
-    __shared__ int s_bad[kMaxN];
+    extern __shared__ float s_log[];           // [n][m]: -log2 of an entry's larger component, infinity for 0
+    __shared__ int s_bad[kMaxN], s_bits;
+    __shared__ float s_norm[kMaxN];            // log2 of the norm
     double sum = 0.0, least = INFINITY;
     for (int r = lane; r < a.m; r += 32) {
         const double2 u = a.U[(size_t)r * a.m + a.col[j]];
         sum = fma(u.x, u.x, fma(u.y, u.y, sum));
         const double c = fmax(fabs(u.x), fabs(u.y));
         if (c > 0.0) least = fmin(least, c);
+        s_log[j * a.m + r] = -__log2f((float)c);
     }
     for (int d = 16; d; d >>= 1) {
         sum += __shfl_xor_sync(0xffffffffu, sum, d);
@@ -90,6 +104,7 @@ __global__ void fixed_setup_kernel(const __grid_constant__ FixedArgs a)
     const bool ok = norm >= 0x1p-40 && norm <= 0x1p40 && least >= 0x1p-20 * norm;
     if (lane == 0) {
         s_bad[j] = !ok;
+        s_norm[j] = __log2f((float)norm);
         int e = 0;
         if (ok) {
             frexp(norm * (1.0 - 0x1p-20), &e);     // a norm of 1 but for rounding counts as 1
@@ -98,9 +113,25 @@ __global__ void fixed_setup_kernel(const __grid_constant__ FixedArgs a)
     }
     if (threadIdx.x <= kMaxN) a.hdr->top[threadIdx.x] = 0;
     if (a.status && threadIdx.x < 2) a.status[threadIdx.x] = 0;
+    if (threadIdx.x == 0) s_bits = 0;
+    __syncthreads();
+    for (int r = threadIdx.x; r < a.m; r += blockDim.x) {
+        float bits = 0.0f, most = 0.0f;
+        int zeros = 0;
+        for (int q = 0; q < a.n; ++q) {
+            const float b = s_log[q * a.m + r];
+            if (isinf(b)) {
+                ++zeros;
+            } else {                           // nothing to use where a column is not ok
+                bits += fmaxf(b + s_norm[q], 0.0f);
+                most = fmaxf(most, b + s_norm[q]);
+            }
+        }
+        if (zeros < a.n) atomicMax(&s_bits, __float_as_int(bits + zeros * most));      // not negative: ordered as integers
+    }
     __syncthreads();
     if (threadIdx.x == 0) {
-        int bad = 0;
+        int bad = __int_as_float(s_bits) > a.most_bits;
         for (int q = 0; q < a.n; ++q) bad |= s_bad[q];
         a.hdr->fp64 = bad;
     }
@@ -363,9 +394,10 @@ cudaError_t launch_expand_fixed(const Plan& p, const double2* U, const int64_t* 
     a.norm_t = p.norm_t;
     a.hdr = (FixedHeader*)header;
     a.status = status;
+    a.most_bits = kRowBits + (float)std::log2(d.sqrtfact[p.n]);
     for (int j = 0; j < p.n; ++j) a.col[j] = p.cols[j];
     for (int j = 0; j <= kMaxN; ++j) a.sqrtfact[j] = d.sqrtfact[j];
-    fixed_setup_kernel<<<1, 32 * p.n, 0, s>>>(a);
+    fixed_setup_kernel<<<1, 32 * p.n, (size_t)p.m * p.n * sizeof(float), s>>>(a);      // 8 KB at most
     note_launches(1);
     cudaError_t e = cudaGetLastError();
     for (int k = 1; k <= p.n && e == cudaSuccess; ++k) {
