@@ -19,11 +19,15 @@
 // the 2-norm of column c.  With M the largest component of level k-1 and
 // sum_r sqrt(s_r) |U_r| <= sqrt(k) |U|, a component of level k is below
 // 2^57 M sqrt(2 k) before it is shifted back to 59 bits: the shift follows from
-// M, which every level leaves in the header, so nothing can overflow and at most
-// 4 of the 59 bits stay unused.  Sums of half products: with 12 terms the cross
+// M, which every level leaves in the header, so nothing can overflow.  What stays
+// unused: level 1 is stored unshifted, 2 + log2(|U| / max |U_r|) of its 59 bits,
+// and where a column's entries are of one magnitude a later level's largest
+// component is about sqrt(k / m) M, (1 + log2 m) / 2 bits below the bound.  So 2 to 3
+// bits at m = 20; 7 of level 1 at m = 1024, n = 2 and 5 of a level at m = 682, n = 3,
+// the most modes the tables take.  Sums of half products: with 12 terms the cross
 // sum is below 24 2^58 + 2^59 < 2^63, the others are smaller.
 //
-// A level rounds once, to 2^-53 of the level's typical amplitude or less.  The
+// A level rounds once, to 2^-52 of the level's typical amplitude or less.  The
 // error is one of absolute size, as that of Glynn's sum, so inputs whose outputs
 // differ by many orders of magnitude by construction keep the FP64 sums: where a
 // column has an entry that is neither zero nor at least 2^-20 of its norm, or a
