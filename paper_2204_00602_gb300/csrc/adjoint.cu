@@ -383,11 +383,8 @@ template <int CJ>
 cudaError_t launch_part(const AdjArgs& a, int B, cudaStream_t s)
 {
     const size_t smem = kWarpsA * warp_smem_bytes(a.n);
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(adjoint_part_kernel<CJ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = allow_dynamic_smem((const void*)adjoint_part_kernel<CJ>, smem);
+    if (e != cudaSuccess) return e;
     const int64_t items = a.chunk * a.parts;
     dim3 grid((unsigned)((items + kWarpsA - 1) / kWarpsA), (unsigned)B);
     adjoint_part_kernel<CJ><<<grid, kWarpsA * 32, smem, s>>>(a);

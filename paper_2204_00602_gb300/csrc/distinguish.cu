@@ -392,9 +392,7 @@ cudaError_t launch_source(const SourcePlan& p, int m, int n, const int* modes, c
         }
         if (blocks > INT32_MAX) return cudaErrorInvalidConfiguration;
         auto go = [&](auto kernel) {
-            cudaError_t r = cudaSuccess;
-            if (smem > 48 * 1024)
-                r = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            const cudaError_t r = allow_dynamic_smem((const void*)kernel, smem);
             if (r != cudaSuccess) return r;
             kernel<<<(unsigned)blocks, 256, smem, s>>>(g);
             note_launches(1);

@@ -748,13 +748,6 @@ size_t batch_smem()
     return b;
 }
 
-template <typename K>
-cudaError_t allow_smem(K kernel, size_t smem)
-{
-    return smem > 48 * 1024 ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
-                            : cudaSuccess;
-}
-
 // Tile shape of one circuit (or B unitaries with the same outputs): the tile
 // size as the batched planner chooses it, and two blocks per SM (what shared
 // memory holds) if the sequences may be split.
@@ -791,7 +784,7 @@ cudaError_t tile_launch(const pcv_batch_desc& d, int B, const TileShape& sh, dou
     a.ostride = d.n_out;
     a.partial = partial;
     const size_t smem = tile_smem(d.n, d.m, sh);
-    cudaError_t e = allow_smem(glynn_tile_kernel, smem);
+    cudaError_t e = allow_dynamic_smem((const void*)glynn_tile_kernel, smem);
     if (e != cudaSuccess) return e;
     const int64_t blocks = (d.n_out + sh.T - 1) / sh.T * sh.parts;
     if (blocks > INT32_MAX) return cudaErrorInvalidConfiguration;
@@ -878,7 +871,7 @@ cudaError_t launch_glynn_batched(const pcv_batch_desc* descs, int n_circ, int64_
                                  int64_t ws_bytes, int sms, int route, cudaStream_t s)
 {
     const size_t smem = batch_smem();
-    cudaError_t e = allow_smem(glynn_persistent_kernel, smem);
+    cudaError_t e = allow_dynamic_smem((const void*)glynn_persistent_kernel, smem);
     if (e != cudaSuccess) return e;
     int64_t max_items = total_outputs / 32 + n_circ + 1;
     char* w = (char*)ws;

@@ -145,10 +145,8 @@ cudaError_t launch_mesh_forward(const double* phases, int B, int m, double2* U, 
 {
     const int nq = m * (m - 1) / 2;
     const size_t smem = ((size_t)m * m + 4 * nq) * sizeof(double2);
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(mesh_forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = allow_dynamic_smem((const void*)mesh_forward_kernel, smem);
+    if (e != cudaSuccess) return e;
     mesh_forward_kernel<<<B, mesh_threads(m), smem, s>>>(phases, m, nq, U);
     note_launches(1);
     return cudaGetLastError();
@@ -159,10 +157,8 @@ cudaError_t launch_mesh_backward(const double* phases, int B, int m, const doubl
 {
     const int nq = m * (m - 1) / 2;
     const size_t smem = ((size_t)2 * m * m + 2 * nq) * sizeof(double2) + (size_t)2 * (m / 2) * m * sizeof(double);
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(mesh_backward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = allow_dynamic_smem((const void*)mesh_backward_kernel, smem);
+    if (e != cudaSuccess) return e;
     mesh_backward_kernel<<<B, mesh_threads(m), smem, s>>>(phases, m, nq, U, G, gphi);
     note_launches(1);
     return cudaGetLastError();

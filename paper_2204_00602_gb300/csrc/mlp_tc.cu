@@ -36,7 +36,6 @@
 #include <cudaTypedefs.h>
 
 #include <algorithm>
-#include <atomic>
 #include <cstdio>
 #include <mutex>
 
@@ -328,18 +327,8 @@ cudaError_t make_map(CUtensorMap* map, const void* base, int inner, int outer, i
 template <int BN, int MODE, int KB>
 cudaError_t launch_tile(const CUtensorMap& ma, const CUtensorMap& mb, const TcArgs& a, size_t smem, cudaStream_t s)
 {
-    // the largest ring once per device (an attribute of the function, not of the launch)
-    static std::atomic<uint64_t> done{0};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    const cudaError_t e = allow_dynamic_smem((const void*)gemm_bf16_tc_kernel<BN, MODE, KB>, smem);
     if (e != cudaSuccess) return e;
-    const uint64_t bit = 1ull << (dev & 63);
-    if (dev > 63 || !(done.load(std::memory_order_relaxed) & bit)) {
-        e = cudaFuncSetAttribute(gemm_bf16_tc_kernel<BN, MODE, KB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)TC_RING_ONE + 1024);
-        if (e != cudaSuccess) return e;
-        done.fetch_or(bit, std::memory_order_relaxed);
-    }
     const dim3 grid((a.N + BN - 1) / BN, (a.M + TC_BM - 1) / TC_BM);
     gemm_bf16_tc_kernel<BN, MODE, KB><<<grid, TC_THREADS, smem, s>>>(ma, mb, a);
     note_launches(1);

@@ -281,6 +281,31 @@ void stage_end(int stage, cudaStream_t s)
 }
 void note_launches(int64_t k) { g_launches.fetch_add(k, std::memory_order_relaxed); }
 void set_error(const char* msg) { g_err = msg; }
+cudaError_t allow_dynamic_smem(const void* kernel, size_t bytes)
+{
+    if (bytes <= 40 * 1024) return cudaSuccess;      // within the default limit with any kernel's static part
+    struct Entry { const void* kernel; int dev, most; };
+    static std::mutex mu;
+    static Entry known[512];
+    static int count = 0;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lk(mu);
+    int i = 0;
+    while (i < count && (known[i].kernel != kernel || known[i].dev != dev)) ++i;
+    if (i == count) {
+        cudaFuncAttributes fa;
+        int optin = 0;
+        if ((e = cudaFuncGetAttributes(&fa, kernel)) != cudaSuccess) return e;
+        if ((e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
+        const int most = optin - (int)fa.sharedSizeBytes;
+        if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most)) != cudaSuccess) return e;
+        if (count == (int)(sizeof known / sizeof known[0])) return bytes <= (size_t)most ? cudaSuccess : cudaErrorInvalidValue;
+        known[count++] = {kernel, dev, most};
+    }
+    return bytes <= (size_t)known[i].most ? cudaSuccess : cudaErrorInvalidValue;
+}
 long long wait_limit(long long dflt)
 {
     const long long v = g_wait_polls.load(std::memory_order_relaxed);

@@ -108,6 +108,12 @@ void stage_begin(int stage, cudaStream_t s);
 void stage_end(int stage, cudaStream_t s);
 void note_launches(int64_t k);
 void set_error(const char* msg);      // message returned by pcv_last_error
+// Lets `kernel` be launched with `bytes` of dynamic shared memory (error where
+// the device cannot).  The limit belongs to the function, not to the launch: it
+// is raised once per device, to all a block can have, and never lowered, so
+// that a small call of one thread cannot come between another's large one and
+// its launch.
+cudaError_t allow_dynamic_smem(const void* kernel, size_t bytes);
 // Bound of one mbarrier wait in the tensor-core kernels: `dflt` unless
 // pcv_set_wait_limit set another.
 long long wait_limit(long long dflt);

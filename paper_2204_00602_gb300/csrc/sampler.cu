@@ -397,9 +397,7 @@ cudaError_t launch_sampler(const Plan& p, const double2* U, const uint8_t* perm,
         // samples per SM as shared memory holds
         auto go = [&](auto kernel, int threads, int samples) {
             const size_t smem = (size_t)samples * subset_bytes(p.m, p.n);
-            cudaError_t r = cudaSuccess;
-            if (smem > 48 * 1024)
-                r = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            cudaError_t r = allow_dynamic_smem((const void*)kernel, smem);
             if (r != cudaSuccess) return r;
             for (int64_t c0 = 0; c0 < count && r == cudaSuccess; c0 += 1 << 30) {      // grid limit
                 SampArgs p1 = a;
@@ -427,9 +425,7 @@ cudaError_t launch_sampler(const Plan& p, const double2* U, const uint8_t* perm,
     }
     const size_t smem = (size_t)p.m * p.n * sizeof(double2);
     const unsigned blocks = (unsigned)((count + kSampWarps - 1) / kSampWarps);
-    if (smem > 48 * 1024 &&
-        (e = cudaFuncSetAttribute(sampler_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-        return e;
+    if ((e = allow_dynamic_smem((const void*)sampler_kernel<16>, smem)) != cudaSuccess) return e;
     sampler_kernel<16><<<blocks, 32 * kSampWarps, smem, s>>>(a);
     note_launches(1);
     return cudaGetLastError();

@@ -139,11 +139,8 @@ template <int KMAX, int GROUP, typename I>
 cudaError_t launch_one(const ExpandArgs& a, cudaStream_t s)
 {
     const size_t smem = (size_t)GROUP * a.m * sizeof(double2) + (size_t)(a.m + 1) * (a.k + 1) * sizeof(I);
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(expand_kernel<KMAX, GROUP, I>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = allow_dynamic_smem((const void*)expand_kernel<KMAX, GROUP, I>, smem);
+    if (e != cudaSuccess) return e;
     const dim3 grid((unsigned)((a.hi - a.lo + kThreads - 1) / kThreads), (unsigned)((a.B + GROUP - 1) / GROUP));
     return launch_level_kernel(expand_kernel<KMAX, GROUP, I>, grid, kThreads, smem, s, a);
 }
@@ -350,9 +347,7 @@ cudaError_t launch_slos(const Plan& p, int B, const double2* U, int64_t lo, int6
         sm.status = (int64_t*)status;
         for (int j = 0; j <= 16; ++j) sm.sqrtfact[j] = d.sqrtfact[j];
         auto go = [&](auto kernel) {
-            cudaError_t e = cudaSuccess;
-            if (smem > 48 * 1024)
-                e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            const cudaError_t e = allow_dynamic_smem((const void*)kernel, smem);
             if (e != cudaSuccess) return e;
             kernel<<<B, kThreads, smem, s>>>(sm);
             note_launches(1);

@@ -427,11 +427,8 @@ cudaError_t go_split(const SplitArgs& a, cudaStream_t s)
 template <int NMAX>
 cudaError_t go_multi(const SplitMultiArgs& a, size_t smem, cudaStream_t s)
 {
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(split_multi_kernel<NMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = allow_dynamic_smem((const void*)split_multi_kernel<NMAX>, smem);
+    if (e != cudaSuccess) return e;
     const dim3 grid((unsigned)((a.o.n_out + a.per_block - 1) / a.per_block), (unsigned)((a.B + kMulti - 1) / kMulti));
     split_multi_kernel<NMAX><<<grid, kThreads, smem, s>>>(a);
     note_launches(1);
