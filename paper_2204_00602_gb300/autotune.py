@@ -1,9 +1,10 @@
 """Autotuner for explicit-output amplitude calls.
 
 For a problem shape (m, n, number of outputs) it times every applicable
-kernel configuration of pcv_amplitudes_ex on the GPU with CUDA events —
-threads per permanent G in {1, 2, 4, 8, 16, 32} for the group kernel, the
-shared-row-sum tile kernel, and blocks per permanent for the block kernel —
+kernel configuration of pcv_amplitudes_ex on the GPU with CUDA events — the
+library's own choice (two half expansions and split tiles are reached through
+it alone), threads per permanent G in {1, 2, 4, 8, 16, 32} for the group kernel,
+the shared-row-sum tile kernel, and blocks per permanent for the block kernel —
 and keeps the fastest in a JSON table keyed by (n, m bucket, n_out bucket).
 `amplitudes_tuned` looks the table up (tuning on a miss) and calls the chosen
 configuration.
@@ -18,7 +19,7 @@ import threading
 import numpy as np
 import torch
 
-from . import PCV_ALGO_BLOCK, PCV_ALGO_GROUP, PCV_ALGO_TILE, amplitudes
+from . import PCV_ALGO_AUTO, PCV_ALGO_BLOCK, PCV_ALGO_GROUP, PCV_ALGO_TILE, amplitudes
 
 _lock = threading.Lock()
 DEFAULT_PATH = os.path.join(os.path.expanduser("~"), ".cache", "pcv", "autotune.json")
@@ -33,7 +34,7 @@ def key(m: int, n: int, n_out: int) -> str:
 
 
 def candidates(m: int, n: int, n_out: int):
-    out = []
+    out = [(PCV_ALGO_AUTO, 0)]
     if 1 <= n <= 16:
         for G in (1, 2, 4, 8, 16, 32):
             if G <= 2 ** (n - 1):
