@@ -177,7 +177,9 @@ int64_t pcv_amplitudes_batched_workspace(int n_circ, int64_t total_outputs);
 /* Amplitudes of many circuits of uneven size (Eq. eqperm per circuit).
  * A routing kernel sends each output either to the shared-row-sum tile
  * kernel or to Glynn's sum with multiplicities (PCV_ALGO_MULT), whichever
- * takes less time for it; a planning kernel sorts the circuits
+ * takes less time for it (the outputs of a circuit's last, partly filled warp
+ * of a tile go to the second only where its single warps end soon beside the
+ * rest of the batch); a planning kernel sorts the circuits
  * by photon number (largest first) and expands them into tile items
  * (circuit, tile of 32..256 outputs, part of the sign vectors: no item holds
  * more than a twelfth of an SM's share of the tile work, given the workspace
@@ -185,8 +187,8 @@ int64_t pcv_amplitudes_batched_workspace(int n_circ, int64_t total_outputs);
  * parts' sums, 12 bytes per output and 48 per circuit and more, keeps whole
  * tiles) and single-output entries.  Two
  * persistent launches then pull from device counters until their queues are
- * empty: blocks take tile items, warps take entries.  No block waits on
- * another.
+ * empty: blocks take tile items, and the one that ends a tile's last part adds
+ * the parts; warps take entries.  No block waits on another.
  *   descs          device, n_circ descriptors (see pcv_batch_desc)
  *   total_outputs  sum of n_out over the circuits (<= INT32_MAX; sizes the
  *                  work lists)

@@ -45,9 +45,13 @@ constexpr int kLow = 4;              // columns kept in shared memory (flipped w
 constexpr int kMinTile = 32;
 constexpr int kPack = 512;           // a circuit's tile size and parts in one int: T + kPack parts
 constexpr int kItemsPerSm = 12;      // a batched item holds at most 1 / (kItemsPerSm sms) of the tile work
-constexpr int kPartSteps = 64;       // sign vectors per split that a part keeps
-constexpr int kStageOne = 3072;      // the same for one circuit (48 KB: eight steps of 324 modes)
+constexpr int kPartSteps = 64;       // sign vectors per split that a part keeps,
+constexpr int kLeastSteps = 8;       // or where that leaves SMs idle: parts up to kLightPerSm blocks per SM
+constexpr int kLightPerSm = 2;
+constexpr float kEntryStart = 2e4f;  // cycles of a multiplicity entry on its warp: at first,
+constexpr float kEntryCycles = 100;  // and per FP64 instruction
 constexpr int kStage = 2560;         // staged row sums of a batched block (40 KB: three blocks per SM)
+constexpr int kStageOne = 3072;      // the same for one circuit (48 KB: eight steps of 324 modes)
 
 // A block's work: outputs and shape of the tile, the part of the sequence.
 struct TileShape {
@@ -356,8 +360,8 @@ __global__ void __launch_bounds__(kThreads, 2) glynn_tile_kernel(const __grid_co
 __device__ void add_parts(const pcv_batch_desc& c, const double2* partial, int parts, const int* idx, int64_t count,
                           int64_t pos)
 {
-    double2 v = partial[pos];
-    for (int q = 1; q < parts; ++q) v = cadd(v, partial[(int64_t)q * count + pos]);
+    double2 v = __ldcg(partial + pos);          // of other blocks: not from this SM's cache
+    for (int q = 1; q < parts; ++q) v = cadd(v, __ldcg(partial + (int64_t)q * count + pos));
     const int64_t o = idx ? idx[pos] : pos;
     if (c.amp) ((double2*)c.amp)[o] = v;
     if (c.prob) c.prob[o] = fma(v.x, v.x, v.y * v.y);
@@ -384,6 +388,7 @@ struct Queue {
     int* shape;               // of circuit c: outputs per tile + kPack * parts (blocks per sequence)
     int64_t* slot_off;        // circuit c's first partial sum (parts > 1)
     double2* partial;         // null: every sequence in one part
+    int* done;                // finished parts of a tile, at its first item
 };
 
 __device__ TileShape batch_shape(const pcv_batch_desc& d, int T, int parts)
@@ -399,7 +404,7 @@ __device__ TileShape batch_shape(const pcv_batch_desc& d, int T, int parts)
 __global__ void __launch_bounds__(kThreads, 2) glynn_persistent_kernel(const pcv_batch_desc* descs, Queue q)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ int s_item;
+    __shared__ int s_item, s_done;
     const int total = *q.total;
     for (;;) {
         if (threadIdx.x == 0) s_item = atomicAdd(q.counter, 1);
@@ -407,19 +412,24 @@ __global__ void __launch_bounds__(kThreads, 2) glynn_persistent_kernel(const pcv
         const int it = s_item;
         __syncthreads();
         if (it >= total) break;
-        const int c = q.item_circ[it], parts = q.shape[c] / kPack;
+        const int c = q.item_circ[it], T = q.shape[c] % kPack, parts = q.shape[c] / kPack;
+        const int tile = q.item_tile[it] / parts, part = q.item_tile[it] % parts;
         const TileOut out{(const double2*)descs[c].U, (double2*)descs[c].amp, descs[c].prob};
-        tile_item(descs[c], out, batch_shape(descs[c], q.shape[c] % kPack, parts), q.item_tile[it] / parts, q.item_tile[it] % parts, smem,
-                  q.idx + q.out_off[c], q.n_tile[c], parts > 1 ? q.partial + q.slot_off[c] : nullptr);
+        double2* partial = parts > 1 ? q.partial + q.slot_off[c] : nullptr;
+        tile_item(descs[c], out, batch_shape(descs[c], T, parts), tile, part, smem, q.idx + q.out_off[c], q.n_tile[c], partial);
+        if (parts == 1) continue;
+        // the block that finishes a tile's last part adds them all, in part order
+        // (a launch of its own for that took 3 us of a small batch's 50)
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0) s_done = atomicAdd(q.done + (it - part), 1);
+        __syncthreads();
+        if (s_done + 1 < parts) continue;
+        __threadfence();
+        const int64_t pos = (int64_t)tile * T + threadIdx.x;
+        if (threadIdx.x < T && pos < q.n_tile[c])
+            add_parts(descs[c], partial, parts, q.idx + q.out_off[c], q.n_tile[c], pos);
     }
-}
-
-__global__ void __launch_bounds__(kThreads) batched_parts_kernel(const pcv_batch_desc* descs, Queue q)
-{
-    const int c = blockIdx.x, parts = q.shape[c] / kPack;
-    if (parts <= 1) return;
-    for (int64_t pos = (int64_t)blockIdx.y * kThreads + threadIdx.x; pos < q.n_tile[c]; pos += (int64_t)gridDim.y * kThreads)
-        add_parts(descs[c], q.partial + q.slot_off[c], parts, q.idx + q.out_off[c], q.n_tile[c], pos);
 }
 
 // A descriptor the kernels cannot run (n or m out of range, an input mode
@@ -521,11 +531,11 @@ __device__ double output_mult_cost(const pcv_batch_desc& c, int64_t o, const int
 // One block per circuit: route each output to the tile kernel or to Glynn's
 // sum with multiplicities; idx[out_off[c] ..] lists the tile outputs first
 // (in order) and the others after them (in reverse order).  A warp of a tile
-// costs as much with one live output as with 32 of them, so the outputs of a
-// last, partly filled warp are re-routed when they cost less on the
-// multiplicity kernel than the whole warp.
+// costs as much with one live output as with 32 of them: rest[c] holds what the
+// outputs of a last, partly filled warp cost on the multiplicity kernel, all and
+// the dearest, and plan_kernel decides about them.
 __global__ void __launch_bounds__(256) classify_kernel(const pcv_batch_desc* descs, const int64_t* out_off, int route,
-                                                       int64_t cap, int* idx, int* n_tile, int* n_mult)
+                                                       int64_t cap, int* idx, int* n_tile, int* n_mult, float2* rest)
 {
     __shared__ int buf[64];
     __shared__ int s_tile, s_mult;
@@ -533,7 +543,10 @@ __global__ void __launch_bounds__(256) classify_kernel(const pcv_batch_desc* des
     const pcv_batch_desc& c = descs[ci];
     const bool valid = desc_ok(c) && out_off[ci] + c.n_out <= cap;
     if (!valid) {
-        if (threadIdx.x == 0) n_tile[ci] = n_mult[ci] = 0;
+        if (threadIdx.x == 0) {
+            n_tile[ci] = n_mult[ci] = 0;
+            rest[ci] = make_float2(0.0f, 0.0f);
+        }
         return;
     }
     const int n = c.n;
@@ -576,33 +589,21 @@ __global__ void __launch_bounds__(256) classify_kernel(const pcv_batch_desc* des
         }
         __syncthreads();
     }
-    if (route == PCV_ALGO_AUTO) {
-        const int tilesz = kMinTile;
-        const int r = s_tile % tilesz;
-        if (r > 0) {
-            // the last r tile outputs sit just below the multiplicity outputs
-            // in the list; moving the boundary re-routes them
-            double part = 0.0;
-            for (int k = threadIdx.x; k < r; k += blockDim.x)
-                part += output_mult_cost(c, list[s_tile - r + k], imu, d_in);
-            for (int off = 16; off > 0; off >>= 1) part += __shfl_xor_sync(0xffffffffu, part, off);
-            __shared__ double wsum[8];
-            if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = part;
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                double tot = 0.0;
-                for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += wsum[w];
-                if (tot < ct * tilesz) {
-                    s_tile -= r;
-                    s_mult += r;
-                }
-            }
-            __syncthreads();
+    if (threadIdx.x < 32) {
+        // the last r tile outputs sit just below the multiplicity outputs in the
+        // list; moving the boundary re-routes them
+        const int r = route == PCV_ALGO_AUTO ? s_tile % kMinTile : 0;
+        const float cost = (int)threadIdx.x < r ? (float)output_mult_cost(c, list[s_tile - r + threadIdx.x], imu, d_in) : 0.0f;
+        float sum = cost, most = cost;
+        for (int off = 16; off > 0; off >>= 1) {
+            sum += __shfl_xor_sync(0xffffffffu, sum, off);
+            most = fmaxf(most, __shfl_xor_sync(0xffffffffu, most, off));
         }
-    }
-    if (threadIdx.x == 0) {
-        n_tile[ci] = s_tile;
-        n_mult[ci] = s_mult;
+        if (threadIdx.x == 0) {
+            n_tile[ci] = s_tile;
+            n_mult[ci] = s_mult;
+            rest[ci] = make_float2(sum, most);
+        }
     }
 }
 
@@ -628,16 +629,28 @@ __device__ int pick_tile(int m, int n, int count)
 // circuits by n (descending), then tile items and multiplicity entries in
 // that order.  A tile's sequence is split in parts so that
 // no item holds more than 1 / (kItemsPerSm sms) of all tile work; a part
-// keeps at least kPartSteps sign vectors per split.
+// keeps at least kPartSteps sign vectors per split, as its start takes some 30 us
+// (kLeastSteps everywhere: 31 circuits of 90 outputs, n <= 15, 300 to 400 us), or
+// kLeastSteps up to kLightPerSm items per SM (3 circuits of 17 outputs, n = 10:
+// 200 to 77 us).
+//
+// The outputs of a partly filled warp go to the multiplicity kernel when that
+// costs less than the warp and takes no longer, each permanent on one warp after
+// the tiles are done, than 1/32 of the time of all tiles (kEntryCycles per FP64
+// instruction of a lane, kEntryStart at first: n = 10 to 20; a tile product 20
+// cycles of an SM).  Decided by the cost alone, 48 circuits of n = 4 to 16 took 4.87
+// ms at 100 outputs each (0.91 so), 6.79 at 513 (3.77), and 3.1 at 512.
 __global__ void __launch_bounds__(1024) plan_kernel(const pcv_batch_desc* descs, int n_circ, Queue q, MultQueue mq,
-                                                    int* order, int* item_off, int* mult_off, const int* n_mult,
-                                                    int* mult_circ, int* mult_out, int max_items, int sms)
+                                                    int* order, int* item_off, int* mult_off, int* n_tile, int* n_mult,
+                                                    const float2* rest, int* mult_circ, int* mult_out, int max_items,
+                                                    int sms)
 {
     __shared__ int bucket[PCV_MAX_PHOTONS + 2];
     __shared__ int cursor[PCV_MAX_PHOTONS + 2];
     __shared__ int buf[64];
     __shared__ int64_t buf64[64];
     __shared__ double s_work[32];
+    __shared__ float s_total;
     __shared__ int carry_t, carry_m;
     __shared__ int64_t carry_s;
     const int tid = threadIdx.x;
@@ -645,17 +658,41 @@ __global__ void __launch_bounds__(1024) plan_kernel(const pcv_batch_desc* descs,
     __syncthreads();
     for (int c = tid; c < n_circ; c += blockDim.x)
         atomicAdd(&bucket[desc_ok(descs[c]) ? descs[c].n : 0], 1);
-    // tile sizes and all tile work (n products per lane and sign vector)
-    double work = 0.0;
+    // tile sizes and all tile work (n products per lane and sign vector), before
+    // and after the partly filled warps' outputs find their kernel; few threads
+    // touch FP64, of which an SM issues an instruction per 16 cycles
+    auto tile_work = [&] {
+        double work = 0.0;
+        for (int c = tid; c < n_circ; c += blockDim.x) {
+            const int cnt = n_tile[c];
+            const int T = cnt > 0 ? pick_tile(descs[c].m, descs[c].n, cnt) : kThreads;
+            q.shape[c] = T;
+            if (cnt > 0) work += ldexp((double)((cnt + T - 1) / T) * T * descs[c].n, descs[c].n - 1);
+        }
+        if (tid / 32 * 32 < n_circ)
+            for (int off = 16; off > 0; off >>= 1) work += __shfl_xor_sync(0xffffffffu, work, off);
+        if ((tid & 31) == 0) s_work[tid >> 5] = work;
+        __syncthreads();
+        if (tid < 32) {
+            work = s_work[tid];
+            for (int off = 16; off > 0; off >>= 1) work += __shfl_xor_sync(0xffffffffu, work, off);
+            if (tid == 0) s_total = (float)work;
+        }
+        __syncthreads();
+    };
+    tile_work();
+    const float patience = s_total * (20.0f / 32.0f / 32.0f) / (float)sms;       // cycles
+    bool moved = false;
     for (int c = tid; c < n_circ; c += blockDim.x) {
-        const int cnt = q.n_tile[c];
-        const int T = cnt > 0 ? pick_tile(descs[c].m, descs[c].n, cnt) : kThreads;
-        q.shape[c] = T;
-        if (cnt > 0) work += ldexp((double)((cnt + T - 1) / T) * T * descs[c].n, descs[c].n - 1);
+        const float2 r = rest[c];
+        if (r.x > 0.0f && kEntryStart + r.y * (kEntryCycles / 32.0f) <= patience && r.x < kMinTile * tile_cost(descs[c].n)) {
+            const int cnt = n_tile[c] % kMinTile;
+            n_tile[c] -= cnt;
+            n_mult[c] += cnt;
+            moved = true;
+        }
     }
-    for (int off = 16; off > 0; off >>= 1) work += __shfl_xor_sync(0xffffffffu, work, off);
-    if ((tid & 31) == 0) s_work[tid >> 5] = work;
-    __syncthreads();
+    if (__syncthreads_or(moved)) tile_work();
     if (tid == 0) {
         int acc = 0;
         for (int n = PCV_MAX_PHOTONS; n >= 0; --n) { cursor[n] = acc; acc += bucket[n]; }
@@ -663,17 +700,16 @@ __global__ void __launch_bounds__(1024) plan_kernel(const pcv_batch_desc* descs,
         carry_s = 0;
     }
     __syncthreads();
-    work = 0.0;
-    for (int w = 0; w < 32; ++w) work += s_work[w];
-    const double most = work / ((double)sms * kItemsPerSm);
+    const float most = s_total / ((float)sms * kItemsPerSm);
     for (int c = tid; c < n_circ; c += blockDim.x) {
         order[atomicAdd(&cursor[desc_ok(descs[c]) ? descs[c].n : 0], 1)] = c;
         int parts = 1;
         if (q.partial && q.n_tile[c] > 0) {
             const int n = descs[c].n;
-            const int64_t room = (1ll << (n - 1)) / ((int64_t)(kThreads / q.shape[c]) * kPartSteps);
-            const double item = ldexp((double)q.shape[c] * n, n - 1);
-            parts = (int)fmax(1.0, fmin((double)room, ceil(item / most)));
+            const float vectors = ldexpf((float)q.shape[c] / kThreads, n - 1);       // of a split
+            const float item = ldexpf((float)(q.shape[c] * n), n - 1) / most;
+            parts = (int)fmaxf(1.0f, fmaxf(fminf(vectors / kPartSteps, ceilf(item)),
+                                           fminf(vectors / kLeastSteps, item * (kLightPerSm / (float)kItemsPerSm))));       // rounded down: one wave
         }
         q.shape[c] += kPack * parts;
     }
@@ -726,6 +762,7 @@ __global__ void __launch_bounds__(1024) plan_kernel(const pcv_batch_desc* descs,
             if (it < max_items) {
                 q.item_circ[it] = c;
                 q.item_tile[it] = t;
+                if (q.partial) q.done[it] = 0;
             }
         }
         const int cm = n_mult[c];
@@ -768,8 +805,8 @@ TileShape pick_shape(int m, int n, int64_t n_out, int B, bool split)
     // the staged sums: up to kMaxChunk steps within 48 KB, one step at least
     t.stage = std::max(std::max(kThreads, S * t.slots), std::min(kStageOne, S * t.slots * kMaxChunk));
     const int64_t tiles = (n_out + t.T - 1) / t.T * B;
-    const int64_t room = (1ll << (n - 1)) / ((int64_t)S * kPartSteps);
-    if (split) t.parts = (int)std::max<int64_t>(1, std::min<int64_t>(room, 152 * 2 / tiles));
+    const int64_t room = (1ll << (n - 1)) / ((int64_t)S * kLeastSteps);
+    if (split) t.parts = (int)std::max<int64_t>(1, std::min<int64_t>(room, 152 * kLightPerSm / tiles));
     return t;
 }
 
@@ -863,7 +900,7 @@ int64_t batched_workspace(int n_circ, int64_t total_outputs)
 int64_t batched_workspace_full(int n_circ, int64_t total_outputs)
 {
     return batched_workspace(n_circ, total_outputs) +
-           (int64_t)(al256((size_t)n_circ * sizeof(int64_t)) + 2 * al256((size_t)split_items(n_circ, total_outputs) * sizeof(int)) +
+           (int64_t)(al256((size_t)n_circ * sizeof(int64_t)) + 3 * al256((size_t)split_items(n_circ, total_outputs) * sizeof(int)) +
                      al256((size_t)split_slots(n_circ, total_outputs) * sizeof(double2)));
 }
 
@@ -899,11 +936,13 @@ cudaError_t launch_glynn_batched(const pcv_batch_desc* descs, int n_circ, int64_
     q.shape = shapes;
     q.slot_off = nullptr;
     q.partial = nullptr;
+    q.done = nullptr;
     if (ws_bytes >= batched_workspace_full(n_circ, total_outputs) && sms <= kPlanSms) {
         max_items = split_items(n_circ, total_outputs);
         q.slot_off = (int64_t*)w;                     w += al256((size_t)n_circ * sizeof(int64_t));
         q.item_circ = (int*)w;                        w += al256((size_t)max_items * sizeof(int));
         q.item_tile = (int*)w;                        w += al256((size_t)max_items * sizeof(int));
+        q.done = (int*)w;                             w += al256((size_t)max_items * sizeof(int));
         q.partial = (double2*)w;
     }
     MultQueue mq;
@@ -913,9 +952,11 @@ cudaError_t launch_glynn_batched(const pcv_batch_desc* descs, int n_circ, int64_
     mq.out = mult_out;
 
     offsets_kernel<<<1, 1024, 0, s>>>(descs, n_circ, out_off);
-    classify_kernel<<<n_circ, 256, 0, s>>>(descs, out_off, route, total_outputs, idx, n_tile, n_mult);
-    plan_kernel<<<1, 1024, 0, s>>>(descs, n_circ, q, mq, order, item_off, mult_off, n_mult, mult_circ, mult_out,
-                                   (int)max_items, sms);
+    // the lists that plan_kernel fills last hold its input until then
+    float2* rest = (float2*)item_off;
+    classify_kernel<<<n_circ, 256, 0, s>>>(descs, out_off, route, total_outputs, idx, n_tile, n_mult, rest);
+    plan_kernel<<<1, 1024, 0, s>>>(descs, n_circ, q, mq, order, item_off, mult_off, n_tile, n_mult, rest, mult_circ,
+                                   mult_out, (int)max_items, sms);
     note_launches(3);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     int per_sm = 0;
@@ -924,10 +965,6 @@ cudaError_t launch_glynn_batched(const pcv_batch_desc* descs, int n_circ, int64_
     if (per_sm < 1) per_sm = 1;
     glynn_persistent_kernel<<<sms * per_sm, kThreads, smem, s>>>(descs, q);
     note_launches(1);
-    if (q.partial) {
-        batched_parts_kernel<<<dim3((unsigned)n_circ, 16), kThreads, 0, s>>>(descs, q);
-        note_launches(1);
-    }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     return launch_glynn_mult_persistent(descs, mq, sms, s);
 }

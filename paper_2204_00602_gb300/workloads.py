@@ -67,7 +67,8 @@ def routed_fp64_instructions(m: int, n: int, outs: np.ndarray):
     mult = np.minimum(cost_out, cost_in)
     to_mult = mult < tile
     # the outputs of a last, partly filled warp go to the multiplicity kernel when
-    # they cost less there than the whole warp (as the routing kernel does)
+    # they cost less there than the whole warp (as the planning kernel does where the
+    # batch is long beside one of them)
     tile_idx = np.flatnonzero(~to_mult)
     tsz = 32
     r = len(tile_idx) % tsz
