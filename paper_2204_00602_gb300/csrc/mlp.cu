@@ -233,15 +233,28 @@ __global__ void __launch_bounds__(64) colsum_bf16_kernel(const __grid_constant__
     }
 }
 
-// Sine and cosine in FP64 from a table of 64 points of the circle: x = k h + r,
-// h = 2 pi / 64, |r| <= h / 2, then the addition theorem with Taylor's
-// polynomials in r (the next terms, r^9 / 9! and r^10 / 10!, are below 5e-18):
-// 18 FP64 instructions for both, where sin() and cos() take about 60 and bound
-// the kernel (4096 x 132 phases: 52 us).  Error below 3e-16, as a float the
-// same value but once in 1e8.
+// Whether x lies within `units` of its last place of the middle between two
+// neighbouring floats (29 bits fewer): only there can an error of that size change
+// the float it rounds to.
+__device__ __forceinline__ bool near_float_middle(double x, uint32_t units)
+{
+    return (((uint32_t)__double2loint(x) - (0x10000000u - units)) & 0x1FFFFFFFu) <= 2 * units;
+}
+
+// Sine and cosine, to be rounded to floats, from a table of 64 points of the
+// circle: x = k h + r, h = 2 pi / 64, |r| <= h / 2, then the addition theorem with
+// Taylor's polynomials in r (the next terms, r^9 / 9! and r^10 / 10!, are below
+// 5e-18): 18 FP64 instructions for both, where sin() and cos() take about 60 and
+// bound the kernel (4096 x 132 phases: 52 us).  The error is below 3e-16: 43
+// units of the last place of the least value but those within h / 2 of a zero,
+// where the table's entry is exactly 0 and r's reduction errs by at most 632 units
+// (over all doubles below 1024 in magnitude).  Where that could change the float,
+// and beyond 1024, sincos(): the floats are those of the FP64 functions.  One
+// phase in 700,000 takes that way (2048 units for all, one in 65,000: a training
+// step of 4,096 rows took 1 us longer).
 __device__ __forceinline__ void sincos_table(double x, const double2* tab, double& s, double& c)
 {
-    if (!(fabs(x) < 1e6)) {
+    if (!(fabs(x) < 1024.0)) {
         sincos(x, &s, &c);
         return;
     }
@@ -258,6 +271,8 @@ __device__ __forceinline__ void sincos_table(double x, const double2* tab, doubl
     const double2 e = tab[k & 63];
     s = e.x + fma(e.x, cm, e.y * sr);
     c = e.y + fma(e.y, cm, -(e.x * sr));
+    const uint32_t units = k & 15 ? 64 : 2048;
+    if (near_float_middle(s, units) || near_float_middle(c, units)) sincos(x, &s, &c);
 }
 
 // x = [sin phi, cos phi, 1, 0...] (bf16, row length ldx).  A thread takes both
@@ -414,7 +429,9 @@ __global__ void f32_to_bf16_kernel(const float* __restrict__ in, int64_t count, 
 // |r| <= 2^-8 + 2^-16, log in = e ln 2 - log c + log1p(r), the series up to r^6
 // (the next term is below 2^-58): 12 FP64 instructions against about 28 (1 M
 // values: 60 us before).  Near 1, where those terms cancel, and outside the
-// normal range: log().
+// normal range: log().  Elsewhere the error is below 3e-16 + 2^-53 |log in|, at
+// most 175 units of the last place, so log() where that could change the float:
+// the floats are those of the FP64 function.
 __global__ void __launch_bounds__(256) log_f64_to_f32_kernel(const double* __restrict__ in, int64_t count,
                                                              float* __restrict__ out)
 {
@@ -437,7 +454,7 @@ __global__ void __launch_bounds__(256) log_f64_to_f32_kernel(const double* __res
         q = fma(r, q, -0.5);
         q = fma(r * r, q, r);
         double y = fma(e, 0.69314718055994530942, t.y) + q;
-        if (hi < 0 || ef == 0 || ef == 0x7FF || fabs(y) < 0.01) y = log(x);
+        if (hi < 0 || ef == 0 || ef == 0x7FF || fabs(y) < 0.01 || near_float_middle(y, 256)) y = log(x);
         out[i] = (float)y;
     }
 }
