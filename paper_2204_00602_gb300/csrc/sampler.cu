@@ -24,8 +24,9 @@
 //                          (n = 14: 0.46 M against 1.6 M), and no sign
 //                          cancellation.  From n = 10 on the levels are in
 //                          fixed point on the integer pipe (16,384 samples of
-//                          n = 14: 17.3 to 10.8 ms; the FP64 pipe took 12.5 of
-//                          it).  Two neighbouring levels live in
+//                          n = 14: 17.3 to 10.6 ms; the FP64 pipe took 12.5 of
+//                          it), but for samples that need the range
+//                          of FP64.  Two neighbouring levels live in
 //                          shared memory (n = 14: 103 KB, two samples per SM;
 //                          n = 15: 206 KB), which ends the form at n = 15;
 //   sampler_kernel         n = 16: one Glynn sum per step (below), one warp
@@ -58,8 +59,8 @@ struct SampArgs {
 };
 
 // Inverse-CDF draw by one warp from the weights of its lanes (wloc[c]: mode
-// lane + 32 c; the cumulative order runs lane by lane), u in [0, 1).
-__device__ int draw_mode(const double* wloc, int m, double u)
+// lane + 32 c; the cumulative order runs lane by lane), u in [0, 1); total: their sum.
+__device__ int draw_mode(const double* wloc, int m, double u, double& total)
 {
     const int lane = threadIdx.x & 31;
     double part = 0.0;
@@ -71,7 +72,7 @@ __device__ int draw_mode(const double* wloc, int m, double u)
         const double v = __shfl_up_sync(0xffffffffu, incl, off);
         if (lane >= off) incl += v;
     }
-    const double total = __shfl_sync(0xffffffffu, incl, 31);
+    total = __shfl_sync(0xffffffffu, incl, 31);
     const double target = u * total;
     // the lane whose cumulative range holds the target picks within its modes
     const double before = incl - part;
@@ -111,11 +112,11 @@ __host__ __device__ inline int subset_level(int n, int odd)
 }
 
 // Shared memory of one sample: two levels, the drawn row, the sub-permanents of
-// the step, the weights, the sample's columns and rows.
+// the step, the weights, the sample's columns, rows and column exponents.
 __host__ __device__ inline size_t subset_bytes(int m, int n)
 {
     return (size_t)(subset_level(n, 0) + subset_level(n, 1) + 2 * n) * sizeof(double2) +
-           (size_t)(m + (m & 1)) * sizeof(double) + 3 * 16 * sizeof(int);      // a multiple of 16
+           (size_t)(m + (m & 1)) * sizeof(double) + 48 * sizeof(int);      // a multiple of 16
 }
 
 constexpr int kBinom = 17;
@@ -123,48 +124,102 @@ constexpr int kBinom = 17;
 // Position of the lowest bit (15 for none: a valid row of the tables).
 __device__ __forceinline__ int low_bit(uint32_t x) { return (__ffs((int)x) - 1) & 15; }
 
-// A group of T threads per sample (T = 32: several samples per block).  FIXED:
-// the levels in fixed point (fixed30.cuh), components at most 2^59.  A drawn row
-// is scaled by a power of two to 57 bits of its norm |a|, and with M the largest
-// component of level k - 1 a component of level k is below 2^57 M sqrt(2 k), which
-// gives the shift back; powers of two cancel in a draw, so no scale is kept.
-template <int T, bool FIXED>
-__global__ void subset_sampler_kernel(const __grid_constant__ SampArgs a)
+// x 2^e on the integer pipe: 0 below 2^-959, x itself beyond 2^961.
+__device__ __forceinline__ double times_pow2(double x, int e)
 {
-    extern __shared__ int4 s_mem[];
-    __shared__ int s_c[kBinom][kBinom];        // C(t, j)
-    for (int q = threadIdx.x; q < kBinom * kBinom; q += blockDim.x) {
-        const int t = q / kBinom, j = q % kBinom;
-        int c = j <= t ? 1 : 0;
-        for (int i = 1; i <= j && j <= t; ++i) c = c * (t + 1 - i) / i;
-        s_c[t][j] = c;
-    }
-    __syncthreads();
-    const int m = a.m, n = a.n;
-    const int grp = threadIdx.x / T, tid = threadIdx.x % T;
-    const int64_t smp = (int64_t)blockIdx.x * (blockDim.x / T) + grp;
-    if (smp >= a.count) return;                // whole groups
+    const int hi = __double2hiint(x), ex = (hi >> 20) & 0x7FF;
+    if (ex < 64) return 0.0;
+    return ex < 1984 ? __hiloint2double(hi + e * (1 << 20), __double2loint(x)) : x;
+}
+
+// |x| as a float but for its last three bits: 0 below FP32's range, infinity beyond.
+__device__ __forceinline__ float abs_float(double x)
+{
+    const int hi = __double2hiint(x) & 0x7FFFFFFF;
+    if (hi < 897 << 20) return 0.0f;
+    return hi < 1151 << 20 ? __int_as_float((hi - (896 << 20)) << 3) : INFINITY;
+}
+
+// Shift of level k's sums for top 2^29 the largest component of level k - 1.
+__device__ __forceinline__ int level_shift(float top, int k)
+{
+    return min(max(ilogbf(top * sqrtf(2.0f * k) * 1.0001f) - 2, 1), 30);
+}
+
+// One sample by a group of T threads, from the table c[t][j] = C(t, j).
+//
+// FIXED: the levels in fixed point (fixed30.cuh), components at most 2^59.  A
+// column is scaled by a power of two to a norm of 1/2 to 1 and a drawn row to 57
+// bits of its norm; with M the largest component of level k - 1 a component of
+// level k is below 2^57 M sqrt(2 k), which gives the shift back.  A factor common to
+// a step's weights cancels in the draw, so no scale is kept but the columns'.
+//
+// The entries of a level share one absolute error, of variance about
+//     var_k = var_{k-1} 4^{27 - sh} |row|^2 k / n + 1/2
+// (sh the shift; k of the row's n columns), and the weights' root one of k var.
+// Where that passes 2^-96 of their sum, false: nothing is written, and the sample
+// is drawn in FP64.  So it is where a column's norm is outside 2^-50 .. 2^50 or a
+// drawn row is not finite.  Emulated at n = 10 and 12, rare rows as often as
+// likely ones, the summed error of a step's probabilities is at most 2.4 times the
+// estimate or 6e-16, so at most 9e-15; Glynn's sums have 1.2e-14.  Haar matrices never
+// get there (80,000 samples of n = 10 to 15: 2^-100 at most); 8 samples in 10,000 of
+// exp(0.1 i H) at m=16 n=10 do, as a rare row leaves larger entries among the
+// columns not yet in use.  Without scales and check inputs with losses down to
+// 2^-29 gave other samples, and 1e-5 couplings probabilities off by 0.1 after rare
+// rows.
+template <int T, bool FIXED>
+__device__ __forceinline__ bool draw_sample(const SampArgs& a, int64_t smp, char* mem, const int (*s_c)[kBinom])
+{
+    const int m = a.m, n = a.n, tid = threadIdx.x % T;
     auto sync = [] {
         if (T == 32) __syncwarp();
         else __syncthreads();
     };
     const int n_even = subset_level(n, 0), n_odd = subset_level(n, 1);
     using Level = std::conditional_t<FIXED, int4, double2>;
-    Level* base = (Level*)((char*)s_mem + (size_t)grp * subset_bytes(m, n));
+    Level* base = (Level*)mem;
     Level* s_a = base + n_even + n_odd;         // A[r_k][.], the drawn row
     double2* s_g = (double2*)(s_a + n);        // entries 0 .. k of level k in FP64
     double* s_w = (double*)(s_g + n);
     int* s_pc = (int*)(s_w + m + (m & 1));               // input mode of each permuted photon
-    int* s_rows = s_pc + 16;
-    unsigned* s_top = (unsigned*)(s_rows + 16);          // of the odd and even levels: max |component| >> 29
-    unsigned* s_nan = s_top + 2;                         // a drawn row is not finite
-    if (tid == 0) *s_nan = 0;
+    int* s_rows = s_pc + 15;
+    int* s_e = s_rows + 15;                              // exponents of the columns' norms
+    unsigned* s_top = (unsigned*)(s_e + 15);             // of the odd and even levels: max |component| >> 29
+    unsigned* s_lost = s_top + 2;
+    if (FIXED && tid == 0) *s_lost = 0;
     if (tid < n) s_pc[tid] = a.cols[min((int)a.perm[smp * n + tid], n - 1)];   // clamp keeps reads in bounds
     sync();
+    if constexpr (FIXED) {
+        // squared norms of the columns, sixteen threads a row
+        float sum = 0.0f;
+        const double2* Uc = a.U + s_pc[tid % 16 < n ? tid % 16 : 0];
+#pragma unroll 8
+        for (int i = tid / 16; i < m; i += T / 16) {
+            const double2 u = __ldg(Uc + (size_t)i * m);
+            const float x = abs_float(u.x), y = abs_float(u.y);
+            sum = fmaf(x, x, fmaf(y, y, sum));
+        }
+        sum += __shfl_xor_sync(0xffffffffu, sum, 16);
+        float* s_sum = (float*)base;
+        if (tid % 32 < 16) s_sum[tid / 32 * 16 + tid % 16] = sum;
+        sync();
+        if (tid < n) {
+            sum = 0.0f;
+            for (int w = 0; w < T / 32; ++w) sum += s_sum[w * 16 + tid];
+            // 2^e at least the norm; one of 1 but for rounding counts as 1
+            s_e[tid] = ((__float_as_int(sum * (1.0f - 0x1p-10f)) >> 23) - 125) >> 1;
+            if (!(sum >= 0x1p-100f && sum <= 0x1p100f)) *s_lost = 1;
+        }
+        sync();
+        if (*s_lost) return false;
+    }
+    float var = 0.0f;                          // warp 0: of level k - 1
     for (int k = 1; k <= n; ++k) {
         // weights: sub-permanent of {0..k-1} \ l is entry k-1-l of level k-1
         const Level* f = base + ((k - 1) & 1 ? n_even : 0);         // level k - 1: even levels first, then odd
-        if (tid == 0) s_top[k & 1] = 0;
+        int sh = 1;                            // of level k
+        if (FIXED && k > 1) sh = level_shift((float)s_top[(k - 1) & 1] + 1.0f, k);
+        if (FIXED && tid == 0) s_top[k & 1] = 0;
         for (int i = tid; i < m; i += T) {
             const double2* Ui = a.U + (size_t)i * m;
             double2 s = make_double2(0.0, 0.0);
@@ -174,37 +229,39 @@ __global__ void subset_sampler_kernel(const __grid_constant__ SampArgs a)
                     if constexpr (FIXED) cmac(s, __ldg(Ui + s_pc[l]), s_g[k - 1 - l]);
                     else cmac(s, __ldg(Ui + s_pc[l]), f[k - 1 - l]);
                 }
-            s_w[i] = FIXED && *s_nan ? NAN : fma(s.x, s.x, s.y * s.y);
+            s_w[i] = fma(s.x, s.x, s.y * s.y);
         }
         sync();
         if (tid < 32) {
-            double wloc[4];
+            double wloc[4], total;
 #pragma unroll
             for (int c = 0; c < 4; ++c) wloc[c] = tid + 32 * c < m ? s_w[tid + 32 * c] : 0.0;
-            const int r = draw_mode(wloc, m, a.uni[smp * n + k - 1]);
+            const int r = draw_mode(wloc, m, a.uni[smp * n + k - 1], total);
             if (tid == 0) s_rows[k - 1] = r;
-            const double2 u = tid < n ? __ldg(a.U + (size_t)r * m + s_pc[tid]) : make_double2(0.0, 0.0);
+            double2 u = tid < n ? __ldg(a.U + (size_t)r * m + s_pc[tid]) : make_double2(0.0, 0.0);
             if constexpr (FIXED) {
+                if (k > 1 && !((float)total * 0x1p-96f >= (float)k * var) && tid == 0) *s_lost = 1;
+                if (tid < n) u = make_double2(times_pow2(u.x, -s_e[tid]), times_pow2(u.y, -s_e[tid]));
                 double sum = fma(u.x, u.x, u.y * u.y);
                 for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
-                if (!(sum <= DBL_MAX) && tid == 0) *s_nan = 1;
-                int e = 0;                         // 2^e at least the row's norm
-                if (sum > 0.0 && sum <= DBL_MAX) frexp(sqrt(sum) * (1.0 - 0x1p-20), &e);
-                const double sc = ldexp(1.0, 57 - e);
+                if (!(sum <= DBL_MAX) && tid == 0) *s_lost = 1;
+                // 2^e at least the row's norm but for 2^-17
+                const int e = sum > 0.0 ? (((__double2hiint(sum) - 16) >> 20) - 1021) >> 1 : 0;
+                const double sc = __hiloint2double((1023 + 57 - e) << 20, 0);
                 if (tid < n) s_a[tid] = split30(__double2ll_rn(u.x * sc), __double2ll_rn(u.y * sc));
+                if (k > 1) var *= __int_as_float((127 + 2 * (27 - sh)) << 23) * (float)times_pow2(sum, -2 * e) * ((float)k / (float)n);
+                var += 0.5f;
             } else if (tid < n) {
                 s_a[tid] = u;
             }
         }
         sync();
+        if (FIXED && *s_lost) return false;
         if (k == n) break;
         // level k: contiguous runs of subsets (increasing masks) per thread.
         // The rank of S is sum_i C(s_i, i + 1) over its elements in order;
         // without s_j the elements after it move down one place.
         Level* cur = base + (k & 1 ? n_even : 0);
-        int sh = 1;
-        if (FIXED && k > 1)
-            sh = min(max(ilogbf(((float)s_top[(k - 1) & 1] + 1.0f) * sqrtf(2.0f * k) * 1.0001f) - 2, 1), 30);
         unsigned top = 0;
         const int cnt = s_c[n][k];
         const int below = s_c[n][k - 1];       // entries of level k - 1
@@ -241,7 +298,8 @@ __global__ void subset_sampler_kernel(const __grid_constant__ SampArgs a)
                     const long long vx = k == 1 ? join30(row.x, row.y) : re.value(sh);
                     const long long vy = k == 1 ? join30(row.z, row.w) : im.value(sh);
                     cur[q] = split30(vx, vy);
-                    if (q <= k) s_g[q] = make_double2((double)vx, (double)vy);
+                    if (q <= k)                // the subset without column k - q
+                        s_g[q] = make_double2(times_pow2((double)vx, -s_e[k - q]), times_pow2((double)vy, -s_e[k - q]));
                     top = max(top, (unsigned)max(llabs(vx) >> 29, llabs(vy) >> 29));
                 } else {
                     cur[q] = k == 1 ? row : acc;
@@ -262,6 +320,42 @@ __global__ void subset_sampler_kernel(const __grid_constant__ SampArgs a)
         int c = 0;
         for (int p = 0; p < n; ++p) c += s_rows[p] == i;
         a.out[smp * m + i] = (uint8_t)c;
+    }
+    return true;
+}
+
+// Not inlined, so that it costs the fixed-point form no registers.
+template <int T>
+__device__ __noinline__ void draw_sample_fp64(const SampArgs& a, int64_t smp, char* mem, const int (*s_c)[kBinom])
+{
+    draw_sample<T, false>(a, smp, mem, s_c);
+}
+
+// Threads of a block at most.
+template <int T, bool FIXED> constexpr int kSubsetThreads = T > 32 ? T : FIXED ? 64 : 256;
+
+// A group of T threads per sample (T = 32: several samples per block); 1024
+// threads per SM, where shared memory holds fewer (n = 10, 11) 896.
+template <int T, bool FIXED>
+__global__ void __launch_bounds__(kSubsetThreads<T, FIXED>, (T == 32 && FIXED ? 896 : 1024) / kSubsetThreads<T, FIXED>)
+subset_sampler_kernel(const __grid_constant__ SampArgs a)
+{
+    extern __shared__ int4 s_mem[];
+    __shared__ int s_c[kBinom][kBinom];        // C(t, j)
+    for (int q = threadIdx.x; q < kBinom * kBinom; q += blockDim.x) {
+        const int t = q / kBinom, j = q % kBinom;
+        int c = j <= t ? 1 : 0;
+        for (int i = 1; i <= j && j <= t; ++i) c = c * (t + 1 - i) / i;
+        s_c[t][j] = c;
+    }
+    __syncthreads();
+    const int64_t smp = (int64_t)blockIdx.x * (blockDim.x / T) + threadIdx.x / T;
+    if (smp >= a.count) return;                // whole groups
+    char* mem = (char*)s_mem + (size_t)(threadIdx.x / T) * subset_bytes(a.m, a.n);
+    if constexpr (FIXED) {
+        if (!draw_sample<T, true>(a, smp, mem, s_c)) draw_sample_fp64<T>(a, smp, mem, s_c);
+    } else {
+        draw_sample<T, false>(a, smp, mem, s_c);
     }
 }
 
@@ -368,7 +462,8 @@ __global__ void __launch_bounds__(32 * kSampWarps) sampler_kernel(const SampArgs
             }
             wloc[c] = w;
         }
-        rows[k - 1] = draw_mode(wloc, m, uni[k - 1]);
+        double total;
+        rows[k - 1] = draw_mode(wloc, m, uni[k - 1], total);
     }
     for (int i = lane; i < m; i += 32) {
         int c = 0;
