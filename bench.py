@@ -244,6 +244,8 @@ def run_ours(args):
         else:
             tc = abi.pcv_distribution_auto_algo(M, N_PH, ws_bytes) == pcv.PCV_ALGO_FACTOR_TC
             kind = "factor_tc" if tc else "factor"
+    # the expansion sums in fixed point by default, in FP64 where it is asked for by name
+    fixed = kind == "slos" and args.algo == "auto"
     flush = torch.empty(L2_FLUSH_BYTES // 4, dtype=torch.float32, device=dev)
 
     def dist_call(Uc, out):
@@ -392,18 +394,20 @@ def run_ours(args):
         # multisets of size k over M modes with d distinct modes: C(M, d) C(k-1, d-1)
         flops_per_call = sum(8 * d * math.comb(M, d) * math.comb(k - 1, d - 1)
                              for k in range(1, N_PH + 1) for d in range(1, min(k, M) + 1))
-        kname = "expand_fixed_kernel (state expansion, sums of 30-bit halves on the integer pipe)"
-        launches_per_call = N_PH + 2
+        kname = "expand_fixed_kernel (state expansion, sums of 30-bit halves on the integer pipe)" if fixed else \
+            "expand_kernel (state expansion, FP64 sums)"
+        launches_per_call = N_PH + (2 if fixed else 1)
     achieved = flops_per_call * calls / (ms * 1e-3) / 1e12 if ms > 0 and flops_per_call else None
     peak_src = f"derived: {sms} SMs x 2 DFMA/clk x 2 flop x {sm_max:.0f} MHz (FP64 ALU)"
     bound = "alu"
     if kind == "factor_tc":
         peak_tflops, bound = measured_peak("bf16_tflops", 1900.0), "tensor"
         peak_src = "MEASURED_PEAKS.json bf16_tflops (burst cuBLAS bf16 GEMM, measured)"
-    unit, fp64_equivalent = "TFLOP/s", None
-    if kind == "slos":
+    unit, fp64_equivalent, limiter = "TFLOP/s", None, None
+    if fixed:
         # the sums leave the FP64 pipe, so what remains as a roof is memory: results written once, every
-        # level below the last written and read once
+        # level below the last written and read once.  The kernel is far from it: it is bound by latency.
+        limiter = "latency of multiply-add chains and gathers; multiplier pipe 49 % busy, DRAM 3 % (ncu, m=18 n=9)"
         fp64_equivalent = {"tflops": achieved, "frac_of_fp64_peak": achieved / peak_tflops if achieved else None,
                            "note": "8 flops per state and occupied mode; computed as integer multiply-adds"}
         moved = 24 * (hi - lo) + 32 * sum(pcv.num_outputs(M, k) for k in range(1, N_PH))
@@ -416,7 +420,7 @@ def run_ours(args):
             "peak_source": peak_src,
             "fp64_probe_tflops": probe_tflops,
             "traffic": traffic, "traffic_source": traffic_note,
-            "launches_per_step": launches_per_call, "fp64_equivalent": fp64_equivalent,
+            "launches_per_step": launches_per_call, "fp64_equivalent": fp64_equivalent, "limiter": limiter,
             "stage_ms_per_step": {k: (v[0] / v[1] if v[1] else None) for k, v in stages.items()}}
 
     # context: the FP64 factorised path (its product kernel against the FP64 peak)
@@ -504,7 +508,7 @@ def run_ours(args):
         "vs_baseline": None,
         "dtype": "f64",
         "dtype_note": "FP64 inputs and results; the sums over a level run as exact fixed-point sums of 57- by 59-bit "
-        "products" if kind == "slos" else None if kind != "factor_tc" else
+        "products" if fixed else None if kind != "factor_tc" else
         "FP64 tables, scaling and results; the complex products run as exact integer digit products "
         "on the bf16 tensor cores (no rounding; agreement with the FP64 path to 1e-11)",
         "data": "synthetic",
