@@ -141,7 +141,7 @@ int64_t batched_workspace(int n_circ, int64_t total_outputs);
 int64_t batched_workspace_full(int n_circ, int64_t total_outputs);
 // copies a descriptor (passed by value) into device memory
 cudaError_t launch_store_desc(const pcv_batch_desc& d, pcv_batch_desc* out, cudaStream_t s);
-// route: PCV_ALGO_AUTO (per output, by FP64 instruction count), PCV_ALGO_TILE
+// route: PCV_ALGO_AUTO (per output, by its time), PCV_ALGO_TILE
 // or PCV_ALGO_MULT (every output to that kernel)
 cudaError_t launch_glynn_batched(const pcv_batch_desc* descs, int n_circ, int64_t total_outputs, void* ws,
                                  int64_t ws_bytes, int sms, int route, cudaStream_t s);

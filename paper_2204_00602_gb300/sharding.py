@@ -4,7 +4,7 @@ Every amplitude is independent, so ranks divide the work with no exchange on
 the data path:
 
 * circuits of an uneven batch: greedy longest-processing-time assignment by
-  each circuit's FP64 instruction count under the batched launch's routing
+  each circuit's time in FP64 instructions under the batched launch's routing
   model (``circuit_cost``, ``lpt_assign``);
 * outputs of one distribution or one list of explicit outputs, and phase sets
   of a mesh batch: contiguous index ranges [r N / P, (r + 1) N / P)

@@ -11,15 +11,15 @@ batched: uneven circuits (m ~ U{8..64}, n ~ U{4..min(24, m)}, Haar U, photons in
 modes 0..n-1, 4096 seeded random outputs each, collision-free for n <= 16,
 uniform multisets above) in persistent launches: each output goes to the
 shared-row-sum tile kernel or to Glynn's sum with multiplicities, whichever
-issues fewer FP64 instructions (--route forces one of them).
+takes less time (--route forces one of them).
 sweep: one Haar unitary per n = 16..30 at m = n^2, 256 collision-free outputs,
-plain Glynn block kernel (m is too large for the shared-row-sum tiles).
+plain Glynn block kernel.
 mesh: the differentiable m=12 n=6 mesh, 64 phase sets, forward (all 12,376
 outputs) + KL + backward per step.
 
 Each prints one JSON line: amplitudes/s, FP64 work per the kernel's
 instruction count, and the fraction of the FP64 peak (152 SMs x 2 DFMA/clk x
-2 flop x clock).
+2 flop x clock; above 1 where the products run on the integer pipe).
 """
 from __future__ import annotations
 
