@@ -13,7 +13,7 @@ uniform multisets above) in persistent launches: each output goes to the
 shared-row-sum tile kernel or to Glynn's sum with multiplicities, whichever
 takes less time (--route forces one of them).
 sweep: one Haar unitary per n = 16..30 at m = n^2, 256 collision-free outputs,
-plain Glynn block kernel.
+the library's own choice of kernel.
 mesh: the differentiable m=12 n=6 mesh, 64 phase sets, forward (all 12,376
 outputs) + KL + backward per step.
 
